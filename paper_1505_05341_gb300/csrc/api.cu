@@ -15,11 +15,10 @@
 namespace ys {
 
 template <int N> cudaError_t run_measure_n(Plan* const* lanes, int W, double* const* rows);
-template <int N> int yz_grid_n(int ell, cudaError_t* err);
+template <int N> YzShape yz_shape_n(int ell, cudaError_t* err);
 template <int N> size_t x_smem_n(int nbins, int nwb, int ell);
 
 thread_local std::string g_last_cuda_error;
-int yz_row_items(int n);
 
 namespace {
 
@@ -53,7 +52,7 @@ void dfree(T*& ptr) {
 }
 
 void free_all(Plan& p) {
-  dfree(p.d_tw); dfree(p.d_nodes); dfree(p.d_rel); dfree(p.d_invw); dfree(p.d_phase);
+  dfree(p.d_tw); dfree(p.d_twl); dfree(p.d_nodes); dfree(p.d_rel); dfree(p.d_invw); dfree(p.d_phase);
   dfree(p.d_col_off); dfree(p.d_pencil); dfree(p.d_lut); dfree(p.d_shell);
   dfree(p.d_mesh); dfree(p.d_z); dfree(p.d_sync); dfree(p.d_g); dfree(p.d_acc); dfree(p.d_sums); dfree(p.d_result);
   dfree(p.d_tile_count); dfree(p.d_tile_off); dfree(p.d_tile_cur); dfree(p.d_rec);
@@ -252,6 +251,17 @@ ys_status build_tables(Plan& p) {
     invw[i] = c.compensate ? (float)(1.0 / W) : 1.0f;
     phase[i] = make_float2((float)std::cos(x), (float)-std::sin(x));
   }
+  // twiddles of the y,z stage's line transforms (LineFft): N = R1 R2 E2
+  const int r1 = is_pow2(n) ? 16 : 12, tpl = n / r1, e2_max = is_pow2(n) ? 256 : 192;
+  std::vector<float2> twl((size_t)(r1 - 1) * tpl);
+  auto unit_root = [](double turn) {
+    return make_float2((float)std::cos(-2.0 * M_PI * turn), (float)std::sin(-2.0 * M_PI * turn));
+  };
+  for (int k = 1; k < r1; ++k)
+    for (int t = 0; t < tpl; ++t) twl[(size_t)(k - 1) * tpl + t] = unit_root((double)t * k / n);
+  if (n == 4 * e2_max)  // E2 = 4, R2 = 16
+    for (int e = 0; e < 4; ++e)
+      for (int q = 0; q < 17; ++q) twl.push_back(unit_root((double)e * q / 64.0));
   // stage-major twiddles (fft_tw_offset): exp(-2 pi i r k / (N_s R_s)) per stage
   for (int st = 1; st < fft_nstages(n); ++st) {
     const int ns = fft_ns_before(n, st), rad = fft_radix(n, st), off = fft_tw_offset(n, st);
@@ -269,13 +279,40 @@ ys_status build_tables(Plan& p) {
       const float hi = (float)v;
       nodes[a * (n + 3) + i + 1] = make_float2(hi, (float)(v - (double)hi));
     }
-  std::vector<float> rel((size_t)p.m * 3 * n);
+  // in units of the power of two just above the largest component (the line-of-sight
+  // weights do not change with the unit)
+  std::vector<double> rel64((size_t)p.m * 3 * n);
+  double far = 0.0;
   for (int j = 0; j < p.m; ++j)
     for (int a = 0; a < 3; ++a)
       for (int i = 0; i < n; ++i) {
         const double s = j == 1 ? 0.5 : 0.0;
-        rel[((size_t)j * 3 + a) * n + i] = (float)(c.box_min[a] + (i + s) * p.H - c.observer[a]);
+        double& r = rel64[((size_t)j * 3 + a) * n + i];
+        r = c.box_min[a] + (i + s) * p.H - c.observer[a];
+        far = std::max(far, std::fabs(r));
       }
+  int unit = 0;
+  std::frexp(far, &unit);
+  std::vector<float2> rel(rel64.size());
+  for (size_t i = 0; i < rel.size(); ++i) {
+    const float v = (float)std::ldexp(rel64[i], -unit);
+    const int ex = v != 0.f ? std::max(-30, std::ilogb(v)) : -30;
+    rel[i] = make_float2(v, std::ldexp(1.f, -ex));
+  }
+  // the node that carries no line-of-sight weight, if the observer sits on one
+  for (int j = 0; j < p.m; ++j) {
+    int at[3];
+    float r2 = 0.f;
+    for (int a = 0; a < 3; ++a) {
+      const float2* r = rel.data() + ((size_t)j * 3 + a) * n;
+      at[a] = 0;
+      for (int i = 1; i < n; ++i)
+        if (std::fabs(r[i].x) < std::fabs(r[at[a]].x)) at[a] = i;
+      r2 += r[at[a]].x * r[at[a]].x;
+    }
+    if (r2 <= YZ_R2_MIN)
+      for (int a = 0; a < 3; ++a) p.org[j][a] = at[a];
+  }
   cudaError_t e;
 #define YS_UP(dst, vec)                                                                                 \
   do {                                                                                                  \
@@ -291,6 +328,7 @@ ys_status build_tables(Plan& p) {
   YS_UP(p.d_invw, invw);
   YS_UP(p.d_phase, phase);
   YS_UP(p.d_tw, tw);
+  YS_UP(p.d_twl, twl);
   YS_UP(p.d_nodes, nodes);
   YS_UP(p.d_rel, rel);
 #undef YS_UP
@@ -341,13 +379,11 @@ void set_tiles(Plan& p, int tx, int ty, int tz) {
 // row items, and must not be claimed before those finish (a claimed item that waits
 // idles its CTA).  Between the two claims the grid works through about
 // D * W_plane - (grid - NZ) * w_row of other items, with W_plane = NZ w_row + NY w_col
-// the work of one plane's items in FFT-line units (a row item: R rows x field pairs,
-// plus field construction; a column item: its basis fields plus the fold).
+// the work of one plane's items in FFT-line units (YzShape).
 int ring_lead_for(const Plan& p, int grid, int pct) {
-  const int nz = yz_row_items(p.n), ny = std::max(1, p.nzc);
-  const double rows = (double)p.n / nz;
-  const double w_row = rows * ((p.nb + 1) / 2) * 1.3, w_col = p.nb * 1.2;
-  const double plane = nz * w_row + ny * w_col;
+  const int nz = p.n / p.yz_rows, ny = std::max(1, (p.nzc + p.yz_cols - 1) / p.yz_cols);
+  const double w_row = p.yz_w_row;
+  const double plane = nz * w_row + ny * p.yz_w_col;
   const double base = std::ceil(std::max(0, grid - nz) * w_row / plane) + 1.0;
   return std::max(2, (int)std::ceil(base * pct / 100.0));
 }
@@ -401,29 +437,20 @@ cudaError_t launch_finalize(Plan* const* lanes, int W, double* const* rows) {
   return cudaGetLastError();
 }
 
-// Row items per plane of the y,z kernel (N / rows per item; mirrors YZ<N, ELL>::R).
-int yz_row_items(int n) {
-  const int E = (n & (n - 1)) == 0 ? 8 : 12;  // fft_elems
-  const int lpp = 256 / (n / E);
-  const int base = n >= 512 ? 8 : 16;
-  const int r = lpp > base ? std::min(lpp, n) : base;
-  return n / r;
-}
-
-int yz_grid_for(Plan& p, cudaError_t* err) {
+YzShape yz_shape_for(Plan& p, cudaError_t* err) {
   switch (p.n) {
-    case 16: return yz_grid_n<16>(p.ell, err);
-    case 32: return yz_grid_n<32>(p.ell, err);
-    case 64: return yz_grid_n<64>(p.ell, err);
-    case 96: return yz_grid_n<96>(p.ell, err);
-    case 128: return yz_grid_n<128>(p.ell, err);
-    case 192: return yz_grid_n<192>(p.ell, err);
-    case 256: return yz_grid_n<256>(p.ell, err);
-    case 384: return yz_grid_n<384>(p.ell, err);
-    case 512: return yz_grid_n<512>(p.ell, err);
-    case 768: return yz_grid_n<768>(p.ell, err);
-    case 1024: return yz_grid_n<1024>(p.ell, err);
-    default: *err = cudaErrorInvalidValue; return 0;
+    case 16: return yz_shape_n<16>(p.ell, err);
+    case 32: return yz_shape_n<32>(p.ell, err);
+    case 64: return yz_shape_n<64>(p.ell, err);
+    case 96: return yz_shape_n<96>(p.ell, err);
+    case 128: return yz_shape_n<128>(p.ell, err);
+    case 192: return yz_shape_n<192>(p.ell, err);
+    case 256: return yz_shape_n<256>(p.ell, err);
+    case 384: return yz_shape_n<384>(p.ell, err);
+    case 512: return yz_shape_n<512>(p.ell, err);
+    case 768: return yz_shape_n<768>(p.ell, err);
+    case 1024: return yz_shape_n<1024>(p.ell, err);
+    default: *err = cudaErrorInvalidValue; return {};
   }
 }
 
@@ -517,7 +544,7 @@ ys_status ys_plan_create(const ys_config* cfg, ys_plan** out) {
   p.m = c.interlace ? 2 : 1;
   p.ell = c.ell_max;
   p.kind = c.assign;
-  p.nb = p.ell == 0 ? 1 : (p.ell == 2 ? 7 : (p.ell == 4 ? 16 : 29));
+  p.nf = p.ell + 1;  // F, and two sources for each degree 2, 4, .. l_max
   p.ng = p.ell == 0 ? 1 : (p.ell == 2 ? 4 : (p.ell == 4 ? 9 : 16));
   p.row_len = ys::result_row_len(c.n_bins, p.ell);
   const int n = p.n;
@@ -543,7 +570,12 @@ ys_status ys_plan_create(const ys_config* cfg, ys_plan** out) {
   const size_t n3 = (size_t)n * n * n;
   // y,z-stage ring: the column items of a plane trail its row items by D planes, and a
   // slot is rewritten S = D + 2 planes later; D covers one grid's worth of items.
-  p.yz_grid_max = ys::yz_grid_for(p, &e);
+  const ys::YzShape shape = ys::yz_shape_for(p, &e);
+  p.yz_grid_max = shape.grid;
+  p.yz_rows = shape.rows;
+  p.yz_cols = shape.cols;
+  p.yz_w_row = shape.w_row;
+  p.yz_w_col = shape.w_col;
   if (e) {
     st = ys::cuda_fail(e);
     ys::free_all(p);
@@ -554,7 +586,7 @@ ys_status ys_plan_create(const ys_config* cfg, ys_plan** out) {
   ys::set_yz_grid(p, p.yz_grid_max, ys::kRingLeadPctMax);
   p.ring_slots_cap = p.ring_slots;
   ys::set_yz_grid(p, p.yz_grid_max, 100);
-  const size_t slot = (size_t)2 * ((p.nb + 1) / 2) * std::max(1, p.nzc) * n;  // field pairs interleaved
+  const size_t slot = (size_t)p.nf * std::max(1, p.nzc) * n;
   if ((e = ys::dalloc(p, p.d_mesh, p.m * n3)) || (e = ys::dalloc(p, p.d_z, slot * p.ring_slots_cap)) ||
       (e = ys::dalloc(p, p.d_sync, (size_t)2 * p.m * n + 2)) ||
       (e = ys::dalloc(p, p.d_g, (size_t)p.m * p.ng * n * std::max(1, p.np_pad))) ||

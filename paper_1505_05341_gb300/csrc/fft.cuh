@@ -1,12 +1,13 @@
 // Shared-memory complex FFTs for the mesh transforms (forward, e^{-2 pi i j k / N}).
 //
-// The method (Sec. 3) places no condition on the FFT algorithm; this one is a
-// Stockham autosort decimation-in-time transform with the result in natural order.
-// N is 2^a (radix-8 stages, then one radix-4 or radix-2) or 3 * 2^a (radix-4 stages,
-// an optional radix-2, then radix-3).  Each thread holds E = 8 (or 12) elements per
-// line and does E / R butterflies per stage; the data go through shared memory
-// between stages.  Twiddles come from a stage-major table (fft_tw_offset) computed
-// in FP64 on the host and rounded to float.
+// The method (Sec. 3) places no condition on the FFT algorithm.  N is 2^a or 3 * 2^a, and
+// results come out in natural order.
+//   y,z stage: lines walked by consecutive threads, 16 (12) elements per thread, two
+//     large radices and a small last one done by the reader (LineFft, below).
+//   x stage: interleaved lines, a Stockham autosort transform with 8 (12) elements per
+//     thread: radix-8 stages, then one radix-4 or radix-2; for 3 * 2^a radix-4 stages, an
+//     optional radix-2, then radix-3.  The data go through shared memory between stages.
+// Twiddles come from tables computed in FP64 on the host and rounded to float.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -14,13 +15,8 @@ namespace ys {
 
 __host__ __device__ constexpr bool is_pow2(int n) { return n > 0 && (n & (n - 1)) == 0; }
 
-// Elements per thread.  Walked by consecutive threads (y,z stage), a line fits one
-// warp up to N = 512 (768); its TPL = N / E threads synchronise among themselves only
-// (line_group_sync).  Interleaved lines (x stage) use 8 or 12 elements.
-__host__ __device__ constexpr int fft_elems(int n) {
-  return is_pow2(n) ? 8 : 12;
-}
-__host__ __device__ constexpr int fft_elems_lf(int n) { return is_pow2(n) ? 8 : 12; }
+// Elements per thread of the x stage's interleaved lines.
+__host__ __device__ constexpr int fft_elems(int n) { return is_pow2(n) ? 8 : 12; }
 
 // Barrier over the TPL consecutive threads that own one line: the warp when the
 // line fits in it, else a named barrier (ids 1..15) shared by those threads only.
@@ -33,7 +29,7 @@ __device__ __forceinline__ void line_group_sync() {
   }
 }
 
-// Number of stages and the radix of stage s (see header comment).
+// Number of stages of the x stage's transform and the radix of stage s.
 __host__ __device__ constexpr int fft_nstages(int n) {
   if (is_pow2(n)) {
     int s = 0, m = n;
@@ -138,24 +134,216 @@ template <> struct Dft<8> {
   }
 };
 
-// Element offset inside a line: with PAD, one complex of padding follows every 16
-// elements.  A float2 access is served per half-warp over 16 bank pairs, so 16
-// consecutive elements that start on a multiple of 16 stay on 16 distinct pairs,
-// while the strided Stockham stores (element R j + r, R = 8 or 4) are spread over the
-// pairs by the pad.
-template <bool PAD>
-__host__ __device__ constexpr int fft_pos(int i) { return PAD ? i + (i >> 4) : i; }
+// 16 = 4 x 4: DFT-4 over the inputs 4 a + b for each b, twiddles w16^(b k1), DFT-4 over b.
+template <> struct Dft<16> {
+  __device__ static __forceinline__ void run(float2* v) {
+    const float h = 0.707106781186547524f, c1 = 0.923879532511286756f, s1 = 0.382683432365089772f;
+    float2 t[4][4];  // [k1][b]
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      float2 u[4] = {v[b], v[4 + b], v[8 + b], v[12 + b]};
+      Dft<4>::run(u);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) t[k][b] = u[k];
+    }
+    t[1][1] = cmul(t[1][1], make_float2(c1, -s1));
+    t[1][3] = cmul(t[1][3], make_float2(s1, -c1));
+    t[3][1] = cmul(t[3][1], make_float2(s1, -c1));
+    t[3][3] = cmul(t[3][3], make_float2(-c1, s1));
+    t[1][2] = __fmul2_rn(add_mi(t[1][2], t[1][2]), make_float2(h, h));    // w16^2 = h (1 - i)
+    t[2][1] = __fmul2_rn(add_mi(t[2][1], t[2][1]), make_float2(h, h));
+    t[2][3] = __fmul2_rn(sub_mi(t[2][3], t[2][3]), make_float2(-h, -h));  // w16^6 = -h (1 + i)
+    t[3][2] = __fmul2_rn(sub_mi(t[3][2], t[3][2]), make_float2(-h, -h));
+    t[2][2] = make_float2(t[2][2].y, -t[2][2].x);                         // w16^4 = -i
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      Dft<4>::run(t[k]);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) v[k + 4 * q] = t[k][q];
+    }
+  }
+};
 
-// Line length in complex elements for a padded / unpadded layout.  Padded lines are
-// 1 mod 16 (lines read at one element by 16 row lanes land on 16 pairs), or 2 mod 16
-// when ROWS_ARE_PAIRS (8 rows x 2 elements per half-warp, the split of the y,z
-// stage's row items from 512^3 up); unpadded ones are odd.
-template <int N, bool PAD, bool ROWS_ARE_PAIRS = false>
-__host__ __device__ constexpr int fft_line_len() {
-  if (!PAD) return N + 1;
-  const int base = N + N / 16;
-  const int want = ROWS_ARE_PAIRS ? 2 : 1;
-  return base + ((want - base % 16) + 16) % 16;
+// 12 = 3 x 4 with coprime factors: inputs (4 a + 3 b) mod 12, outputs (4 k + 9 q) mod 12,
+// no twiddles (the prime-factor mapping).
+template <> struct Dft<12> {
+  __device__ static __forceinline__ void run(float2* v) {
+    float2 t[3][4];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      float2 u[3] = {v[(3 * b) % 12], v[(4 + 3 * b) % 12], v[(8 + 3 * b) % 12]};
+      Dft<3>::run(u);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) t[k][b] = u[k];
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      Dft<4>::run(t[k]);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) v[(4 * k + 9 * q) % 12] = t[k][q];
+    }
+  }
+};
+
+template <> struct Dft<1> {
+  __device__ static __forceinline__ void run(float2*) {}
+};
+
+// ---------------------------------------------------------------------------
+// Line transforms of the y,z stage: one line of N complex elements by TPL consecutive
+// threads with R1 = 16 (12) elements each, N = R1 R2 E2.
+//   1. Thread t holds x[t + TPL r] and does one radix-R1 butterfly in registers,
+//      multiplies by exp(-2 pi i t k1 / N) and stores element (k1, t) at k1 P + t.
+//   2. Butterfly (k1, e), e < E2, takes (k1, e + E2 s), s < R2, through a radix-R2
+//      butterfly, multiplies by exp(-2 pi i e q / (R2 E2)) and puts the results back
+//      where its inputs were.
+//   3. The reader does the last radix E2 (1, 2 or 4) on the E2 neighbouring elements
+//      of a slot: frequency kappa + (N / E2) h, kappa = k1 + R1 q, is
+//      sum_e exp(-2 pi i e h / E2) element[slot(kappa) + e].
+// A line thus crosses shared memory twice (three times with radix-8 stages of 8
+// elements per thread at N = 512), and its twiddles stay in registers.  The pitch P
+// and the line length LINE keep every access conflict-free: the E2 elements of a slot
+// are adjacent and a warp's k1 step through the banks by E2 (steps 1 and 2), and
+// LINE is odd in units of a slot's (at most 16-byte) load, for readers that go across lines.
+// ---------------------------------------------------------------------------
+template <int N>
+struct LineFft {
+  static constexpr bool P2 = is_pow2(N);
+  static constexpr int R1 = P2 ? 16 : 12;
+  static constexpr int E2 = P2 ? (N > 256 ? N / 256 : 1) : (N > 192 ? N / 192 : 1);
+  static constexpr int R2 = N / (R1 * E2);
+  static constexpr int TPL = N / R1;
+  static constexpr int UNITS = R1 * E2;                  // butterflies of step 2
+  static constexpr int NB2 = (UNITS + TPL - 1) / TPL;    // and per thread
+  static constexpr int P = E2 == 1 ? (TPL | 1) : TPL + E2;
+  static constexpr int LINE = E2 == 1 ? ((R1 * P) | 1) : R1 * P + (6 - (R1 * P) % 4) % 4;
+  static constexpr int M = N / E2;
+  static constexpr int HALF_ITEMS = E2 == 1 ? N / 2 : M / 2;  // items of line_halves
+  // Twiddle table: exp(-2 pi i t k / N) at (k - 1) TPL + t, 1 <= k < R1, then for E2 = 4
+  // exp(-2 pi i e q / (4 R2)) at 17 e + q.
+  static constexpr int TWN = (R1 - 1) * TPL + (E2 == 4 ? 4 * 17 : 0);
+  static_assert(R1 * R2 * E2 == N && TPL * R1 == N, "factors");
+  __host__ __device__ static constexpr int slot(int kappa) { return (kappa % R1) * P + (kappa / R1) * E2; }
+};
+
+// Line handled by thread group g.  Where several groups share a half-warp, their lines
+// are TPL apart, so that the groups' elements fall on different banks (LINE is odd).
+template <int TPL>
+__device__ __forceinline__ int line_of_group(int g) {
+  if constexpr (TPL >= 16) return g;
+  constexpr int G = 16 / TPL;
+  return (g % G) * TPL + (g / G) % TPL + (g / 16) * 16;
+}
+
+// exp(-2 pi i q / 32), q < 16
+__device__ constexpr float kW32[16][2] = {
+      {1.000000000000000000e+00f, -0.000000000000000000e+00f},
+      {9.807852804032304306e-01f, -1.950903220161282481e-01f},
+      {9.238795325112867385e-01f, -3.826834323650897818e-01f},
+      {8.314696123025452357e-01f, -5.555702330196021776e-01f},
+      {7.071067811865475727e-01f, -7.071067811865474617e-01f},
+      {5.555702330196022887e-01f, -8.314696123025452357e-01f},
+      {3.826834323650898373e-01f, -9.238795325112867385e-01f},
+      {1.950903220161283314e-01f, -9.807852804032304306e-01f},
+      {6.123233995736766036e-17f, -1.000000000000000000e+00f},
+      {-1.950903220161281926e-01f, -9.807852804032304306e-01f},
+      {-3.826834323650897263e-01f, -9.238795325112867385e-01f},
+      {-5.555702330196019556e-01f, -8.314696123025454577e-01f},
+      {-7.071067811865474617e-01f, -7.071067811865475727e-01f},
+      {-8.314696123025453467e-01f, -5.555702330196021776e-01f},
+      {-9.238795325112867385e-01f, -3.826834323650898928e-01f},
+      {-9.807852804032304306e-01f, -1.950903220161286089e-01f}};
+
+// The twiddles of thread t of a line, from the table.
+template <int N>
+__device__ __forceinline__ void load_twiddles(float2 (&tw)[LineFft<N>::R1 - 1], const float2* table, int t) {
+#pragma unroll
+  for (int k = 0; k < LineFft<N>::R1 - 1; ++k) tw[k] = table[k * LineFft<N>::TPL + t];
+}
+
+// Steps 1 and 2 for the line at `line`; v: the thread's R1 elements.  Every thread of a
+// warp calls this (ok: whether its line exists); tw: exp(-2 pi i t k / N), k = 1..R1 - 1;
+// wE: the table's part for E2 = 4.
+template <int N>
+__device__ __forceinline__ void line_fft(float2 (&v)[LineFft<N>::R1], float2* line, int t,
+                                         const float2 (&tw)[LineFft<N>::R1 - 1], const float2* wE, bool ok) {
+  using L = LineFft<N>;
+  constexpr int R1 = L::R1, R2 = L::R2, E2 = L::E2, P = L::P, TPL = L::TPL;
+  if (ok) {
+    Dft<R1>::run(v);
+    line[t] = v[0];
+#pragma unroll
+    for (int k = 1; k < R1; ++k) line[k * P + t] = cmul(v[k], tw[k - 1]);
+  }
+  line_group_sync<TPL>();
+  if constexpr (R2 > 1) {
+#pragma unroll
+    for (int i = 0; i < L::NB2; ++i) {
+      const int u = t + i * TPL;
+      if (ok && (L::UNITS % TPL == 0 || u < L::UNITS)) {
+        const int e = u % E2;
+        float2* q = line + (u / E2) * P + e;
+        float2 b[R2];
+#pragma unroll
+        for (int s = 0; s < R2; ++s) b[s] = q[E2 * s];
+        Dft<R2>::run(b);
+        if constexpr (E2 == 2) {
+          static_assert(E2 != 2 || R2 == 16, "w32 twiddles");
+          if (e) {
+#pragma unroll
+            for (int s = 1; s < R2; ++s) b[s] = cmul(b[s], make_float2(kW32[s][0], kW32[s][1]));
+          }
+        } else if constexpr (E2 == 4) {
+#pragma unroll
+          for (int s = 1; s < R2; ++s) b[s] = cmul(b[s], wE[17 * e + s]);
+        }
+#pragma unroll
+        for (int s = 0; s < R2; ++s) q[E2 * s] = b[s];
+      }
+    }
+  }
+}
+
+// The two half spectra of a line that holds real lines a + i b: emit(k, A_k, B_k) for
+// the k < nk of item i (0 <= i < HALF_ITEMS covers every k < N / 2 once).  With
+// C_k the line's transform, A_k = (C_k + C_{N-k}^*) / 2, B_k = (C_k - C_{N-k}^*) / (2 i).
+template <int N, class Emit>
+__device__ __forceinline__ void line_halves(const float2* line, int i, int nk, Emit&& emit) {
+  using L = LineFft<N>;
+  constexpr int M = L::M;
+  auto out = [&](int k, float2 c, float2 m) {
+    if (k < nk)
+      emit(k, make_float2(0.5f * (c.x + m.x), 0.5f * (c.y - m.y)), make_float2(0.5f * (c.y + m.y), -0.5f * (c.x - m.x)));
+  };
+  if constexpr (L::E2 == 1) {
+    if (i >= nk) return;
+    const float2 c = line[L::slot(i)];
+    out(i, c, i ? line[L::slot(N - i)] : c);
+  } else {
+    // kappa = i and M - i (M / 2 for i = 0) hold each other's mirror frequencies
+    const int k0 = i, k1 = i ? M - i : M / 2;
+    if (L::E2 == 2 && k0 >= nk && k1 >= nk) return;
+    const float4* s0 = reinterpret_cast<const float4*>(line + L::slot(k0));
+    const float4* s1 = reinterpret_cast<const float4*>(line + L::slot(k1));
+    const float4 p = s0[0], q = s1[0];
+    const float2 p0 = make_float2(p.x, p.y), p1 = make_float2(p.z, p.w);
+    const float2 q0 = make_float2(q.x, q.y), q1 = make_float2(q.z, q.w);
+    if constexpr (L::E2 == 2) {
+      const float2 a0 = cadd(p0, p1), a1 = csub(p0, p1), b0 = cadd(q0, q1), b1 = csub(q0, q1);
+      out(k0, a0, i ? b1 : a0);
+      out(k1, b0, i ? a1 : b1);
+    } else {
+      const float4 pp = s0[1], qq = s1[1];
+      float2 a[4] = {p0, p1, make_float2(pp.x, pp.y), make_float2(pp.z, pp.w)};
+      float2 b[4] = {q0, q1, make_float2(qq.x, qq.y), make_float2(qq.z, qq.w)};
+      Dft<4>::run(a);
+      Dft<4>::run(b);
+      out(k0, a[0], i ? b[3] : a[0]);
+      out(k0 + M, a[1], i ? b[2] : a[3]);
+      out(k1, b[0], i ? a[3] : b[3]);
+      out(k1 + M, b[1], i ? a[2] : b[2]);
+    }
+  }
 }
 
 // Twiddles are stored stage by stage: for stage s >= 1 (N_s = fft_ns_before(N, s)
@@ -169,87 +357,6 @@ __host__ __device__ constexpr int fft_tw_offset(int n, int stage) {
   return off;
 }
 
-// One Stockham stage over `nl` lines of length N stored in shared memory at
-// buf[line * ls + elem * es].  LF: consecutive threads take consecutive lines (for
-// layouts whose lines interleave); otherwise consecutive threads walk one line.
-// NL > 0: the number of lines is a compile-time constant (passes unrolled, separated
-// by a line-group barrier so that no pass's addresses are hoisted into another);
-// NL == 0: nl lines at run time.
-//
-// Padded lines walked by consecutive threads (the y,z stage) take a fast path: element
-// i sits at i + i/16, and (a + 16 m)/16 = a/16 + m, so when the threads per line and
-// the input stride are multiples of 16 every load is one per-thread base address plus
-// a compile-time offset.  The stores go to outb + r N_s with outb = k (mod N_s R): for
-// N_s a multiple of 16 the same holds, and for N_s dividing 16 (with k < N_s and N_s R
-// a multiple of 16) element outb + r N_s sits at pos(outb) + r N_s + (r N_s)/16.
-template <int N, int S, bool LF, bool PAD, int NL = 0>
-__device__ __forceinline__ void fft_stage(float2* buf, int es, int ls, int nl_rt, const float2* tw) {
-  constexpr int R = fft_radix(N, S);
-  constexpr int E = LF ? fft_elems_lf(N) : fft_elems(N);
-  constexpr int TPL = N / E;        // threads per line
-  constexpr int NB = E / R;         // butterflies per thread
-  constexpr int NS = fft_ns_before(N, S);
-  constexpr int STRIDE = N / R;
-  constexpr bool FAST_LD = !LF && PAD && TPL % 16 == 0 && STRIDE % 16 == 0;
-  constexpr bool FAST_ST = !LF && PAD && (NS % 16 == 0 || (16 % NS == 0 && (NS * R) % 16 == 0));
-  const float2* tws = tw + fft_tw_offset(N, S);
-  // Lines walked by consecutive threads only need their own threads synchronised.
-  const int tid = threadIdx.x;
-  const int lpp = blockDim.x / TPL;  // lines per pass
-  const bool in_pass = tid < lpp * TPL;
-  const int lane_line = LF ? tid % lpp : tid / TPL;
-  const int tl = LF ? tid / lpp : tid % TPL;
-  const int nl = NL > 0 ? NL : nl_rt;
-#pragma unroll 1
-  for (int base_line = 0; base_line < nl; base_line += lpp) {
-    const int line = base_line + lane_line;
-    const bool ok = in_pass && line < nl;
-    float2 v[E];
-    if (ok) {
-      const float2* lp = buf + line * ls;
-      if constexpr (FAST_LD) {
-        const float2* src = lp + (tl + (tl >> 4));
-#pragma unroll
-        for (int q = 0; q < NB; ++q)
-#pragma unroll
-          for (int r = 0; r < R; ++r) v[q * R + r] = src[(q * TPL + r * STRIDE) / 16 * 17];
-      } else {
-#pragma unroll
-        for (int q = 0; q < NB; ++q) {
-          const int j = tl + q * TPL;
-#pragma unroll
-          for (int r = 0; r < R; ++r) v[q * R + r] = lp[fft_pos<PAD>(j + r * STRIDE) * es];
-        }
-      }
-    }
-    if constexpr (LF) __syncthreads(); else line_group_sync<TPL>();
-    if (ok) {
-      float2* lp = buf + line * ls;
-#pragma unroll
-      for (int q = 0; q < NB; ++q) {
-        const int j = tl + q * TPL;
-        const int k = j % NS;
-        if (NS > 1) {
-          const float2* tk = tws + k * (R - 1);
-#pragma unroll
-          for (int r = 1; r < R; ++r) v[q * R + r] = cmul(v[q * R + r], tk[r - 1]);
-        }
-        Dft<R>::run(&v[q * R]);
-        const int outb = (j / NS) * NS * R + k;
-        if constexpr (FAST_ST) {
-          float2* dst = lp + (outb + (outb >> 4));
-#pragma unroll
-          for (int r = 0; r < R; ++r) dst[r * NS + (r * NS) / 16] = v[q * R + r];
-        } else {
-#pragma unroll
-          for (int r = 0; r < R; ++r) lp[fft_pos<PAD>(outb + r * NS) * es] = v[q * R + r];
-        }
-      }
-    }
-    if constexpr (LF) __syncthreads(); else line_group_sync<TPL>();
-  }
-}
-
 // Padded buffers of interleaved lines (x stage: element x of line p at x P + p):
 // PADP > 0 inserts PADP elements after every 8 PADP, so that the stores of a radix-8
 // first stage, 8 P apart across a warp, land on distinct bank pairs.
@@ -258,15 +365,16 @@ __host__ __device__ constexpr int lf_pad(int i) {
   return PADP > 0 ? i + (i / (8 * PADP)) * PADP : i;
 }
 
-// Out-of-place stage: reads the lines from src and writes them to dst (no barrier
+// Out-of-place stage over nl interleaved lines (element i of line l at l ls + i es;
+// consecutive threads take consecutive lines): reads src and writes dst (no barrier
 // inside; the caller synchronises before dst is read).  With two buffers a stage
 // needs one barrier instead of the two an in-place stage needs.  PIN / POUT: the
 // padding (lf_pad) of src / dst.
-template <int N, int S, bool LF, int PIN = 0, int POUT = 0>
+template <int N, int S, int PIN = 0, int POUT = 0>
 __device__ __forceinline__ void fft_stage_oop(const float2* src, float2* dst, int es, int ls, int nl,
                                               const float2* tw) {
   constexpr int R = fft_radix(N, S);
-  constexpr int E = LF ? fft_elems_lf(N) : fft_elems(N);
+  constexpr int E = fft_elems(N);
   constexpr int TPL = N / E;
   constexpr int NB = E / R;
   constexpr int NS = fft_ns_before(N, S);
@@ -275,8 +383,7 @@ __device__ __forceinline__ void fft_stage_oop(const float2* src, float2* dst, in
   const int tid = threadIdx.x;
   const int lpp = blockDim.x / TPL;
   const bool in_pass = tid < lpp * TPL;
-  const int lane_line = LF ? tid % lpp : tid / TPL;
-  const int tl = LF ? tid / lpp : tid % TPL;
+  const int lane_line = tid % lpp, tl = tid / lpp;
 #pragma unroll 1
   for (int base_line = 0; base_line < nl; base_line += lpp) {
     const int line = base_line + lane_line;
@@ -311,7 +418,7 @@ __device__ __forceinline__ void fft_stage_oop(const float2* src, float2* dst, in
 template <int N, int S, int END, int PA = 0, int PB = 0, bool Done = (S >= END)>
 struct FftPingPong {
   __device__ static __forceinline__ void run(float2* a, float2* b, int es, int ls, int nl, const float2* tw) {
-    fft_stage_oop<N, S, true, PA, PB>(a, b, es, ls, nl, tw);
+    fft_stage_oop<N, S, PA, PB>(a, b, es, ls, nl, tw);
     __syncthreads();
     FftPingPong<N, S + 1, END, PB, PA>::run(b, a, es, ls, nl, tw);
   }
@@ -321,29 +428,16 @@ struct FftPingPong<N, S, END, PA, PB, true> {
   __device__ static __forceinline__ void run(float2*, float2*, int, int, int, const float2*) {}
 };
 
-// Terminate the recursion at S == number of stages.
-template <int N, int S, bool LF, bool PAD = false, int NL = 0, bool Done = (S >= fft_nstages(N))>
-struct FftRun {
-  __device__ static __forceinline__ void run(float2* buf, int es, int ls, int nl, const float2* tw) {
-    fft_stage<N, S, LF, PAD, NL>(buf, es, ls, nl, tw);
-    FftRun<N, S + 1, LF, PAD, NL>::run(buf, es, ls, nl, tw);
-  }
-};
-template <int N, int S, bool LF, bool PAD, int NL>
-struct FftRun<N, S, LF, PAD, NL, true> {
-  __device__ static __forceinline__ void run(float2*, int, int, int, const float2*) {}
-};
-
 // Last stage into registers: stages 0 .. S-2 must already have run on the lines.
 // Each thread loads its butterfly inputs from line `line` of buf (element i at
 // line + i es, padded by lf_pad<PADL>), applies twiddles and the DFT, and keeps the
 // outputs: v[q * R + r] is element (tl + q * TPL) + r * (N / R).
-template <int N, bool LF, bool PAD, int PADL = 0>
+template <int N, int PADL = 0>
 __device__ __forceinline__ void fft_last_stage_regs(const float2* buf, int line, int es, int tl, const float2* tw,
-                                                    float2 (&v)[LF ? fft_elems_lf(N) : fft_elems(N)]) {
+                                                    float2 (&v)[fft_elems(N)]) {
   constexpr int S = fft_nstages(N) - 1;
   constexpr int R = fft_radix(N, S);
-  constexpr int E = LF ? fft_elems_lf(N) : fft_elems(N);
+  constexpr int E = fft_elems(N);
   constexpr int TPL = N / E;
   constexpr int NB = E / R;
   constexpr int NS = fft_ns_before(N, S);
@@ -353,7 +447,7 @@ __device__ __forceinline__ void fft_last_stage_regs(const float2* buf, int line,
   for (int q = 0; q < NB; ++q) {
     const int j = tl + q * TPL;
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[q * R + r] = buf[lf_pad<PADL>(line + fft_pos<PAD>(j + r * STRIDE) * es)];
+    for (int r = 0; r < R; ++r) v[q * R + r] = buf[lf_pad<PADL>(line + (j + r * STRIDE) * es)];
   }
 #pragma unroll
   for (int q = 0; q < NB; ++q) {
@@ -365,35 +459,6 @@ __device__ __forceinline__ void fft_last_stage_regs(const float2* buf, int line,
       for (int r = 1; r < R; ++r) v[q * R + r] = cmul(v[q * R + r], tk[r - 1]);
     }
     Dft<R>::run(&v[q * R]);
-  }
-}
-
-// First stage from registers: the caller holds, for its butterflies q < E/R0, the
-// inputs v[q * R0 + r] = x[fft_in_index<N>(tl, q, r)] of one line; this does the
-// stage-0 butterflies (no twiddles: N_s = 1) and stores the results to the line lp.
-// The remaining stages run with FftRun<N, 1, LF> after a line-group barrier.
-template <int N>
-__host__ __device__ constexpr int fft_in_index(int tl, int q, int r) {
-  return tl + q * (N / fft_elems(N)) + r * (N / fft_radix(N, 0));
-}
-
-template <int N, bool PAD>
-__device__ __forceinline__ void fft_stage0_regs(float2 (&v)[fft_elems(N)], float2* lp, int es, int tl) {
-  constexpr int R = fft_radix(N, 0);
-  constexpr int E = fft_elems(N);
-  constexpr int TPL = N / E;
-#pragma unroll
-  for (int q = 0; q < E / R; ++q) {
-    Dft<R>::run(&v[q * R]);
-    const int j = tl + q * TPL;
-    if constexpr (PAD && 16 % R == 0) {
-      float2* dst = lp + fft_pos<true>(j * R) * es;  // element R j + r sits r after R j (R | 16)
-#pragma unroll
-      for (int r = 0; r < R; ++r) dst[r * es] = v[q * R + r];
-    } else {
-#pragma unroll
-      for (int r = 0; r < R; ++r) lp[fft_pos<PAD>(j * R + r) * es] = v[q * R + r];
-    }
   }
 }
 

@@ -14,9 +14,8 @@ fields actually transformed (the "basis") are
   in every LOS field, so the identity above only holds for F'),
   degree 2, c <= 1 : (2,0,0) (1,1,0) (0,2,0) (1,0,1) (0,1,1),
   degree 4, c <= 1 : (4,0,0) (3,1,0) (2,2,0) (1,3,0) (0,4,0) (3,0,1) (2,1,1) (1,2,1) (0,3,1).
-16 real fields = 8 complex transforms for l <= 4 (7 fields for l <= 2).  For l <= 6
-the degree-6 monomials with c <= 1 add 13 fields (29 in all) and the groups
-(6, 0..6) add 7 (16 in all).
+16 fields for l <= 4 (7 for l <= 2).  For l <= 6 the degree-6 monomials with c <= 1 add
+13 fields (29 in all) and the groups (6, 0..6) add 7 (16 in all).
 
 Run:  python gen_group_table.py > group_table.inc
 """
@@ -129,19 +128,10 @@ def emit(ell_max):
     lines.append(f"    accumulate<0, {nb}>(psi, ky, kz, g);")
     lines.append("  }")
     arr = ", ".join(f"{a}, {b}, {c}, {d}" for a, b, c, d in bs)
-    lines.append("  // mono_c(beta, i): i = 0, 1, 2 exponents of r_hat_x, r_hat_y, r_hat_z; i = 3 degree.")
+    lines.append("  // mono_c(beta, i): i = 0, 1, 2 exponents of r_hat_x, r_hat_y, r_hat_z; i = 3 degree\n  // (0 = F itself, -1 = F with the node at r = 0 removed).")
     lines.append("  __host__ __device__ static constexpr int mono_c(int beta, int i) {")
     lines.append(f"    constexpr int t[{4 * nb}] = {{{arr}}};")
     lines.append("    return t[4 * beta + i];")
-    lines.append("  }")
-    lines.append("  // Exponents (a, b, c) of r_hat_x^a r_hat_y^b r_hat_z^c and the degree of basis field")
-    lines.append("  // beta; degree 0 = F itself, -1 = F with the node at r = 0 removed.")
-    lines.append("  __device__ static __forceinline__ void mono(int beta, int& a, int& b, int& c, int& d) {")
-    lines.append("    switch (beta) {")
-    for i, (a, b, c, d) in enumerate(bs):
-        lines.append(f"      case {i}: a = {a}; b = {b}; c = {c}; d = {d}; break;")
-    lines.append("      default: a = 0; b = 0; c = 0; d = -2; break;")
-    lines.append("    }")
     lines.append("  }")
     lines.append("};")
     return "\n".join(lines)

@@ -11,7 +11,7 @@ cudaError_t launch_finalize(Plan* const* lanes, int W, double* const* rows);
 
 // CTAs of the persistent y,z kernel that fit on the device at once.
 template <int N, int ELL>
-int yz_grid(cudaError_t* err) {
+YzShape yz_shape(cudaError_t* err) {
   using Y = YZ<N, ELL>;
   int dev = 0, sms = 0, per = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -19,7 +19,15 @@ int yz_grid(cudaError_t* err) {
   if (!e) e = cudaFuncSetAttribute(k_yz<N, ELL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Y::smem);
   if (!e) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_yz<N, ELL>, Y::THREADS, Y::smem);
   if (err) *err = e;
-  return e ? 0 : std::max(1, per) * sms;
+  YzShape sh;
+  sh.grid = e ? 0 : std::max(1, per) * sms;
+  sh.rows = Y::R;
+  sh.cols = Y::KC;
+  // a row item: its lines, the field construction and the split; a column item: its
+  // lines, the ring loads and the fold
+  sh.w_row = 1.5 * Y::RLINES;
+  sh.w_col = 1.6 * Y::CLINES;
+  return sh;
 }
 
 // l_max = 6 needs the 29 basis lines of a column item in shared memory: N <= 512.
@@ -27,15 +35,15 @@ template <int N>
 constexpr bool ell6_supported() { return N <= 512; }
 
 template <int N>
-int yz_grid_n(int ell, cudaError_t* err) {
+YzShape yz_shape_n(int ell, cudaError_t* err) {
   switch (ell) {
-    case 0: return yz_grid<N, 0>(err);
-    case 2: return yz_grid<N, 2>(err);
+    case 0: return yz_shape<N, 0>(err);
+    case 2: return yz_shape<N, 2>(err);
     case 6:
-      if constexpr (ell6_supported<N>()) return yz_grid<N, 6>(err);
+      if constexpr (ell6_supported<N>()) return yz_shape<N, 6>(err);
       if (err) *err = cudaErrorInvalidValue;
-      return 0;
-    default: return yz_grid<N, 4>(err);
+      return {};
+    default: return yz_shape<N, 4>(err);
   }
 }
 
@@ -55,7 +63,7 @@ cudaError_t run_yz(Plan* const* lanes, int W) {
     YZParams& prm = pm.lane[l];
     prm.mesh = p.d_mesh;
     prm.rel = p.d_rel;
-    prm.tw = p.d_tw;
+    prm.tw = p.d_twl;
     prm.ring = p.d_z;
     prm.gout = p.d_g;
     prm.col_off = p.d_col_off;
@@ -70,7 +78,9 @@ cudaError_t run_yz(Plan* const* lanes, int W) {
     prm.D = p.ring_lead;
     prm.spin_limit = p.yz_wait_ns;  // 1 s unless a test shortened it; then the kernel reports a timeout
     prm.skip_plane = p.fault_skip_plane;
-    items += (p.m * N + p.ring_lead) * (N / Y::R + p.nzc);
+    for (int j = 0; j < 2; ++j)
+      for (int a = 0; a < 3; ++a) prm.org[j][a] = p.org[j][a];
+    items += (p.m * N + p.ring_lead) * (N / Y::R + (p.nzc + Y::KC - 1) / Y::KC);
     pm.end[l] = items;
   }
   pm.nlanes = W;

@@ -4,15 +4,14 @@
 //
 // Data flow per mesh (x-major mesh F[ix][iy][iz]):
 //  k_yz (persistent, ticketed work list; see the block comment above YZParams)
-//     row item     one x-plane, R rows: F and 1/|r|^2 per node, then for each pair of
-//                  basis fields (F, F', F r_hat^a r_hat^b r_hat^c with c <= 1) the
-//                  two real fields as one complex FFT along z, split into the two
-//                  half spectra (k_z < nzc) and written to a ring slot laid out
-//                  [field pair][k_z][y][2] (y contiguous, the pair's fields side by side).
-//     column item  one k_z column of one plane: FFT along y of every basis field,
-//                  folded with k_y, k_z polynomial weights into the groups G_{n,p}
-//                  (power p of k_x; GroupTable); only the pencils (k_y, k_z) with
-//                  k_y^2 + k_z^2 < n2_hi are written, layout [mesh][group][x][pencil].
+//     row item     one x-plane, R rows: the source fields F, F / |r|^d and F Z / |r|^d
+//                  transformed along z (real lines in pairs), split into half spectra
+//                  (k_z < nzc) and written to a ring slot laid out [k_z][source][y].
+//     column item  KC k_z columns of one plane: sources times X^a Y^b are the basis fields,
+//                  transformed along y, folded with k_y, k_z polynomial weights into
+//                  the groups G_{n,p} (power p of k_x; GroupTable); only the pencils
+//                  (k_y, k_z) with k_y^2 + k_z^2 < n2_hi are written, layout
+//                  [mesh][group][x][pencil].
 //  k_x_combine  P pencils per CTA, tiles loaded by TMA: FFT along x of every group of
 //             every mesh, interlacing phase and window compensation per mode, A_0
 //             and k^n A_n = sum_p k_x^p G_{n,p}, then w |A_0|^2, w Re A_0 A_2^*,
@@ -35,62 +34,70 @@ namespace ys {
 
 #include "group_table.inc"
 
-// Basis fields at the nodes.  A field is F times r_hat_x^a r_hat_y^b r_hat_z^c of
-// degree d = a + b + c in {2, 4} (c <= 1), or F itself (d = 0), or F without the
-// node at r = 0 (d = -1), or nothing (d = -2, past the last field).  With
-// r = (X, Y, Z) from the observer, r_hat^(a,b,c) = X^a Y^b Z^c / |r|^d, and along one
-// z-line X and Y are fixed: K = X^a Y^b is one number per line and field, so a node
-// costs one reciprocal of |r|^2 shared by all fields plus two or three products per
-// field.
-
-// v^EXP for a small exponent 0 <= EXP <= 7, by the bits of EXP.
-template <int EXP>
-__device__ __forceinline__ float ipow_ct(float v) {
-  const float v2 = v * v;
-  float r = (EXP & 1) ? v : 1.f;
-  if constexpr ((EXP & 2) != 0) r *= v2;
-  if constexpr ((EXP & 4) != 0) r *= v2 * v2;
-  return r;
-}
-
-// Field value at a node: f the mesh value, i2 = 1/|r|^2 (0 where r = 0), z = Z, K the
-// line constant X^a Y^b; C, D the field's z power and degree (D = 2, 4 or 6 divides
-// by |r|^D).  Each pair of fields is built with its exponents known at compile time.
-template <int C, int D>
-__device__ __forceinline__ float basis_value_ct(float f, float i2, float z, float K) {
-  if constexpr (D == 0) return f;
-  else if constexpr (D == -1) return i2 > 0.f ? f : 0.f;
-  else if constexpr (D == -2) return 0.f;
-  else {
-    float v = (f * K) * i2;
-    if constexpr (D >= 4) v *= i2;
-    if constexpr (D == 6) v *= i2;
-    if constexpr (C != 0) v *= z;
-    return v;
+// Source fields and basis fields.  A basis field is F times r_hat_x^a r_hat_y^b
+// r_hat_z^c of degree d = a + b + c in {2, 4, 6} (c <= 1), or F itself, or F without the
+// node at r = 0 (F').  With r = (X, Y, Z) from the observer and X, Y fixed along a
+// z-line, the field is X^a Y^b times the source field h_{c,d} = F Z^c / |r|^d: the
+// factor passes through the z transform, so only the sources (F and, per degree,
+// c = 0 and 1: 5 real lines instead of 16 for l_max = 4) are transformed along z, and
+// the y stage multiplies their spectra by X^a Y^b before its own transforms.
+//   source 0: F;  sources 1 + 2 u, 2 + 2 u: F / |r|^d and F Z / |r|^d, d = 2 u + 2.
+// F' needs no line of its own: it differs from F at one node at most, whose
+// transform is a phase (see column_fold).
+//
+// Ranges.  r is held in units of a power of two near the largest |r| component (the
+// monomials have degree 0, so the unit cancels exactly).  The sources of one row are
+// scaled by rho^(d - c) and X, Y divided by rho, rho = max(2^floor(log2 |X|),
+// 2^floor(log2 |Y|)), at least 2^-30.  With rho within a factor of two of the row's
+// distance from the z axis through the observer, both sources of a degree, which share
+// a complex line, and the factors (X / rho)^a (Y / rho)^b are O(F) and O(1): neither
+// source's rounding shows in the other's field (one rho per x-plane instead lost 3.5
+// bits next to the observer's planes), and nothing overflows next to the observer.
+// Nodes with |r|^2 <= YZ_R2_MIN carry no line-of-sight weight, as the node at r = 0.
+// Line l of a column item: basis field 0 (l = 0) or l + 1 (F' is left out); its source
+// field and the exponents of X and Y.
+template <int ELL>
+struct YLines {
+  static constexpr int NL = ELL == 0 ? 1 : GroupTable<ELL>::NB - 1;
+  unsigned char src[NL], a[NL], b[NL];
+  constexpr YLines() : src(), a(), b() {
+    for (int l = 0; l < NL; ++l) {
+      const int beta = l == 0 ? 0 : l + 1;
+      const int d = GroupTable<ELL>::mono_c(beta, 3);
+      src[l] = (unsigned char)(d == 0 ? 0 : d - 1 + GroupTable<ELL>::mono_c(beta, 2));
+      a[l] = (unsigned char)GroupTable<ELL>::mono_c(beta, 0);
+      b[l] = (unsigned char)GroupTable<ELL>::mono_c(beta, 1);
+    }
   }
-}
+};
+template <int ELL> __constant__ constexpr YLines<ELL> kYLines{};
 
 // ---------------------------------------------------------------------------
 // y,z stage: one persistent kernel over a ticketed work list.
 //
 // Planes p = 0 .. m N - 1 (mesh j = p / N, x index p % N).  Per plane there are NZ
-// "row items" (R rows of the plane: the basis fields, complex FFTs of two real
-// fields along z, the split into the two half spectra for k_z < nzc, written to a
-// ring slot laid out [field pair][k_z][y][2]) and NY = nzc "column items" (one k_z column:
-// FFT along y of every basis field, the k_y, k_z polynomial fold into the k_x-power
-// groups, written for the pencils of that column).  Tickets are handed out in steps:
-// step t = row items of plane t, then column items of plane t - D.  Row items of
-// plane p reuse ring slot p mod S once the column items of plane p - S are done;
-// column items of plane p start once its row items are done.  Both waits are on
+// "row items" (R rows of the plane: the source fields, their transforms along z and the
+// split into half spectra for k_z < nzc, written to a ring slot) and NY "column items"
+// (KC k_z columns: the basis fields' transforms along y, the k_y, k_z polynomial fold
+// into the k_x-power groups, written for the pencils of those columns).  Tickets are
+// handed out in steps: step t = row items of plane t, then column items of plane t - D.
+// Row items of plane p reuse ring slot p mod S once the column items of plane p - S are
+// done; column items of plane p start once its row items are done.  Both waits are on
 // per-plane completion counters (release / acquire), bounded in time; a CTA only
 // ever waits on items claimed before its own, so the list cannot deadlock.
+//
+// What bounds it (512^3, l_max = 4, one mesh): instruction issue (51 % of the slots; 30 %
+// of the instructions are packed or scalar float arithmetic) and barriers, with
+// 16 warps per SM (128 registers); shared memory 57 % busy.  12.1 -> 6.5 ms for the
+// interlaced pair against transforming every basis field along z (16 real lines per
+// row instead of 5) with radix-8 stages; l_max = 6 30.8 -> 13.9 ms, 1024^3 87 -> 40 ms.
 // ---------------------------------------------------------------------------
 
 struct YZParams {
   const float* mesh;     // [m][N][N][N]
-  const float* rel;      // [m][3][N] node - observer
-  const float2* tw;      // [N]
-  float2* ring;          // [S][NB][nzc][N]
+  const float2* rel;     // [m][3][N] node - observer v, and 2^-floor(log2 |v|) (at most 2^30)
+  const float2* tw;      // [TWN] twiddles of the line transforms (LineFft<N>)
+  float2* ring;          // [S][nzc][NF][N]
   float2* gout;          // [m][NG][N][np]
   const int* col_off;    // [nzc + 1]
   int* done_z;           // [m N]
@@ -98,6 +105,7 @@ struct YZParams {
   int* ticket;           // [1]
   int* err;              // [1]
   int nzc, np, m, S, D;
+  int org[2][3];         // node at r = 0 of each mesh (x < 0: none)
   long long spin_limit;  // ns
   int skip_plane;        // >= 0: that plane's row items withhold their completion (test hook)
 };
@@ -150,123 +158,40 @@ __device__ __forceinline__ bool wait_geq(const int* addr, int target, int* err, 
 
 template <int N, int ELL>
 struct YZ {
-  using T = GroupTable<ELL>;
-  static constexpr int NB = T::NB, NG = T::NG, NPAIR = (NB + 1) / 2;
-  static constexpr int E = fft_elems(N), TPL = N / E;
-  static constexpr int R0 = fft_radix(N, 0);
-  static constexpr int THREADS = 256;
-  static constexpr int LPP = THREADS / TPL;                  // lines per pass
-  static constexpr bool WARP_LOCAL = TPL <= 32;
-  static constexpr int R0WS = (N >= 512 ? 8 : 16);
-  static constexpr int R = (LPP > R0WS ? (LPP < N ? LPP : N) : R0WS);  // rows per row item
-  static constexpr int PASSES = (R + LPP - 1) / LPP;
-  static constexpr int LL = fft_line_len<N, true, (R0WS == 8)>();  // padded line length
-  static constexpr size_t smem_z = sizeof(float2) * 2 * R * LL;
-  static constexpr size_t smem_y = sizeof(float2) * NB * LL;
-  static constexpr size_t smem_nodes = sizeof(float2) * R * N;  // (F, 1/|r|^2) per node of a row item
-  static constexpr size_t smem = sizeof(float2) * N + smem_nodes + (smem_z > smem_y ? smem_z : smem_y);
+  using L = LineFft<N>;
+  static constexpr int NG = GroupTable<ELL>::NG;
+  static constexpr int ND = ELL / 2;             // degrees 2, 4, 6: one complex line (c = 0, 1) per row each
+  static constexpr int NF = 1 + 2 * ND;          // source fields
+  static constexpr int NL = YLines<ELL>::NL;     // y lines per column
+  static constexpr int TPL = L::TPL, LINE = L::LINE, R1 = L::R1;
+  // 512 threads where a column's lines leave room for one CTA per SM only
+  static constexpr int THREADS = (size_t)NL * LINE * sizeof(float2) > 100 * 1024 || N >= 768 ? 512 : 256;
+  static constexpr int GROUPS = THREADS / TPL;   // lines transformed at once
+  // Rows per row item: a line per thread group, at least 8 rows (64-byte runs in the
+  // ring); half of that for l_max = 6 where the item's lines would take too much.
+  static constexpr int R0 = ELL == 0 ? 2 * GROUPS : (N <= 256 ? (ELL == 6 ? GROUPS / 2 : GROUPS) : 8);
+  static constexpr int R = R0 > N ? N : (N % R0 ? 8 : R0);
+  // With twice as many groups as rows, half of the groups take the upper degrees and F.
+  static constexpr bool SPLIT = ND > 1 && GROUPS >= 2 * R && (TPL >= 32 || R % (32 / TPL) == 0);
+  static constexpr int DSPLIT = SPLIT ? (ND + 1) / 2 : ND;  // degrees of the first half
+  static constexpr int RLINES = R * ND + R / 2;  // the F lines hold two rows each
+  // Columns per column item: as many as the thread groups transform at once.
+  static constexpr int kc() {
+    int k = 1;
+    while (2 * k * NL <= GROUPS && k < 16) k *= 2;
+    return k;
+  }
+  static constexpr int KC = kc();
+  static constexpr int CLINES = NL * KC;
+  static constexpr int LPG = (CLINES + GROUPS - 1) / GROUPS;  // lines per thread group
+  static constexpr int LINES = (RLINES > CLINES ? RLINES : CLINES) * LINE;  // elements of the line buffers
+  static constexpr int TWN = L::TWN;                                         // and of the twiddles
+  static constexpr size_t smem = sizeof(float2) * (LINES + TWN);
   static_assert(N % R == 0, "rows per item must divide N");
-  // Resident CTAs per SM the register budget is set for: two when two CTAs' shared
-  // memory fits the SM (228 KB, less 1 KB reserved per CTA), else one.
-  static constexpr int MIN_BLOCKS = 2 * (smem + 1024 + 64) <= 228 * 1024 ? 2 : 1;
+  // Resident CTAs per SM the register budget is set for: two of 256 threads when their
+  // shared memory fits the SM (228 KB, less 1 KB reserved per CTA), else one.
+  static constexpr int MIN_BLOCKS = THREADS == 256 && 2 * (smem + 1024 + 64) <= 228 * 1024 ? 2 : 1;
 };
-
-
-// Monomial of basis field beta (its exponents a, b, c and degree d, i = 0..3) at
-// compile time; fields past the last one (an odd count's partner) are zero.
-template <int ELL>
-__host__ __device__ constexpr int mono_ct(int beta, int i) {
-  return beta < GroupTable<ELL>::NB ? GroupTable<ELL>::mono_c(beta, i) : (i == 3 ? -2 : 0);
-}
-
-// Pair PR's two basis fields at the nodes of the R rows, built with their exponents
-// known at compile time, and the first FFT stage from registers into C.
-template <int N, int ELL, int PR>
-__device__ __forceinline__ void pair_stage0_ct(float2* C, const float2* nodes, float X, const float* __restrict__ rely,
-                                               const float* __restrict__ relz, int row0) {
-  using Y = YZ<N, ELL>;
-  constexpr int E = Y::E, TPL = Y::TPL, R0 = Y::R0, R = Y::R, LL = Y::LL, LPP = Y::LPP;
-  constexpr int FA = 2 * PR, FB = 2 * PR + 1;
-  constexpr int AA = mono_ct<ELL>(FA, 0), AB = mono_ct<ELL>(FA, 1), AC = mono_ct<ELL>(FA, 2), AD = mono_ct<ELL>(FA, 3);
-  constexpr int BA = mono_ct<ELL>(FB, 0), BB = mono_ct<ELL>(FB, 1), BC = mono_ct<ELL>(FB, 2), BD = mono_ct<ELL>(FB, 3);
-  const int tl = threadIdx.x % TPL;
-#pragma unroll
-  for (int ps = 0; ps < Y::PASSES; ++ps) {
-    const int row = ps * LPP + threadIdx.x / TPL;
-    if (row < R) {
-      const float Yc = rely[row0 + row];
-      const float2* nrow = nodes + row * N;
-      float2* lp = C + row * LL;
-      const float Ka = ipow_ct<AA>(X) * ipow_ct<AB>(Yc), Kb = ipow_ct<BA>(X) * ipow_ct<BB>(Yc);
-#pragma unroll 1
-      for (int q = 0; q < E / R0; ++q) {
-        float2 v[R0];
-#pragma unroll
-        for (int r = 0; r < R0; ++r) {
-          const int z = fft_in_index<N>(tl, q, r);
-          const float Zc = (AC | BC) ? relz[z] : 0.f;
-          const float2 fi = nrow[z];  // written by this thread in row_item
-          v[r] = make_float2(basis_value_ct<AC, AD>(fi.x, fi.y, Zc, Ka), basis_value_ct<BC, BD>(fi.x, fi.y, Zc, Kb));
-        }
-        Dft<R0>::run(v);
-        const int jq = tl + q * TPL;
-        if constexpr (16 % R0 == 0) {
-          float2* dst = lp + fft_pos<true>(jq * R0);  // element R0 jq + r sits r after R0 jq
-#pragma unroll
-          for (int r = 0; r < R0; ++r) dst[r] = v[r];
-        } else {
-#pragma unroll
-          for (int r = 0; r < R0; ++r) lp[fft_pos<true>(jq * R0 + r)] = v[r];
-        }
-      }
-    }
-  }
-}
-
-// Run-time pair index to the compile-time build above (a uniform chain of tests).
-template <int N, int ELL, int PR = 0>
-__device__ __forceinline__ void pair_stage0(int pr, float2* C, const float2* nodes, float X,
-                                            const float* __restrict__ rely, const float* __restrict__ relz, int row0) {
-  if constexpr (PR < YZ<N, ELL>::NPAIR) {
-    if (pr == PR) pair_stage0_ct<N, ELL, PR>(C, nodes, X, rely, relz, row0);
-    else pair_stage0<N, ELL, PR + 1>(pr, C, nodes, X, rely, relz, row0);
-  }
-}
-
-// One pair of basis fields (fa = 2 pr, fb = 2 pr + 1) for the R rows of a row item:
-// fields at the nodes (first FFT stage from registers, one butterfly at a time),
-// FFT along z, then the split of the two real fields into their half spectra,
-// written to the ring slot.  C is one of two line buffers, so the split of this pair
-// can overlap the FFT of the next.
-template <int N, int ELL>
-__device__ __forceinline__ void row_pair(int pr, float2* C, const float2* nodes, float X,
-                                         const float* __restrict__ rely, const float* __restrict__ relz, int row0,
-                                         const float2* tw, float2* __restrict__ zslot, int nzc) {
-  using Y = YZ<N, ELL>;
-  constexpr int TPL = Y::TPL, R = Y::R, LL = Y::LL;
-  pair_stage0<N, ELL>(pr, C, nodes, X, rely, relz, row0);
-  line_group_sync<TPL>();  // each line is written and read by its own threads
-  FftRun<N, 1, false, true, R>::run(C, 1, LL, R, tw);
-  __syncthreads();
-  // Split: thread t takes row r = t mod R and k_z = t / R + i KS.  When KS is a
-  // multiple of 16 the padded positions of k_z and N - k_z move by fixed steps.
-  static_assert(Y::THREADS % R == 0, "split stride");
-  constexpr int KS = Y::THREADS / R, PSTEP = KS / 16 * 17;
-  constexpr bool STEP = KS % 16 == 0;
-  const int r = threadIdx.x % R, kz0 = threadIdx.x / R;
-  const float2* crow = C + r * LL;
-  const float2* pk = crow + fft_pos<true>(kz0);
-  const float2* pm = crow + fft_pos<true>(N - kz0);  // only read for k_z > 0
-  // The ring holds the two fields of a pair side by side: one 16-byte store per node.
-  float4* za = reinterpret_cast<float4*>(zslot) + ((size_t)pr * nzc + kz0) * N + row0 + r;
-  for (int kz = kz0; kz < nzc; kz += KS, pk += PSTEP, pm -= PSTEP, za += (size_t)KS * N) {
-    const float2 ck = STEP ? *pk : crow[fft_pos<true>(kz)];
-    const float2 cm = kz ? (STEP ? *pm : crow[fft_pos<true>(N - kz)]) : ck;
-    // Two real fields a + i b: A = (C_k + C_{-k}^*)/2, B = (C_k - C_{-k}^*)/(2i) (B = 0
-    // past the last field).
-    *za = make_float4(0.5f * (ck.x + cm.x), 0.5f * (ck.y - cm.y), 0.5f * (ck.y + cm.y), -0.5f * (ck.x - cm.x));
-  }
-}
 
 // 1/x for a normal x > 0: the hardware approximation refined by one Newton-Raphson
 // step, y' = y + y (1 - x y), which leaves it within about an ulp (the correctly
@@ -276,109 +201,300 @@ __device__ __forceinline__ float recip_nr(float x) {
   return fmaf(y, fmaf(-x, y, 1.f), y);
 }
 
-// Row item: the mesh value F and 1/|r|^2 of every node of the R rows are formed once
-// (each thread for the nodes it later reads, so no barrier is needed), then every
-// pair of basis fields is built from them, transformed along z and split.
+// Row item: the source fields of R rows of one x-plane, transformed along z.  Each
+// degree's two real fields (c = 0, 1) go through one complex line; F goes through
+// half a line per row (rows 2 p and 2 p + 1 as real and imaginary part).  All lines of
+// the item stay in shared memory, so one barrier separates the transforms from the
+// split into half spectra, which writes runs of R rows to the ring slot
+// [k_z][source][y].
 template <int N, int ELL>
-__device__ __forceinline__ void row_item(float2* work, float2* nodes, const float* __restrict__ plane, float X,
-                                         const float* __restrict__ rely, const float* __restrict__ relz, int row0,
-                                         const float2* tw, float2* __restrict__ zslot, int nzc, int* ticket,
-                                         int& next) {
+__device__ __forceinline__ void row_item(float2* S, const float2* tws, const float* __restrict__ plane, float2 X,
+                                         const float2* __restrict__ rely, const float2* __restrict__ relz, int row0,
+                                         float2* __restrict__ zslot, int nzc, int* ticket, int& next) {
   using Y = YZ<N, ELL>;
-  constexpr int R = Y::R, LL = Y::LL, E = Y::E, TPL = Y::TPL, R0 = Y::R0, LPP = Y::LPP;
-  const int tl = threadIdx.x % TPL;
+  using L = typename Y::L;
+  constexpr int R = Y::R, LINE = L::LINE, R1 = L::R1, TPL = L::TPL, GROUPS = Y::GROUPS, ND = Y::ND, NF = Y::NF;
+  const int t = threadIdx.x % TPL, g = line_of_group<TPL>(threadIdx.x / TPL);
+  float2 tw[R1 - 1];
+  load_twiddles<N>(tw, tws, t);
+  const float2* wE = tws + (R1 - 1) * TPL;
+  if constexpr (ND > 0) {
+#pragma unroll 1
+    for (int r0 = 0; r0 < R; r0 += GROUPS) {
+      const bool upper = Y::SPLIT && g >= R;
+      const int r = r0 + g - (upper ? R : 0);
+      const bool ok = R % GROUPS == 0 || r < R;
+      if (TPL >= 32 && !ok) break;
+      float f[R1], i2[R1], irho = 1.f;
+      if (ok) {
+        const float2 Yc = rely[row0 + r];
+        const float xy2 = fmaf(X.x, X.x, Yc.x * Yc.x);
+        irho = fminf(X.y, Yc.y);  // a power of two, as 1 / irho: exact
+        const float rho2 = 1.f / (irho * irho);
+        const float* frow = plane + (size_t)(row0 + r) * N + t;
 #pragma unroll
-  for (int ps = 0; ps < Y::PASSES; ++ps) {
-    const int row = ps * LPP + threadIdx.x / TPL;
-    if (row < R) {
-      const float Yc = rely[row0 + row];
-      const float xy2 = fmaf(X, X, Yc * Yc);
-      const float* frow = plane + (size_t)(row0 + row) * N;
-      float2* nrow = nodes + row * N;
+        for (int k = 0; k < R1; ++k) f[k] = frow[k * TPL];
 #pragma unroll
-      for (int q = 0; q < E / R0; ++q)
-#pragma unroll
-        for (int r = 0; r < R0; ++r) {
-          const int z = fft_in_index<N>(tl, q, r);
-          const float Zc = relz[z];
+        for (int k = 0; k < R1; ++k) {
+          const float Zc = relz[t + k * TPL].x;
           const float r2 = fmaf(Zc, Zc, xy2);
-          nrow[z] = make_float2(frow[z], r2 > 0.f ? recip_nr(r2) : 0.f);
+          i2[k] = r2 > YZ_R2_MIN ? rho2 * recip_nr(r2) : 0.f;
         }
+      }
+#pragma unroll
+      for (int d = 0; d < ND; ++d) {
+        float2 v[R1];
+        if (ok) {
+#pragma unroll
+          for (int k = 0; k < R1; ++k) {
+            f[k] *= i2[k];
+            v[k] = make_float2(f[k], f[k] * (relz[t + k * TPL].x * irho));
+          }
+        }
+        if (Y::SPLIT && (d >= Y::DSPLIT) != upper) continue;
+        line_fft<N>(v, S + (d * R + r) * LINE, t, tw, wE, ok);
+      }
     }
   }
 #pragma unroll 1
-  for (int pr = 0; pr < Y::NPAIR; ++pr) {
-    if (pr == Y::NPAIR - 1 && threadIdx.x == 0) next = atomicAdd(ticket, 1);  // see k_yz
-    row_pair<N, ELL>(pr, work + (pr & 1) * R * LL, nodes, X, rely, relz, row0, tw, zslot, nzc);
+  for (int p0 = 0; p0 < R / 2; p0 += GROUPS) {
+    const int p = p0 + g - (Y::SPLIT ? R : 0);
+    const bool ok = p >= 0 && p < R / 2;
+    if (TPL >= 32 && !ok) break;
+    float2 v[R1];
+    if (ok) {
+      const float* frow = plane + (size_t)(row0 + 2 * p) * N + t;
+#pragma unroll
+      for (int k = 0; k < R1; ++k) v[k] = make_float2(frow[k * TPL], frow[N + k * TPL]);
+    }
+    line_fft<N>(v, S + (ND * R + p) * LINE, t, tw, wE, ok);
+  }
+  if (threadIdx.x == 0) next = atomicAdd(ticket, 1);  // see k_yz
+  __syncthreads();
+  // Two real lines a + i b: A_k = (C_k + C_{N-k}^*)/2, B_k = (C_k - C_{N-k}^*)/(2i).
+  if constexpr (ND > 0) {
+    constexpr int RL = R < 16 ? R : 16, KS = Y::THREADS / RL;
+#pragma unroll 1
+    for (int rb = 0; rb < R; rb += RL) {
+      const int r = rb + threadIdx.x % RL;
+#pragma unroll 1
+      for (int d = 0; d < ND; ++d) {
+        const float2* line = S + (d * R + r) * LINE;
+        float2* out = zslot + (size_t)(1 + 2 * d) * N + row0 + r;
+        for (int i = threadIdx.x / RL; i < L::HALF_ITEMS; i += KS)
+          line_halves<N>(line, i, nzc, [&](int kz, float2 A, float2 B) {
+            float2* o = out + (size_t)kz * NF * N;
+            o[0] = A;
+            o[N] = B;
+          });
+      }
+    }
+  }
+  {
+    constexpr int PL = R / 2 < 16 ? R / 2 : 16, KS = Y::THREADS / PL;
+#pragma unroll 1
+    for (int pb = 0; pb < R / 2; pb += PL) {
+      const int p = pb + threadIdx.x % PL;
+      const float2* line = S + (ND * R + p) * LINE;
+      float2* out = zslot + row0 + 2 * p;
+      for (int i = threadIdx.x / PL; i < L::HALF_ITEMS; i += KS)
+        line_halves<N>(line, i, nzc, [&](int kz, float2 A, float2 B) {
+          *reinterpret_cast<float4*>(out + (size_t)kz * NF * N) = make_float4(A.x, A.y, B.x, B.y);
+        });
+    }
   }
 }
 
+// Fold of one column (k_z): the y transforms of the basis fields at k_y become the
+// k_x-power groups, written for the column's pencils.  The column's lines start at S.
+// F' at the plane of the node at r = 0 (org): the transform of F less that node's
+// value times its phase.
 template <int N, int ELL>
 __device__ __forceinline__ void column_fold(const float2* S, int kz, const int* __restrict__ col_off,
-                                         float2* __restrict__ gout, int j, int ix, int np) {
+                                            float2* __restrict__ gout, int j, int ix, int np, const int* org,
+                                            const float* __restrict__ mesh, int tid, int nthr) {
   using Y = YZ<N, ELL>;
-  constexpr int NG = Y::NG, LL = Y::LL;
+  using L = typename Y::L;
+  constexpr int NG = Y::NG, NL = Y::NL, LINE = L::LINE, M = N / L::E2;
+  [[maybe_unused]] constexpr bool HOLD = NL <= 15;  // both halves of every line in registers
   const int p0 = col_off[kz];
   const int cnt = col_off[kz + 1] - p0;
   const int kymax = (cnt - 1) / 2;
   const size_t gstep = (size_t)N * np;  // between groups
-  float2* g0 = gout + ((size_t)j * NG * N + ix) * np + p0;
-  // Lanes start at a multiple of 16 of the line position (k_y = -kymax sits at
-  // N - kymax), so each half-warp reads 16 consecutive, 16-aligned elements.
-  const int lead = (N - kymax) & 15;
-  for (int q = (int)threadIdx.x - lead; q < cnt; q += blockDim.x) {
-    if (q < 0) continue;
-    const int ky = q - kymax;
-    const float2* sp = S + fft_pos<true>(ky < 0 ? ky + N : ky);
-    float2 g[NG];
-    GroupTable<ELL>::combine([&](int f) { return sp[f * LL]; }, (float)ky, (float)kz, g);
-    float2* gp = g0 + q;
+  float2* g0 = gout + ((size_t)j * NG * N + ix) * np + p0 + kymax;
+  const bool at_org = ELL > 0 && ix == org[0];
+  float f0 = 0.f;
+  if (at_org) f0 = mesh[((size_t)ix * N + org[1]) * N + org[2]];
+  // line(l): the transform of the column's line l at k_y
+  auto emit = [&](auto&& line, int ky) {
+    const float2 F0 = line(0);
+    float2 Fp = F0;
+    if (at_org) {
+      const int turn = (((ky * org[1] + kz * org[2]) % N) + N) % N;
+      float sn, cs;
+      sincospif((float)(2 * turn) / (float)N, &sn, &cs);
+      Fp = make_float2(fmaf(-f0, cs, Fp.x), fmaf(f0, sn, Fp.y));
+    }
+    float2 gr[NG];
+    GroupTable<ELL>::combine([&](int f) { return f == 0 ? F0 : (f == 1 ? Fp : line(f - 1)); }, (float)ky, (float)kz, gr);
+    float2* gp = g0 + ky;
 #pragma unroll
-    for (int gi = 0; gi < NG; ++gi) gp[gi * gstep] = g[gi];
+    for (int gi = 0; gi < NG; ++gi) gp[gi * gstep] = gr[gi];
+  };
+  if constexpr (L::E2 == 1) {
+    // Lanes start at a multiple of 16 of the line position (k_y = -kymax sits at
+    // N - kymax), so each half-warp reads 16 consecutive, 16-aligned frequencies.
+    const int lead = (N - kymax) & 15;
+    for (int q = tid - lead; q < cnt; q += nthr) {
+      if (q < 0) continue;
+      const int ky = q - kymax;
+      const float2* sp = S + L::slot(ky < 0 ? ky + N : ky);
+      emit([&](int l) { return sp[l * LINE]; }, ky);
+    }
+  } else if constexpr (L::E2 == 2) {
+    // slots of kappa hold the halves of k_y = kappa and kappa - N/2
+    for (int kap = tid; kap < M; kap += nthr) {
+      const bool up = kap <= kymax, dn = M - kap <= kymax;
+      if (!up && !dn) continue;
+      const float2* sp = S + L::slot(kap);
+      if constexpr (HOLD) {
+        float2 Ta[NL], Tb[NL];
+#pragma unroll
+        for (int l = 0; l < NL; ++l) {
+          const float4 q = *reinterpret_cast<const float4*>(sp + l * LINE);
+          const float2 x = make_float2(q.x, q.y), y = make_float2(q.z, q.w);
+          Ta[l] = cadd(x, y);
+          Tb[l] = csub(x, y);
+        }
+        if (up) emit([&](int l) { return Ta[l]; }, kap);
+        if (dn) emit([&](int l) { return Tb[l]; }, kap - M);
+      } else {
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {
+          if (half ? !dn : !up) continue;
+          const float2 sg = half ? make_float2(-1.f, -1.f) : make_float2(1.f, 1.f);
+          emit([&](int l) {
+            const float4 q = *reinterpret_cast<const float4*>(sp + l * LINE);
+            return __ffma2_rn(make_float2(q.z, q.w), sg, make_float2(q.x, q.y));
+          }, kap - half * M);
+        }
+      }
+    }
+  } else {
+    // four quarters: unit (kappa, odd) gives k_y = kappa + odd M and kappa + (odd - 2) M
+    for (int u = tid; u < 2 * M; u += nthr) {
+      const int odd = u >= M ? 1 : 0, kap = u - odd * M;
+      const int kya = kap + odd * M, kyb = kap + (odd - 2) * M;
+      const bool up = kya <= kymax, dn = -kyb <= kymax;
+      if (!up && !dn) continue;
+      const float2* sp = S + L::slot(kap);
+      float2 Ta[NL], Tb[NL];
+#pragma unroll
+      for (int l = 0; l < NL; ++l) {
+        const float4 q0 = *reinterpret_cast<const float4*>(sp + l * LINE);
+        const float4 q1 = *reinterpret_cast<const float4*>(sp + l * LINE + 2);
+        const float2 x0 = make_float2(q0.x, q0.y), x1 = make_float2(q0.z, q0.w);
+        const float2 x2 = make_float2(q1.x, q1.y), x3 = make_float2(q1.z, q1.w);
+        if (odd) {
+          const float2 s = csub(x0, x2), d = csub(x1, x3);
+          Ta[l] = add_mi(s, d);
+          Tb[l] = sub_mi(s, d);
+        } else {
+          const float2 s = cadd(x0, x2), d = cadd(x1, x3);
+          Ta[l] = cadd(s, d);
+          Tb[l] = csub(s, d);
+        }
+      }
+      if (up) emit([&](int l) { return Ta[l]; }, kya);
+      if (dn) emit([&](int l) { return Tb[l]; }, kyb);
+    }
   }
 }
 
+// Column item: the y transforms of KC columns (k_z) of one plane.  A thread group
+// loads a source line, multiplies it by (X / rho)^a (Y / rho)^b and transforms it, LPG
+// lines in turn.  The exponents are uniform over the group, so the tests on their bits
+// skip whole unrolled loops where a group is a warp or more.
 template <int N, int ELL>
-__device__ __forceinline__ void column_item(float2* S, const float2* __restrict__ zs, int nzc, int kz,
-                                            const int* __restrict__ col_off, const float2* tw,
-                                            float2* __restrict__ gout, int j, int ix, int np, int* ticket, int& next) {
+__device__ __forceinline__ void column_item(float2* S, const float2* tws, const float2* __restrict__ zslot, int kz0,
+                                            const YZParams& prm, int j, int ix, int* ticket, int& next) {
   using Y = YZ<N, ELL>;
-  constexpr int NB = Y::NB, NP = Y::NPAIR, E = Y::E, TPL = Y::TPL, R0 = Y::R0, LL = Y::LL, LPP = Y::LPP;
-  const int tl = threadIdx.x % TPL;
-  // One ring line holds a pair of fields (16 bytes per node): a thread group loads
-  // both and runs the first FFT stage of each.
-  for (int base = 0; base < NP; base += LPP) {
-    const int pr = base + threadIdx.x / TPL;
-    if (pr < NP) {
-      const float4* line = reinterpret_cast<const float4*>(zs) + ((size_t)pr * nzc + kz) * N;
-      float2 va[E], vb[E];
+  using L = typename Y::L;
+  constexpr int LINE = L::LINE, R1 = L::R1, TPL = L::TPL, NF = Y::NF, NL = Y::NL, KC = Y::KC, LPG = Y::LPG;
+  const int t = threadIdx.x % TPL, g = line_of_group<TPL>(threadIdx.x / TPL);
+  const int ncol = min(KC, prm.nzc - kz0);
+  const float2* __restrict__ rel = prm.rel + (size_t)j * 3 * N;
+  const float2* __restrict__ rely = rel + N + t;
+  const float2 X = rel[ix];
+  {
+    float2 tw[R1 - 1];
+    load_twiddles<N>(tw, tws, t);
+    const float2* wE = tws + (R1 - 1) * TPL;
+#pragma unroll 1
+    for (int i = 0; i < LPG; ++i) {
+      const int l = g * LPG + i, c = l / NL, ln = l - c * NL;
+      const bool ok = c < ncol;
+      if (TPL >= 32 && !ok) break;
+      float2 v[R1];
+      if (ok) {
+        const float2* zl = zslot + ((size_t)(kz0 + c) * NF + kYLines<ELL>.src[ln]) * N + t;
 #pragma unroll
-      for (int q = 0; q < E / R0; ++q)
+        for (int k = 0; k < R1; ++k) v[k] = __ldcg(zl + k * TPL);
+        if constexpr (ELL > 0) {
+          const int ea = kYLines<ELL>.a[ln], eb = kYLines<ELL>.b[ln];
+          if (ea | eb) {
+            float2 u[R1];  // (X, Y) / rho, then its squares and fourth powers
+            float K[R1];
 #pragma unroll
-        for (int r = 0; r < R0; ++r) {
-          const float4 t = __ldcg(line + fft_in_index<N>(tl, q, r));
-          va[q * R0 + r] = make_float2(t.x, t.y);
-          vb[q * R0 + r] = make_float2(t.z, t.w);
+            for (int k = 0; k < R1; ++k) {
+              const float2 Yc = rely[k * TPL];
+              const float irho = fminf(X.y, Yc.y);
+              u[k] = __fmul2_rn(make_float2(X.x, Yc.x), make_float2(irho, irho));
+              K[k] = (ea & 1) ? u[k].x : 1.f;
+            }
+            if (eb & 1) {
+#pragma unroll
+              for (int k = 0; k < R1; ++k) K[k] *= u[k].y;
+            }
+            if ((ea | eb) > 1) {
+#pragma unroll
+              for (int k = 0; k < R1; ++k) {
+                u[k] = __fmul2_rn(u[k], u[k]);
+                if (ea & 2) K[k] *= u[k].x;
+                if (eb & 2) K[k] *= u[k].y;
+              }
+            }
+            if (ELL >= 4 && (ea | eb) > 3) {
+#pragma unroll
+              for (int k = 0; k < R1; ++k) {
+                u[k] = __fmul2_rn(u[k], u[k]);
+                if (ea & 4) K[k] *= u[k].x;
+                if (eb & 4) K[k] *= u[k].y;
+              }
+            }
+#pragma unroll
+            for (int k = 0; k < R1; ++k) v[k] = __fmul2_rn(v[k], make_float2(K[k], K[k]));
+          }
         }
-      fft_stage0_regs<N, true>(va, S + 2 * pr * LL, 1, tl);
-      if (2 * pr + 1 < NB) fft_stage0_regs<N, true>(vb, S + (2 * pr + 1) * LL, 1, tl);
+      }
+      line_fft<N>(v, S + l * LINE, t, tw, wE, ok);
     }
   }
-  __syncthreads();  // every ring load is done; lines 2 pr, 2 pr + 1 came from pair pr's threads
-  // The ring lines of this column are dead once read: drop them from L2 without a
+  __syncthreads();  // every ring load is done, every line transformed
+  // The ring lines of these columns are dead once read: drop them from L2 without a
   // write-back (the slot is rewritten only after this item's completion is
-  // released).  Each line is N * 16 bytes, a whole number of 128-byte lines.
-  for (int base = 0; base < NP; base += LPP) {
-    const int pr = base + threadIdx.x / TPL;
-    if (pr < NP) {
-      const float4* line = reinterpret_cast<const float4*>(zs) + ((size_t)pr * nzc + kz) * N;
-      for (int c = tl; c < N / 8; c += TPL) asm volatile("discard.global.L2 [%0], 128;" ::"l"(line + c * 8) : "memory");
-    }
+  // released).  A column is NF * N * 8 bytes, a whole number of 128-byte lines.
+  {
+    const float2* dead = zslot + (size_t)kz0 * NF * N;
+    for (int c = threadIdx.x; c < ncol * (NF * N / 16); c += Y::THREADS)
+      asm volatile("discard.global.L2 [%0], 128;" ::"l"(dead + c * 16) : "memory");
   }
-  FftRun<N, 1, false, true, NB>::run(S, 1, LL, NB, tw);
-  __syncthreads();
   if (threadIdx.x == 0) next = atomicAdd(ticket, 1);  // see k_yz
-  column_fold<N, ELL>(S, kz, col_off, gout, j, ix, np);
+  constexpr int NTHR = Y::THREADS / KC;
+  const int c = threadIdx.x / NTHR;
+  if (c < ncol)
+    column_fold<N, ELL>(S + c * NL * LINE, kz0 + c, prm.col_off, prm.gout, j, ix, prm.np, prm.org[j],
+                        prm.mesh + (size_t)j * N * N * N, threadIdx.x % NTHR, NTHR);
 }
 
 // Completion of one item: every thread's writes are ordered before thread 0's
@@ -389,17 +505,18 @@ __device__ __forceinline__ void signal_release(int* counter) {
 }
 
 template <int N, int ELL>
-__global__ void __launch_bounds__(256, YZ<N, ELL>::MIN_BLOCKS) k_yz(const __grid_constant__ YZMulti pm) {
+__global__ void __launch_bounds__(YZ<N, ELL>::THREADS, YZ<N, ELL>::MIN_BLOCKS) k_yz(const __grid_constant__ YZMulti pm) {
   using Y = YZ<N, ELL>;
+  using L = typename Y::L;
   constexpr int R = Y::R;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_item;
   __shared__ int s_ok;
-  float2* tw = reinterpret_cast<float2*>(smem_raw);
-  float2* nodes = tw + N;
-  float2* work = nodes + (Y::smem_nodes / sizeof(float2));
-  for (int k = threadIdx.x; k < N; k += blockDim.x) tw[k] = pm.lane[0].tw[k];  // same N: same twiddles
-  const int NZ = N / R;
+  float2* work = reinterpret_cast<float2*>(smem_raw);
+  // Twiddles of the line transforms (same N: the same for every lane).
+  float2* tws = work + Y::LINES;
+  for (int k = threadIdx.x; k < Y::TWN; k += Y::THREADS) tws[k] = pm.lane[0].tw[k];
+  constexpr int NZ = N / R;
   const int total = pm.end[pm.nlanes - 1];
   const size_t n3 = (size_t)N * N * N;
   if (threadIdx.x == 0) s_item = atomicAdd(pm.ticket, 1);
@@ -407,11 +524,11 @@ __global__ void __launch_bounds__(256, YZ<N, ELL>::MIN_BLOCKS) k_yz(const __grid
   int gitem = s_item;
   for (;;) {
     if (gitem >= total) break;
-    // Thread 0 claims the next ticket shortly before this item ends (before the last
-    // field pair of a row item, before the fold of a column item), so that the
-    // atomic's round trip overlaps the item's tail.  A claimed item starts that
-    // little later; claiming a whole item ahead delayed the items waiting on it too
-    // much.  Items wait only on items of earlier tickets, so the list cannot deadlock.
+    // Thread 0 claims the next ticket shortly before this item ends (before the split
+    // of a row item, before the fold of a column item), so that the atomic's round
+    // trip overlaps the item's tail.  A claimed item starts that little later;
+    // claiming a whole item ahead delayed the items waiting on it too much.  Items
+    // wait only on items of earlier tickets, so the list cannot deadlock.
     int next = -1;
     {  // L2 prefetch of the mesh rows of the row item one grid of tickets ahead
       const int ahead = gitem + (int)gridDim.x;
@@ -420,7 +537,7 @@ __global__ void __launch_bounds__(256, YZ<N, ELL>::MIN_BLOCKS) k_yz(const __grid
         while (ahead >= pm.end[la]) ++la;
         const YZParams& pa = pm.lane[la];
         const int ia = ahead - (la > 0 ? pm.end[la - 1] : 0);
-        const int ipa = NZ + pa.nzc, sta = ia / ipa, sba = ia - sta * ipa;
+        const int ipa = NZ + (pa.nzc + Y::KC - 1) / Y::KC, sta = ia / ipa, sba = ia - sta * ipa;
         if (sba < NZ && sta < pa.m * N) {
           const int ja = sta / N, xa = sta - ja * N;
           const float* rows = pa.mesh + ja * n3 + (size_t)xa * N * N + (size_t)sba * R * N;
@@ -432,9 +549,9 @@ __global__ void __launch_bounds__(256, YZ<N, ELL>::MIN_BLOCKS) k_yz(const __grid
     while (gitem >= pm.end[l]) ++l;
     const YZParams& prm = pm.lane[l];
     const int item = gitem - (l > 0 ? pm.end[l - 1] : 0);
-    const int NY = prm.nzc, IPS = NZ + NY;
+    const int NY = (prm.nzc + Y::KC - 1) / Y::KC, IPS = NZ + NY;
     const int mN = prm.m * N;
-    const size_t slot_elems = (size_t)2 * Y::NPAIR * prm.nzc * N;  // float2 units, field pairs interleaved
+    const size_t slot_elems = (size_t)Y::NF * prm.nzc * N;  // float2 units
     const int step = item / IPS, sub = item - step * IPS;
     if (sub < NZ) {
       const int p = step;  // row item of plane p
@@ -444,9 +561,9 @@ __global__ void __launch_bounds__(256, YZ<N, ELL>::MIN_BLOCKS) k_yz(const __grid
         __syncthreads();
         if (!s_ok) break;
         const int j = p / N, ix = p - j * N;
-        const float* rel = prm.rel + (size_t)j * 3 * N;
-        row_item<N, ELL>(work, nodes, prm.mesh + j * n3 + (size_t)ix * N * N, rel[ix], rel + N, rel + 2 * N, sub * R,
-                         tw, prm.ring + (size_t)(p % prm.S) * slot_elems, prm.nzc, pm.ticket, next);
+        const float2* rel = prm.rel + (size_t)j * 3 * N;
+        row_item<N, ELL>(work, tws, prm.mesh + j * n3 + (size_t)ix * N * N, rel[ix], rel + N, rel + 2 * N, sub * R,
+                         prm.ring + (size_t)(p % prm.S) * slot_elems, prm.nzc, pm.ticket, next);
         if (p != prm.skip_plane) signal_release(prm.done_z + p);
         else __syncthreads();  // withheld: the column items of plane p wait until their limit
       }
@@ -457,8 +574,8 @@ __global__ void __launch_bounds__(256, YZ<N, ELL>::MIN_BLOCKS) k_yz(const __grid
         __syncthreads();
         if (!s_ok) break;
         const int j = p / N, ix = p - j * N;
-        column_item<N, ELL>(work, prm.ring + (size_t)(p % prm.S) * slot_elems, prm.nzc, sub - NZ, prm.col_off, tw,
-                            prm.gout, j, ix, prm.np, pm.ticket, next);
+        column_item<N, ELL>(work, tws, prm.ring + (size_t)(p % prm.S) * slot_elems, (sub - NZ) * Y::KC, prm, j, ix,
+                            pm.ticket, next);
         signal_release(prm.done_y + p);
       }
     }
@@ -566,7 +683,7 @@ __device__ __forceinline__ float two_sum_err(float a, float b) {
 template <int N, int ELL, int M, int PX = k3_pencils(N)>
 struct XCombine {
   static constexpr int P = PX;  // pencils per CTA
-  static constexpr int E = fft_elems_lf(N);
+  static constexpr int E = fft_elems(N);
   static constexpr int TPL = N / E;
   static constexpr int THREADS = P * TPL;
   static constexpr int NW = THREADS / 32;
@@ -695,7 +812,7 @@ k_x_combine(const __grid_constant__ XMulti pm, int np_pad, const short2* __restr
     const float2* Tf = (SM_STAGES % 2 == 0) ? Tb : Wk;
     constexpr int PADF = (SM_STAGES % 2 == 0) ? 0 : XC::PADW;
     float2 v[E];
-    fft_last_stage_regs<N, true, false, PADF>(Tf, p, P, tl, tw, v);
+    fft_last_stage_regs<N, PADF>(Tf, p, P, tl, tw, v);
     const int first = group_first(gi);
     const int pw = gi - first;  // power of k_x
 #pragma unroll

@@ -48,11 +48,27 @@ struct Geom {
   int tdim[3];      // tile extent per axis
 };
 
+// Nodes with |r|^2 (r from the observer, in units of the mesh's largest |r| component
+// rounded up to a power of two) at most this, 2^-60, carry no line-of-sight weight: at
+// 2^-30 of the mesh's extent the direction is rounding noise, and one node at most is
+// that near.
+constexpr float YZ_R2_MIN = 8.673617379884035e-19f;
+
+// Launch shape of the y,z kernel for one mesh size and l_max.
+struct YzShape {
+  int grid = 0;             // resident CTAs
+  int rows = 1, cols = 1;   // rows per row item, columns per column item
+  double w_row = 1, w_col = 1;  // their work in FFT-line units (for the ring lead)
+};
+
 struct Plan {
   ys_config cfg;
   cudaStream_t stream = nullptr;
   int n = 0, m = 1, ell = 0, kind = 2;
-  int nb = 1, ng = 1;            // basis fields / k_x-power groups
+  int nf = 1, ng = 1;            // source fields of the z transforms / k_x-power groups
+  int yz_rows = 1, yz_cols = 1;  // rows per row item, columns per column item of the y,z kernel
+  double yz_w_row = 1, yz_w_col = 1;  // their work, in FFT-line units
+  int org[2][3] = {{-1, 0, 0}, {-1, 0, 0}};  // node at the observer of each mesh (x < 0: none)
   int row_len = 0;               // doubles in a result row (result_row_len)
   double H = 0, kf = 0;
   Geom geom{};
@@ -73,9 +89,10 @@ struct Plan {
   bool direct_assign = false;    // assignment by global reductions into an L2-resident mesh
   bool direct_ok = false;        // the mesh set is small enough for it (m N^3 floats <= 64 MB)
   // device tables
-  float2* d_tw = nullptr;        // [n] exp(-2 pi i j / n)
+  float2* d_tw = nullptr;        // [n] stage-major twiddles of the x stage (fft_tw_offset)
+  float2* d_twl = nullptr;       // twiddles of the y,z stage's line transforms (LineFft)
   float2* d_nodes = nullptr;     // [3][n + 3] node positions (hi, lo), index offset 1
-  float* d_rel = nullptr;        // [m][3][n] node - observer (float)
+  float2* d_rel = nullptr;       // [m][3][n] node - observer v in units of a power of two, 2^-floor(log2 |v|)
   float* d_invw = nullptr;       // [n] per-axis 1 / sinc^p by FFT index (1 if !compensate)
   float2* d_phase = nullptr;     // [n] per-axis exp(-i pi m / n) by FFT index
   int* d_col_off = nullptr;      // [nzc + 1] first pencil of each k_z column
@@ -84,7 +101,7 @@ struct Plan {
   double* d_shell = nullptr;     // [2][n_bins] mode count and sum |k| (host-built)
   // buffers
   float* d_mesh = nullptr;       // [m][n][n][n]
-  float2* d_z = nullptr;         // [S][nb][nzc][n] y,z-stage ring of z-transformed planes
+  float2* d_z = nullptr;         // [S][nzc][nf][n] y,z-stage ring of z-transformed planes
   int* d_sync = nullptr;         // [2 m n + 2] per-plane counters, ticket, error flag
   float2* d_g = nullptr;         // [m][ng][n][np_pad] grouped y,z transforms
   CUtensorMap gmap;              // 2D tensor map of d_g for the x-stage TMA loads
