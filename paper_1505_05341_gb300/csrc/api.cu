@@ -81,20 +81,22 @@ __global__ void k_finalize(const __grid_constant__ FinMulti fm, const double* __
   const double alpha = alpha_cfg >= 0.0 ? alpha_cfg : sums[SUM_WG] / sums[SUM_WR];
   const double I = alpha * sums[SUM_WR2N];
   const double S = sums[SUM_WG2] + alpha * alpha * sums[SUM_WR2];
+  const double inv_I = 1.0 / I;
   const double nan = __longlong_as_double(0x7ff8000000000000ULL);
   for (int b = threadIdx.x; b < nbins; b += blockDim.x) {
     const double nm = shell[b];
     double km = nan, p0 = nan, p2 = nan, p4 = nan, p6 = nan;
     if (nm > 0.0) {
-      km = shell[nbins + b] / nm;
-      const double m0 = acc[b] / nm, m2 = acc[nbins + b] / nm, m4 = acc[2 * nbins + b] / nm;
+      const double inv_nm = 1.0 / nm;  // FP64 divisions are long chains on this GPU: one per shell
+      km = shell[nbins + b] * inv_nm;
+      const double m0 = acc[b] * inv_nm, m2 = acc[nbins + b] * inv_nm, m4 = acc[2 * nbins + b] * inv_nm;
       // Eqs. (6)-(8), shot noise subtracted from the monopole only (Eq. 3).
-      p0 = (m0 - S) / I;
-      if (ell >= 2) p2 = 2.5 / I * (3.0 * m2 - m0);
-      if (ell >= 4) p4 = 1.125 / I * (35.0 * m4 - 30.0 * m2 + 3.0 * m0);
+      p0 = (m0 - S) * inv_I;
+      if (ell >= 2) p2 = 2.5 * inv_I * (3.0 * m2 - m0);
+      if (ell >= 4) p4 = 1.125 * inv_I * (35.0 * m4 - 30.0 * m2 + 3.0 * m0);
       // l = 6, the same step one order up: 13/I <Re A_0 L_6^*>, L_6(mu) =
       // (231 mu^6 - 315 mu^4 + 105 mu^2 - 5) / 16 written with the mu-power sums.
-      if (ell >= 6) p6 = 0.8125 / I * (231.0 * acc[3 * nbins + b] / nm - 315.0 * m4 + 105.0 * m2 - 5.0 * m0);
+      if (ell >= 6) p6 = 0.8125 * inv_I * (231.0 * (acc[3 * nbins + b] * inv_nm) - 315.0 * m4 + 105.0 * m2 - 5.0 * m0);
     }
     res[b] = km;
     res[nbins + b] = nm;
@@ -106,7 +108,7 @@ __global__ void k_finalize(const __grid_constant__ FinMulti fm, const double* __
   if (threadIdx.x == 0) {
     res[5 * nbins + 0] = alpha;
     res[5 * nbins + 1] = I;
-    res[5 * nbins + 2] = S / I;
+    res[5 * nbins + 2] = S * inv_I;
     res[5 * nbins + 3] = sums[SUM_BAD];
     res[5 * nbins + 4] = (double)flags[0];
   }
@@ -369,7 +371,9 @@ void set_tiles(Plan& p, int tx, int ty, int tz) {
   const int t[3] = {tx, ty, tz};
   p.ntiles = 1;
   for (int a = 0; a < 3; ++a) {
-    p.geom.tdim[a] = std::min(t[a], p.n);
+    p.geom.tdim[a] = std::min(t[a], p.n);  // 8, 16 or 32: every supported n is at least 16
+    p.geom.tshift[a] = 0;
+    while (1 << p.geom.tshift[a] < p.geom.tdim[a]) ++p.geom.tshift[a];
     p.geom.tiles[a] = p.n / p.geom.tdim[a];
     p.ntiles *= p.geom.tiles[a];
   }

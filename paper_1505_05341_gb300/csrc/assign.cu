@@ -11,19 +11,22 @@
 // tile it touches (at most 8), so tiles never write each other's nodes: no global
 // atomics on the mesh and no zero-fill pass.
 //
-//   k_count   : cell index per particle, FP64-accumulated sums, per-tile counts
-//   k_scan    : exclusive scan of the counts (one CTA)
-//   k_bin     : one 16-byte record (position, signed weight) per tile touched;
-//               records whose stencils lie inside one tile fill its list from the
-//               front, the others from the back, so the deposit walks the interior
-//               ones without per-node range checks
-//               (the deposit locates the particle again: 20-byte records with the
-//               cell index cost two partial L2 sector writes each)
-//   k_deposit : per-tile shared-memory deposit and store
+//   k_particles : cell index per particle, compensated sums, per-tile counts
+//   k_scan      : exclusive scan of the counts
+//   k_bin_agg / k_bin : one 16-byte record (position, signed weight) per tile touched;
+//                 records whose stencils lie inside one tile fill its list from the
+//                 front, the others from the back, so the deposit walks the interior
+//                 ones without per-node range checks
+//                 (the deposit locates the particle again: 20-byte records with the
+//                 cell index cost two partial L2 sector writes each)
+//   k_deposit   : per-tile shared-memory deposit and store
+//
+// Both catalogues go through one launch of each pass (Cats).
 //
 // Sub-cell offsets are formed against a host-built FP64 table of node positions
 // split into float (hi, lo) pairs, so d = u - floor(u) keeps ~1e-7 accuracy even
 // where u = (x - box_min)/H itself is only good to ~1e-5 in float.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -36,10 +39,74 @@ namespace {
 
 constexpr int THREADS = 256;
 
-__device__ __forceinline__ double warp_sum(double v) {
+// Galaxies and randoms of one launch: blocks [0, blocks0) take the galaxies, the others
+// the randoms.
+struct Cats {
+  const float* x[2];
+  const float* y[2];
+  const float* z[2];
+  const float* w[2];
+  const float* nbar[2];
+  int64_t n[2];
+  int blocks0;
+};
+
+// This block's catalogue (0 galaxies, 1 randoms), its place among that catalogue's
+// blocks and their number.
+__device__ __forceinline__ int block_catalogue(const Cats& c, int& bid, int& nblk) {
+  const int k = (int)blockIdx.x >= c.blocks0;
+  bid = blockIdx.x - (k ? c.blocks0 : 0);
+  nblk = k ? gridDim.x - c.blocks0 : c.blocks0;
+  return k;
+}
+
+// (s, c) += (s2, c2) for float sums with their collected rounding errors (TwoSum).
+__device__ __forceinline__ void pair_add(float& s, float& c, float s2, float c2) {
+  const float t = s + s2, bb = t - s;
+  c += c2 + ((s - (t - bb)) + (s2 - bb));
+  s = t;
+}
+
+// Sums of w, w^2 and w^2 nbar over this thread's particles: compensated float (Kahan).
+struct ThreadSums {
+  float s[3] = {0.f, 0.f, 0.f}, c[3] = {0.f, 0.f, 0.f};
+  __device__ __forceinline__ void kahan(int k, float v) {
+    const float y = v - c[k], t = s[k] + y;
+    c[k] = (t - s[k]) - y;
+    s[k] = t;
+  }
+};
+
+// Adds the block's sums (and its count of particles outside the box) to the catalogue
+// sums.  Threads meet in compensated float pairs (~2^-46; an FP64 shuffle tree of three
+// sums took 15 x 16 cycles of the SM per warp) and each CTA makes one FP64 atomic per
+// sum: per-warp atomics on the three addresses alone took ~30 us per catalogue.
+template <int NT>
+__device__ __forceinline__ void block_sums(ThreadSums& ts, unsigned bad, int is_ran, double* __restrict__ sums) {
+  __shared__ float2 red[NT / 32][3];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+  for (int k = 0; k < 3; ++k) {
+    float s = ts.s[k], c = -ts.c[k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      pair_add(s, c, __shfl_xor_sync(0xffffffffu, s, o), __shfl_xor_sync(0xffffffffu, c, o));
+    if (lane == 0) red[wid][k] = make_float2(s, c);
+  }
+  const int nbad = __syncthreads_or(bad != 0);
+  if (nbad) {
+    unsigned tot = bad;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+    if (lane == 0 && tot) atomicAdd(&sums[SUM_BAD], (double)tot);
+  }
+  if (threadIdx.x < 3) {
+    const int k = threadIdx.x;
+    float s = red[0][k].x, c = red[0][k].y;
+    for (int q = 1; q < NT / 32; ++q) pair_add(s, c, red[q][k].x, red[q][k].y);
+    const int slot = is_ran ? (k == 0 ? SUM_WR : (k == 1 ? SUM_WR2 : SUM_WR2N)) : (k == 0 ? SUM_WG : SUM_WG2);
+    if (is_ran || k < 2) atomicAdd(&sums[slot], (double)s + (double)c);
+  }
 }
 
 // Cell index i and offset d in [0, 1) of coordinate x along one axis.  Returns
@@ -48,16 +115,13 @@ __device__ __forceinline__ bool locate(float x, int axis, const Geom& g, const f
                                        int& i_out, float& d_out) {
   const int n = g.n;
   const float u0 = (x - g.bmin[axis]) * g.inv_h;
-  const bool finite = isfinite(u0);
-  const float uc = finite ? fminf(fmaxf(u0, -2.f), (float)n + 2.f) : 0.f;
-  int i = (int)floorf(uc);
-  i = max(-1, min(n, i));
+  int i = max(-1, min(n, __float2int_rd(u0)));  // (the conversion saturates; NaN gives 0)
   const float2* nd = nodes + axis * (n + 3) + 1;  // nd[i] for i in [-1, n + 1]
   float2 nv = nd[i];
   float d = ((x - nv.x) - nv.y) * g.inv_h;
-  // One-cell correction of the float guess; a particle within rounding of a node can
-  // land on d = 1.0f (or a hair below 0) after it, so d is clamped into [0, 1):
-  // the stencils are continuous across the node, so either side gives the same mesh.
+  // One-cell correction of the float guess (rarely needed); a particle within rounding
+  // of a node can land on d = 1.0f (or a hair below 0) after it, so d is clamped into
+  // [0, 1): the stencils are continuous across the node, so either side gives the same mesh.
   if (d < 0.f) {
     i = max(i - 1, -1);
     nv = nd[i];
@@ -68,8 +132,9 @@ __device__ __forceinline__ bool locate(float x, int axis, const Geom& g, const f
     d = fmaxf(((x - nv.x) - nv.y) * g.inv_h, 0.f);
   }
   d = fminf(fmaxf(d, 0.f), 0.99999994f);
-  const bool ok = finite && i >= 0 && i < n;
+  const bool ok = (unsigned)i < (unsigned)n && u0 == u0;
   if (!ok) {
+    const bool finite = isfinite(u0);
     const float uw = finite ? u0 - floorf(u0 / (float)n) * (float)n : 0.f;
     int iw = (int)floorf(uw);
     iw = max(0, min(n - 1, iw));
@@ -129,36 +194,73 @@ __device__ __forceinline__ void node_range(int i, float d, int& lo, int& hi) {
 
 __device__ __forceinline__ int wrapn(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
 
-// Tiles touched along one axis (1 or 2 of them).
-__device__ __forceinline__ int axis_tiles(int lo, int hi, int n, int tdim, int (&t)[2]) {
-  t[0] = wrapn(lo, n) / tdim;
-  t[1] = wrapn(hi, n) / tdim;
-  return t[0] == t[1] ? 1 : 2;
+// Tiles a particle's stencils touch, one or two per axis: first, and first plus any sum of
+// dx, dy, dz; inner when the stencils lie inside one tile without periodic wrap.
+struct Touched {
+  int first, dx, dy, dz;  // dx, dy, dz: 0 where the axis has one tile only
+  bool inner, ok;         // ok: the particle is inside the box
+  // f(tile) for every tile but the first
+  template <class F>
+  __device__ __forceinline__ void others(F&& f) const {
+    const int all = (dx ? 1 : 0) | (dy ? 2 : 0) | (dz ? 4 : 0);
+    for (int m = all; m; m = (m - 1) & all)  // the non-empty subsets of the axes with two tiles
+      f(first + ((m & 1) ? dx : 0) + ((m & 2) ? dy : 0) + ((m & 4) ? dz : 0));
+  }
+};
+
+template <int KIND, int M>
+__device__ __forceinline__ Touched touched_tiles(float x, float y, float z, const Geom& g,
+                                                 const float2* __restrict__ nodes) {
+  int ci[3], t0[3], d[3];
+  float cd[3];
+  Touched r;
+  r.ok = locate(x, 0, g, nodes, ci[0], cd[0]);
+  r.ok &= locate(y, 1, g, nodes, ci[1], cd[1]);
+  r.ok &= locate(z, 2, g, nodes, ci[2], cd[2]);
+  r.inner = true;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    int lo, hi;
+    node_range<KIND, M>(ci[a], cd[a], lo, hi);
+    t0[a] = wrapn(lo, g.n) >> g.tshift[a];
+    d[a] = (wrapn(hi, g.n) >> g.tshift[a]) - t0[a];
+    r.inner = r.inner && d[a] == 0 && lo >= 0 && hi < g.n;
+  }
+  r.first = (t0[0] * g.tiles[1] + t0[1]) * g.tiles[2] + t0[2];
+  r.dx = d[0] * g.tiles[1] * g.tiles[2];
+  r.dy = d[1] * g.tiles[2];
+  r.dz = d[2];
+  return r;
 }
 
-// HIST (counting pass only): the tile counts go to a histogram in shared memory
-// (ntiles counters), added to the global counts once per CTA at the end -- a few
-// CTAs per SM and a grid-stride loop, instead of one global atomic per (particle,
-// tile) on counters that every SM contends for.
-template <int KIND, int M, bool HIST = false, int NT = THREADS>
+// Counting pass.  HIST: the tile counts go to a histogram in shared memory (ntiles
+// counters), added to the global counts once per CTA at the end -- a few CTAs per SM and
+// a grid-stride loop, instead of one global atomic per (particle, tile) on counters that
+// every SM contends for.
+template <int KIND, int M, bool HIST, int NT>
 __global__ void __launch_bounds__(NT)
-k_particles(const float* __restrict__ px, const float* __restrict__ py, const float* __restrict__ pz,
-            const float* __restrict__ pw, const float* __restrict__ pnbar, int64_t n, int is_ran,
-            Geom g, const float2* __restrict__ nodes, unsigned* __restrict__ tile_count,
-            double* __restrict__ sums, int ntiles) {
+k_particles(const __grid_constant__ Cats cats, Geom g, const float2* __restrict__ nodes,
+            unsigned* __restrict__ tile_count, double* __restrict__ sums, int ntiles) {
   extern __shared__ unsigned s_hist[];
   if (HIST) {
     for (int t = threadIdx.x; t < ntiles; t += NT) s_hist[t] = 0u;
     __syncthreads();
   }
-  // Compensated float sums per thread (Kahan), FP64 across threads.
-  float s_w = 0.f, c_w = 0.f, s_w2 = 0.f, c_w2 = 0.f, s_w2n = 0.f, c_w2n = 0.f;
+  int bid, nblk;
+  const int is_ran = block_catalogue(cats, bid, nblk);
+  const float* __restrict__ px = cats.x[is_ran];
+  const float* __restrict__ py = cats.y[is_ran];
+  const float* __restrict__ pz = cats.z[is_ran];
+  const float* __restrict__ pw = cats.w[is_ran];
+  const float* __restrict__ pnbar = is_ran ? cats.nbar[1] : nullptr;
+  const int64_t n = cats.n[is_ran];
+  ThreadSums ts;
   unsigned bad = 0;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t stride = (int64_t)nblk * NT;
   // Two particles per iteration (the same order as one per iteration): their loads are issued
   // together, so that the latencies overlap.
   constexpr int U = 2;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; base < n; base += U * stride) {
+  for (int64_t base = (int64_t)bid * NT + threadIdx.x; base < n; base += U * stride) {
     float xs[U], ys[U], zs[U], ws[U], nbs[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -167,42 +269,23 @@ k_particles(const float* __restrict__ px, const float* __restrict__ py, const fl
       ys[u] = py[i];
       zs[u] = pz[i];
       ws[u] = pw ? pw[i] : 1.f;
-      nbs[u] = (is_ran && pnbar) ? pnbar[i] : 0.f;
+      nbs[u] = pnbar ? pnbar[i] : 0.f;
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       if (base + u * stride >= n) break;
       const float x = xs[u], y = ys[u], z = zs[u], w = ws[u];
-      int ci[3];
-      float cd[3];
-      bool ok = locate(x, 0, g, nodes, ci[0], cd[0]);
-      ok &= locate(y, 1, g, nodes, ci[1], cd[1]);
-      ok &= locate(z, 2, g, nodes, ci[2], cd[2]);
-      int tt[3][2], nt[3];
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        int lo, hi;
-        node_range<KIND, M>(ci[a], cd[a], lo, hi);
-        nt[a] = axis_tiles(lo, hi, g.n, g.tdim[a], tt[a]);
-      }
-      bad += ok ? 0u : 1u;
-      {  // Kahan updates
-        float yv = w - c_w, t = s_w + yv;
-        c_w = (t - s_w) - yv; s_w = t;
-        yv = w * w - c_w2; t = s_w2 + yv;
-        c_w2 = (t - s_w2) - yv; s_w2 = t;
-        if (is_ran && pnbar) {
-          yv = w * w * nbs[u] - c_w2n; t = s_w2n + yv;
-          c_w2n = (t - s_w2n) - yv; s_w2n = t;
-        }
-      }
-      for (int a = 0; a < nt[0]; ++a)
-        for (int b = 0; b < nt[1]; ++b)
-          for (int c = 0; c < nt[2]; ++c) {
-            const int tile = (tt[0][a] * g.tiles[1] + tt[1][b]) * g.tiles[2] + tt[2][c];
-            if (HIST) atomicAdd(&s_hist[tile], 1u);
-            else atomicAdd(&tile_count[tile], 1u);
-          }
+      const Touched tt = touched_tiles<KIND, M>(x, y, z, g, nodes);
+      bad += tt.ok ? 0u : 1u;
+      ts.kahan(0, w);
+      ts.kahan(1, w * w);
+      if (pnbar) ts.kahan(2, w * w * nbs[u]);
+      auto count = [&](int tile) {
+        if constexpr (HIST) atomicAdd(&s_hist[tile], 1u);
+        else atomicAdd(&tile_count[tile], 1u);
+      };
+      count(tt.first);
+      if (!tt.inner) tt.others(count);
     }
   }
   if (HIST) {
@@ -210,50 +293,93 @@ k_particles(const float* __restrict__ px, const float* __restrict__ py, const fl
     for (int t = threadIdx.x; t < ntiles; t += NT)
       if (s_hist[t]) atomicAdd(&tile_count[t], s_hist[t]);
   }
-  {
-    __shared__ double red[NT / 32][4];
-    double v0 = warp_sum((double)s_w - (double)c_w);
-    double v1 = warp_sum((double)s_w2 - (double)c_w2);
-    double v2 = warp_sum((double)s_w2n - (double)c_w2n);
-    double v3 = warp_sum((double)bad);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) { red[wid][0] = v0; red[wid][1] = v1; red[wid][2] = v2; red[wid][3] = v3; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double t0 = 0, t1 = 0, t2 = 0, t3 = 0;
-      for (int k = 0; k < NT / 32; ++k) { t0 += red[k][0]; t1 += red[k][1]; t2 += red[k][2]; t3 += red[k][3]; }
-      if (is_ran) {
-        atomicAdd(&sums[SUM_WR], t0);
-        atomicAdd(&sums[SUM_WR2], t1);
-        atomicAdd(&sums[SUM_WR2N], t2);
-      } else {
-        atomicAdd(&sums[SUM_WG], t0);
-        atomicAdd(&sums[SUM_WG2], t1);
-      }
-      if (t3 != 0.0) atomicAdd(&sums[SUM_BAD], t3);
-    }
-  }
+  block_sums<NT>(ts, bad, is_ran, sums);
+}
+
+// Signed weight factor of a catalogue: 1 for galaxies, -alpha for randoms.
+__device__ __forceinline__ float catalogue_scale(int is_ran, double alpha_cfg, const double* __restrict__ sums) {
+  return is_ran ? (float)(-(alpha_cfg >= 0.0 ? alpha_cfg : sums[SUM_WG] / sums[SUM_WR])) : 1.f;
 }
 
 // Binning pass: one 16-byte record (position, signed weight) per tile a particle's
 // stencils touch; records whose stencils lie inside one tile (no periodic wrap) fill
-// the tile's list from the front (tile_cur), the others from the back (tile_back, the
-// end of each list after the scan).  Each thread takes U particles per iteration, whose
-// loads and first-tile cursor atomics are independent, so that their latencies
-// overlap (one particle per iteration leaves the pass waiting on each memory round trip).
+// the tile's list from the front (cursor tile_cur), the others from the back (the
+// tile's remaining count tile_left, from off[tile]).
+//
+// Few tiles (k_bin_agg, up to BIN_AGG_TILES): a CTA counts the records of a chunk of
+// particles per tile in shared memory, reserves each tile's range with one global
+// atomic, and hands out the slots from shared-memory cursors.  One global atomic per
+// record serialises on the tiles' cursors when there are few of them: 6.6e6 particles
+// on the 512 tiles of a 128^3 mesh took 790 us.
+// Many tiles (k_bin): a chunk would hold about one record per tile, so each record takes
+// its own global atomic; each thread takes U particles per iteration, whose loads and
+// first-tile cursor atomics are independent, so that their latencies overlap.
+constexpr int BIN_AGG_TILES = 4096;
+constexpr int BIN_AGG_NT = 512;
+
+template <int KIND, int M>
+__global__ void __launch_bounds__(BIN_AGG_NT)
+k_bin_agg(const __grid_constant__ Cats cats, int per_thread, Geom g, const float2* __restrict__ nodes, int ntiles,
+          const unsigned* __restrict__ off, unsigned* __restrict__ tile_left, unsigned* __restrict__ tile_cur,
+          float4* __restrict__ rec, const double* __restrict__ sums, double alpha_cfg) {
+  extern __shared__ unsigned s_cur[];  // [2][ntiles]: interior, border
+  for (int t = threadIdx.x; t < 2 * ntiles; t += BIN_AGG_NT) s_cur[t] = 0u;
+  int bid, nblk;
+  const int is_ran = block_catalogue(cats, bid, nblk);
+  const float* __restrict__ px = cats.x[is_ran];
+  const float* __restrict__ py = cats.y[is_ran];
+  const float* __restrict__ pz = cats.z[is_ran];
+  const float* __restrict__ pw = cats.w[is_ran];
+  const int64_t first = (int64_t)bid * BIN_AGG_NT * per_thread;
+  px += first;
+  py += first;
+  pz += first;
+  if (pw) pw += first;
+  const int last = (int)min(cats.n[is_ran] - first, (int64_t)BIN_AGG_NT * per_thread);
+  __syncthreads();
+#pragma unroll 2
+  for (int i = threadIdx.x; i < last; i += BIN_AGG_NT) {
+    const Touched tt = touched_tiles<KIND, M>(px[i], py[i], pz[i], g, nodes);
+    unsigned* cnt = s_cur + (tt.inner ? 0 : ntiles);
+    atomicAdd(cnt + tt.first, 1u);
+    if (!tt.inner) tt.others([&](int tile) { atomicAdd(cnt + tile, 1u); });
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < ntiles; t += BIN_AGG_NT) {
+    const unsigned f = s_cur[t], b = s_cur[ntiles + t];
+    if (f) s_cur[t] = atomicAdd(&tile_cur[t], f);
+    if (b) s_cur[ntiles + t] = off[t] + atomicSub(&tile_left[t], b) - b;
+  }
+  __syncthreads();
+  const float wscale = catalogue_scale(is_ran, alpha_cfg, sums);
+#pragma unroll 2
+  for (int i = threadIdx.x; i < last; i += BIN_AGG_NT) {
+    const float4 q = make_float4(px[i], py[i], pz[i], (pw ? pw[i] : 1.f) * wscale);
+    const Touched tt = touched_tiles<KIND, M>(q.x, q.y, q.z, g, nodes);
+    unsigned* cur = s_cur + (tt.inner ? 0 : ntiles);
+    rec[atomicAdd(cur + tt.first, 1u)] = q;
+    if (!tt.inner) tt.others([&](int tile) { rec[atomicAdd(cur + tile, 1u)] = q; });
+  }
+}
+
 template <int KIND, int M, int U>
 __global__ void __launch_bounds__(THREADS)
-k_bin(const float* __restrict__ px, const float* __restrict__ py, const float* __restrict__ pz,
-      const float* __restrict__ pw, int64_t n, int is_ran, Geom g, const float2* __restrict__ nodes,
-      unsigned* __restrict__ tile_back, unsigned* __restrict__ tile_cur, float4* __restrict__ rec,
+k_bin(const __grid_constant__ Cats cats, Geom g, const float2* __restrict__ nodes, const unsigned* __restrict__ off,
+      unsigned* __restrict__ tile_left, unsigned* __restrict__ tile_cur, float4* __restrict__ rec,
       const double* __restrict__ sums, double alpha_cfg) {
-  float wscale = 1.f;
-  if (is_ran) wscale = (float)(-(alpha_cfg >= 0.0 ? alpha_cfg : sums[SUM_WG] / sums[SUM_WR]));
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; base < n; base += U * stride) {
+  int bid, nblk;
+  const int is_ran = block_catalogue(cats, bid, nblk);
+  const float* __restrict__ px = cats.x[is_ran];
+  const float* __restrict__ py = cats.y[is_ran];
+  const float* __restrict__ pz = cats.z[is_ran];
+  const float* __restrict__ pw = cats.w[is_ran];
+  const int64_t n = cats.n[is_ran];
+  const float wscale = catalogue_scale(is_ran, alpha_cfg, sums);
+  const int64_t stride = (int64_t)nblk * blockDim.x;
+  for (int64_t base = (int64_t)bid * blockDim.x + threadIdx.x; base < n; base += U * stride) {
     float4 q[U];
-    int tt[U][3][2], nt[U][3];
-    bool inner[U], valid[U];
+    Touched tt[U];
+    bool valid[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int64_t idx = base + u * stride;
@@ -262,71 +388,79 @@ k_bin(const float* __restrict__ px, const float* __restrict__ py, const float* _
       q[u] = make_float4(px[i], py[i], pz[i], (pw ? pw[i] : 1.f) * wscale);
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      int ci[3];
-      float cd[3];
-      locate(q[u].x, 0, g, nodes, ci[0], cd[0]);
-      locate(q[u].y, 1, g, nodes, ci[1], cd[1]);
-      locate(q[u].z, 2, g, nodes, ci[2], cd[2]);
-      inner[u] = true;
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        int lo, hi;
-        node_range<KIND, M>(ci[a], cd[a], lo, hi);
-        nt[u][a] = axis_tiles(lo, hi, g.n, g.tdim[a], tt[u][a]);
-        inner[u] = inner[u] && nt[u][a] == 1 && lo >= 0 && hi < g.n;
-      }
-    }
+    for (int u = 0; u < U; ++u) tt[u] = touched_tiles<KIND, M>(q[u].x, q[u].y, q[u].z, g, nodes);
     unsigned slot[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       if (!valid[u]) continue;
-      const int tile = (tt[u][0][0] * g.tiles[1] + tt[u][1][0]) * g.tiles[2] + tt[u][2][0];
-      slot[u] = inner[u] ? atomicAdd(&tile_cur[tile], 1u) : atomicSub(&tile_back[tile], 1u) - 1u;
+      const int tile = tt[u].first;
+      slot[u] = tt[u].inner ? atomicAdd(&tile_cur[tile], 1u) : off[tile] + atomicSub(&tile_left[tile], 1u) - 1u;
     }
 #pragma unroll
     for (int u = 0; u < U; ++u)
       if (valid[u]) rec[slot[u]] = q[u];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      if (!valid[u] || inner[u]) continue;
-      for (int a = 0; a < nt[u][0]; ++a)
-        for (int b = 0; b < nt[u][1]; ++b)
-          for (int c = 0; c < nt[u][2]; ++c) {
-            if (a == 0 && b == 0 && c == 0) continue;  // the first tile is done
-            const int tile = (tt[u][0][a] * g.tiles[1] + tt[u][1][b]) * g.tiles[2] + tt[u][2][c];
-            rec[atomicSub(&tile_back[tile], 1u) - 1u] = q[u];
-          }
+      if (!valid[u] || tt[u].inner) continue;
+      tt[u].others([&](int tile) { rec[off[tile] + atomicSub(&tile_left[tile], 1u) - 1u] = q[u]; });
     }
   }
 }
 
-// Exclusive scan of the tile counts (single CTA of 1024 threads); the counts are
-// replaced by the end of each tile's list, the binning pass's back cursors.
+// Exclusive scan of the tile counts into off and the front cursors cur, one CTA per 1024
+// tiles.  Each CTA sums all counts before its own (at most 1 MB, from L2) instead of
+// waiting for the CTAs before it: 32768 tiles 102 -> 6 us, 262144 tiles 785 -> 16 us
+// against one CTA for all.
 __global__ void __launch_bounds__(1024)
-k_scan(unsigned* __restrict__ count, int ntiles, unsigned* __restrict__ off, unsigned* __restrict__ cur) {
-  __shared__ unsigned part[1024];
-  const int t = threadIdx.x;
-  const int per = (ntiles + 1023) / 1024;
-  const int b = t * per, e = min(ntiles, b + per);
-  unsigned s = 0;
-  for (int i = b; i < e; ++i) s += count[i];
-  part[t] = s;
+k_scan(const unsigned* __restrict__ count, int ntiles, unsigned* __restrict__ off, unsigned* __restrict__ cur) {
+  __shared__ unsigned part[33];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const uint4* c4 = reinterpret_cast<const uint4*>(count);
+  unsigned before = 0;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < (int)blockIdx.x * 256; i += 1024) {
+    const uint4 v = c4[i];
+    before += v.x + v.y + v.z + v.w;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+  if (lane == 0) part[wid] = before;
   __syncthreads();
-  for (int o = 1; o < 1024; o <<= 1) {  // Hillis-Steele inclusive scan
-    const unsigned v = t >= o ? part[t - o] : 0u;
-    __syncthreads();
-    part[t] += v;
-    __syncthreads();
+  if (wid == 0) {
+    unsigned v = part[lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) part[32] = v;
   }
-  unsigned run = t > 0 ? part[t - 1] : 0u;
-  for (int i = b; i < e; ++i) {
-    off[i] = run;
-    cur[i] = run;
-    run += count[i];
-    count[i] = run;  // from here on the back cursor of tile i
+  __syncthreads();
+  const unsigned base = part[32];
+  __syncthreads();
+  const int i = blockIdx.x * 1024 + threadIdx.x;
+  const unsigned c = i < ntiles ? count[i] : 0u;
+  unsigned incl = c;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
   }
-  if (t == 1023) off[ntiles] = part[1023];
+  if (lane == 31) part[wid] = incl;
+  __syncthreads();
+  if (wid == 0) {
+    unsigned v = part[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned u = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += u;
+    }
+    part[lane] = v;
+  }
+  __syncthreads();
+  const unsigned excl = base + (wid > 0 ? part[wid - 1] : 0u) + incl - c;
+  if (i < ntiles) {
+    off[i] = excl;
+    cur[i] = excl;
+    if (i == ntiles - 1) off[ntiles] = excl + c;
+  }
 }
 
 // Stencil walk of one record: add(k, wxy, wz) for every node of the record's stencil,
@@ -432,17 +566,27 @@ __device__ __forceinline__ void deposit_inner(const float4& q, float wq, const G
 //
 // rmesh (shared randoms): the kept random mesh sum_ran w W, written as
 // F = (galaxy deposit) - alpha rmesh, with alpha from the catalogue sums.
-template <int KIND, int M, bool FIXED>
+//
+// MULTI: a cluster of CTAs shares one tile (deposit_cluster gives its size), where there
+// are too few tiles to fill the GPU: each CTA deposits its share of the records into its
+// own copy, and each sums its share of the nodes over the cluster's copies (integers:
+// the same bits whatever the split) before storing them.
+template <int KIND, int M, bool FIXED, bool MULTI>
 __global__ void __launch_bounds__(THREADS, 3)
 k_deposit(Geom g, const float2* __restrict__ nodes, const unsigned* __restrict__ off,
           const unsigned* __restrict__ split, const float4* __restrict__ rec, float* __restrict__ mesh,
           const float* __restrict__ rmesh, const double* __restrict__ sums, double alpha_cfg) {
   extern __shared__ float s_tile[];
   __shared__ float s_wmax[THREADS / 32];
+  __shared__ float s_part;  // this CTA's largest |w|, NaN if a weight is not finite
+  namespace cg = cooperative_groups;
+  [[maybe_unused]] cg::cluster_group cluster = cg::this_cluster();
+  const unsigned cl = MULTI ? cluster.num_blocks() : 1u, rank = MULTI ? cluster.block_rank() : 0u;
   const int n = g.n;
   const int tdx = g.tdim[0], tdy = g.tdim[1], tdz = g.tdim[2];
   const int tvol = tdx * tdy * tdz;
-  const int tile = blockIdx.x;
+  const int tile = blockIdx.x / cl;
+  const unsigned tid = rank * THREADS + threadIdx.x, step = cl * THREADS;  // over the tile's records
   const int tz = tile % g.tiles[2];
   const int ty = (tile / g.tiles[2]) % g.tiles[1];
   const int tx = tile / (g.tiles[2] * g.tiles[1]);
@@ -461,7 +605,7 @@ k_deposit(Geom g, const float2* __restrict__ nodes, const unsigned* __restrict__
     const float* wrec = reinterpret_cast<const float*>(rec) + 3;
     float wm = 0.f;
     bool bad = false;
-    for (unsigned r = b + threadIdx.x; r < e; r += blockDim.x) {
+    for (unsigned r = b + tid; r < e; r += step) {
       const float w = wrec[(size_t)r * 4];
       bad |= !isfinite(w);
       wm = fmaxf(wm, fabsf(w));
@@ -472,6 +616,15 @@ k_deposit(Geom g, const float2* __restrict__ nodes, const unsigned* __restrict__
     bad = __syncthreads_or(bad);  // also orders s_wmax and the zero fill
 #pragma unroll
     for (int k = 0; k < THREADS / 32; ++k) wm = fmaxf(wm, s_wmax[k]);
+    if constexpr (MULTI) {  // over the cluster
+      if (threadIdx.x == 0) s_part = bad ? __int_as_float(0x7fc00000) : wm;
+      cluster.sync();
+      for (unsigned q = 0; q < cl; ++q) {
+        const float v = *cluster.map_shared_rank(&s_part, q);
+        bad |= isnan(v);
+        wm = fmaxf(wm, v);
+      }
+    }
     fixed = !bad && nrec < (1u << 30);
     if (fixed && nrec > 0) {
       const float ln = log2f((float)nrec), lw = log2f(wm);
@@ -497,26 +650,27 @@ k_deposit(Geom g, const float2* __restrict__ nodes, const unsigned* __restrict__
       atomicAdd(s_hi + k, __float_as_int(t) - kbits);
       atomicAdd(s_lo + k, __float_as_int(__fadd_rn(lf, 12582912.f)) - 0x4B400000);  // + 1.5 2^23
     };
-    for (unsigned r = b + threadIdx.x; r < mid; r += blockDim.x) {
+    for (unsigned r = b + tid; r < mid; r += step) {
       const float4 q = rec[r];
       deposit_inner<KIND, M>(q, q.w * scale, g, nodes, o, td, tvol, add);
     }
-    for (unsigned r = mid + threadIdx.x; r < e; r += blockDim.x) {
+    for (unsigned r = mid + tid; r < e; r += step) {
       const float4 q = rec[r];
       deposit_record<KIND, M>(q, q.w * scale, g, nodes, o, td, tvol, trash, add);
     }
   } else {
     auto add = [&](int k, float wxy, float wz) { atomicAdd(s_tile + k, wxy * wz); };
-    for (unsigned r = b + threadIdx.x; r < mid; r += blockDim.x) {
+    for (unsigned r = b + tid; r < mid; r += step) {
       const float4 q = rec[r];
       deposit_inner<KIND, M>(q, q.w, g, nodes, o, td, tvol, add);
     }
-    for (unsigned r = mid + threadIdx.x; r < e; r += blockDim.x) {
+    for (unsigned r = mid + tid; r < e; r += step) {
       const float4 q = rec[r];
       deposit_record<KIND, M>(q, q.w, g, nodes, o, td, tvol, trash, add);
     }
   }
-  __syncthreads();
+  if constexpr (MULTI) cluster.sync();
+  else __syncthreads();
   const size_t n3 = (size_t)n * n * n;
   const float ran_scale =
       rmesh ? (float)(-(alpha_cfg >= 0.0 ? alpha_cfg : sums[SUM_WG] / sums[SUM_WR])) : 0.f;
@@ -524,43 +678,73 @@ k_deposit(Geom g, const float2* __restrict__ nodes, const unsigned* __restrict__
   // fma once more (within one ulp of the exact sum, and the same bits on every run)
   const float unscale = __int_as_float((127 - sc) << 23);       // 2^-s
   const float hscale = __int_as_float((127 + sb - sc) << 23);   // 2^(sb-s)
-  const int* s_hi = reinterpret_cast<const int*>(s_tile);
-  // tile sides are powers of two (8, 16 or 32 for every supported mesh)
-  const int shz = __ffs(tdz) - 1, shy = __ffs(tdy) - 1, shv = shz + shy + __ffs(tdx) - 1;
-  for (int k = threadIdx.x; k < M * tvol; k += blockDim.x) {
+  int* s_hi = reinterpret_cast<int*>(s_tile);
+  const int shz = g.tshift[2], shy = g.tshift[1], shv = shz + shy + g.tshift[0];
+  for (int k = tid; k < M * tvol; k += step) {
     const int mj = k >> shv;
     const int lz = k & (tdz - 1);
     const int ly = (k >> shz) & (tdy - 1);
     const int lx = (k >> (shz + shy)) & (tdx - 1);
     const size_t at = mj * n3 + ((size_t)(o[0] + lx) * n + (o[1] + ly)) * n + (o[2] + lz);
-    const float v = fixed ? __fmaf_rn(__int2float_rn(s_hi[k]), hscale, __int2float_rn(s_hi[words + k]) * unscale)
-                          : s_tile[k];
+    float v;
+    if constexpr (MULTI) {
+      if (fixed) {
+        int hi = 0, lo = 0;
+        for (unsigned q = 0; q < cl; ++q) {
+          const int* part = cluster.map_shared_rank(s_hi, q);
+          hi += part[k];
+          lo += part[words + k];
+        }
+        v = __fmaf_rn(__int2float_rn(hi), hscale, __int2float_rn(lo) * unscale);
+      } else {
+        v = 0.f;
+        for (unsigned q = 0; q < cl; ++q) v += cluster.map_shared_rank(s_tile, q)[k];
+      }
+    } else {
+      v = fixed ? __fmaf_rn(__int2float_rn(s_hi[k]), hscale, __int2float_rn(s_hi[words + k]) * unscale) : s_tile[k];
+    }
     mesh[at] = rmesh ? fmaf(ran_scale, rmesh[at], v) : v;
   }
+  if constexpr (MULTI) cluster.sync();  // every copy stays until the last CTA has read it
 }
 
 // FP64 sums of a random catalogue (sum w, sum w^2, sum w^2 nbar) for the kept copy.
 __global__ void k_ran_sums(const float* __restrict__ w, const float* __restrict__ nbar, int64_t n,
                            double* __restrict__ out) {
-  double s1 = 0.0, s2 = 0.0, s3 = 0.0;
+  double s[3] = {0.0, 0.0, 0.0};
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const double v = w ? (double)w[i] : 1.0;
-    s1 += v;
-    s2 += v * v;
-    if (nbar) s3 += v * v * (double)nbar[i];
+    s[0] += v;
+    s[1] += v * v;
+    if (nbar) s[2] += v * v * (double)nbar[i];
   }
-  s1 = warp_sum(s1);
-  s2 = warp_sum(s2);
-  s3 = warp_sum(s3);
-  if ((threadIdx.x & 31) == 0) {
-    atomicAdd(&out[0], s1);
-    atomicAdd(&out[1], s2);
-    atomicAdd(&out[2], s3);
+  for (int k = 0; k < 3; ++k) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&out[k], s[k]);
   }
 }
 
-// rmesh != nullptr (shared randoms): ran is empty, the random sums come from rsums
-// (sum w, sum w^2, sum w^2 nbar) and the deposit subtracts alpha rmesh.
+// Catalogue sums of Eqs. (1) and (3) without the counting pass.
+__global__ void __launch_bounds__(THREADS)
+k_sums(const __grid_constant__ Cats cats, double* __restrict__ sums) {
+  int bid, nblk;
+  const int is_ran = block_catalogue(cats, bid, nblk);
+  const float* __restrict__ pw = cats.w[is_ran];
+  const float* __restrict__ pnbar = is_ran ? cats.nbar[1] : nullptr;
+  const int64_t n = cats.n[is_ran];
+  ThreadSums ts;
+  const int64_t stride = (int64_t)nblk * THREADS;
+#pragma unroll 4
+  for (int64_t i = (int64_t)bid * THREADS + threadIdx.x; i < n; i += stride) {
+    const float w = pw ? pw[i] : 1.f;
+    ts.kahan(0, w);
+    ts.kahan(1, w * w);
+    if (pnbar) ts.kahan(2, w * w * pnbar[i]);
+  }
+  block_sums<THREADS>(ts, 0u, is_ran, sums);
+}
+
 // ---------------------------------------------------------------------------
 // Direct assignment for meshes that stay resident in L2 (m N^3 floats of at most
 // 64 MB, half of it): one pass over each catalogue adds every stencil weight
@@ -569,51 +753,23 @@ __global__ void k_ran_sums(const float* __restrict__ w, const float* __restrict_
 // (4-12 bytes, then 16) instead of the sort's count, bin and deposit passes.
 // ---------------------------------------------------------------------------
 
-// Catalogue sums of Eqs. (1) and (3): Kahan-compensated float per thread, FP64
-// across threads (the same slots as the sorted path's counting pass).
-__global__ void __launch_bounds__(THREADS)
-k_sums(const float* __restrict__ pw, const float* __restrict__ pnbar, int64_t n, int is_ran,
-       double* __restrict__ sums) {
-  float s_w = 0.f, c_w = 0.f, s_w2 = 0.f, c_w2 = 0.f, s_w2n = 0.f, c_w2n = 0.f;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += stride) {
-    const float w = pw ? pw[idx] : 1.f;
-    float yv = w - c_w, t = s_w + yv;
-    c_w = (t - s_w) - yv; s_w = t;
-    yv = w * w - c_w2; t = s_w2 + yv;
-    c_w2 = (t - s_w2) - yv; s_w2 = t;
-    if (is_ran && pnbar) {
-      yv = w * w * pnbar[idx] - c_w2n; t = s_w2n + yv;
-      c_w2n = (t - s_w2n) - yv; s_w2n = t;
-    }
-  }
-  const double v0 = warp_sum((double)s_w - (double)c_w);
-  const double v1 = warp_sum((double)s_w2 - (double)c_w2);
-  const double v2 = warp_sum((double)s_w2n - (double)c_w2n);
-  if ((threadIdx.x & 31) == 0) {
-    if (is_ran) {
-      atomicAdd(&sums[SUM_WR], v0);
-      atomicAdd(&sums[SUM_WR2], v1);
-      atomicAdd(&sums[SUM_WR2N], v2);
-    } else {
-      atomicAdd(&sums[SUM_WG], v0);
-      atomicAdd(&sums[SUM_WG2], v1);
-    }
-  }
-}
-
 template <int KIND, int M>
 __global__ void __launch_bounds__(THREADS)
-k_direct(const float* __restrict__ px, const float* __restrict__ py, const float* __restrict__ pz,
-         const float* __restrict__ pw, int64_t n, int is_ran, Geom g, const float2* __restrict__ nodes,
-         double* __restrict__ sums, double alpha_cfg, float* __restrict__ mesh) {
-  float wscale = 1.f;
-  if (is_ran) wscale = (float)(-(alpha_cfg >= 0.0 ? alpha_cfg : sums[SUM_WG] / sums[SUM_WR]));
+k_direct(const __grid_constant__ Cats cats, Geom g, const float2* __restrict__ nodes, double* __restrict__ sums,
+         double alpha_cfg, float* __restrict__ mesh) {
+  int bid, nblk;
+  const int is_ran = block_catalogue(cats, bid, nblk);
+  const float* __restrict__ px = cats.x[is_ran];
+  const float* __restrict__ py = cats.y[is_ran];
+  const float* __restrict__ pz = cats.z[is_ran];
+  const float* __restrict__ pw = cats.w[is_ran];
+  const int64_t n = cats.n[is_ran];
+  const float wscale = catalogue_scale(is_ran, alpha_cfg, sums);
   const int nn = g.n;
   const size_t n3 = (size_t)nn * nn * nn;
   unsigned bad = 0;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += stride) {
+  const int64_t stride = (int64_t)nblk * blockDim.x;
+  for (int64_t idx = (int64_t)bid * blockDim.x + threadIdx.x; idx < n; idx += stride) {
     const float x = px[idx], y = py[idx], z = pz[idx];
     const float w = (pw ? pw[idx] : 1.f) * wscale;
     int ci[3];
@@ -651,6 +807,34 @@ k_direct(const float* __restrict__ px, const float* __restrict__ py, const float
   if ((threadIdx.x & 31) == 0 && tot) atomicAdd(&sums[SUM_BAD], (double)tot);
 }
 
+// The two catalogues of a launch of `grid` blocks, shared out by their particle counts
+// (at least one block each).
+Cats make_cats(const ys_catalog& gal, const ys_catalog& ran, int& grid) {
+  Cats c{};
+  const ys_catalog* k[2] = {&gal, &ran};
+  for (int i = 0; i < 2; ++i) {
+    c.x[i] = k[i]->x;
+    c.y[i] = k[i]->y;
+    c.z[i] = k[i]->z;
+    c.w[i] = k[i]->w;
+    c.nbar[i] = k[i]->nbar;
+    c.n[i] = k[i]->n;
+  }
+  const double total = (double)gal.n + (double)ran.n;
+  if (gal.n > 0 && ran.n > 0) {
+    grid = std::max(grid, 2);
+    c.blocks0 = std::min(grid - 1, std::max(1, (int)(grid * (gal.n / total) + 0.5)));
+  } else {
+    grid = std::max(grid, 1);
+    c.blocks0 = gal.n > 0 ? grid : 0;
+  }
+  return c;
+}
+
+int blocks_for(int64_t n, int per_block, int most) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>((n + per_block - 1) / per_block, most));
+}
+
 template <int KIND, int M>
 cudaError_t run_direct(Plan& p, const ys_catalog& gal, const ys_catalog& ran) {
   cudaStream_t st = p.stream;
@@ -661,28 +845,54 @@ cudaError_t run_direct(Plan& p, const ys_catalog& gal, const ys_catalog& ran) {
   int dev = 0, sms = 0;
   if ((err = cudaGetDevice(&dev)) || (err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)))
     return err;
-  auto blocks = [&](int64_t n) {
-    return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + THREADS - 1) / THREADS, (int64_t)sms * 8));
-  };
-  const ys_catalog* cats[2] = {&gal, &ran};
-  for (int c = 0; c < 2; ++c) {
-    const ys_catalog& k = *cats[c];
-    if (k.n == 0) continue;
+  const int64_t total = gal.n + ran.n;
+  if (total == 0) return cudaSuccess;
+  {
+    int grid = blocks_for(total, 4 * THREADS, sms * 8);
+    const Cats cats = make_cats(gal, ran, grid);
     LaunchScope ls(p, 0);
-    k_sums<<<blocks(k.n), THREADS, 0, st>>>(k.w, k.nbar, k.n, c, p.d_sums);
+    k_sums<<<grid, THREADS, 0, st>>>(cats, p.d_sums);
     if ((err = cudaGetLastError())) return err;
   }
-  for (int c = 0; c < 2; ++c) {
-    const ys_catalog& k = *cats[c];
-    if (k.n == 0) continue;
-    LaunchScope ls(p, 3);
-    k_direct<KIND, M><<<blocks(k.n), THREADS, 0, st>>>(k.x, k.y, k.z, k.w, k.n, c, p.geom, p.d_nodes, p.d_sums,
-                                                       p.cfg.alpha, p.d_mesh);
-    if ((err = cudaGetLastError())) return err;
-  }
-  return cudaSuccess;
+  int grid = blocks_for(total, THREADS, sms * 8);
+  const Cats cats = make_cats(gal, ran, grid);
+  LaunchScope ls(p, 3);
+  k_direct<KIND, M><<<grid, THREADS, 0, st>>>(cats, p.geom, p.d_nodes, p.d_sums, p.cfg.alpha, p.d_mesh);
+  return cudaGetLastError();
 }
 
+// The counting pass with NT threads per CTA.
+template <int KIND, int M, int NT>
+cudaError_t run_count(Plan& p, const ys_catalog& gal, const ys_catalog& ran, int sms) {
+  cudaError_t err;
+  const int64_t total = gal.n + ran.n;
+  // shared-memory histograms while the tile counters fit (a few CTAs per SM)
+  const size_t hist_bytes = sizeof(unsigned) * (size_t)p.ntiles;
+  const bool hist = hist_bytes <= 160u * 1024u;
+  auto kern = hist ? k_particles<KIND, M, true, NT> : k_particles<KIND, M, false, NT>;
+  const size_t smem = hist ? hist_bytes : 0;
+  int per = 0;
+  if (hist && (err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return err;
+  if ((err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, NT, smem))) return err;
+  int grid = blocks_for(total, NT, std::max(1, per) * sms);
+  const Cats cats = make_cats(gal, ran, grid);
+  LaunchScope ls(p, 0);
+  kern<<<grid, NT, smem, p.stream>>>(cats, p.geom, p.d_nodes, p.d_tile_count, p.d_sums, p.ntiles);
+  return cudaGetLastError();
+}
+
+// CTAs per tile of the deposit: doubled (up to 8) while there are fewer than five per SM
+// and a CTA would still get 256 records.  6.6e6 particles, CIC: 512 tiles (128^3) 198 us
+// with one CTA each (1.1 waves of three per SM) and 157 us with four; 1728 tiles (192^3)
+// 142 us with one and 182 us with two, so the line lies between.
+int deposit_cluster(int ntiles, int64_t particles, int sms) {
+  int cl = 1;
+  while (cl < 8 && (int64_t)ntiles * cl < 5 * sms && particles / ((int64_t)ntiles * 2 * cl) >= 256) cl *= 2;
+  return cl;
+}
+
+// rmesh != nullptr (shared randoms): ran is empty, the random sums come from rsums
+// (sum w, sum w^2, sum w^2 nbar) and the deposit subtracts alpha rmesh.
 template <int KIND, int M>
 cudaError_t run_assign(Plan& p, const ys_catalog& gal, const ys_catalog& ran, const float* rmesh = nullptr,
                        const double* rsums = nullptr) {
@@ -692,70 +902,74 @@ cudaError_t run_assign(Plan& p, const ys_catalog& gal, const ys_catalog& ran, co
   if ((err = cudaMemsetAsync(p.d_sums, 0, sizeof(double) * SUM_COUNT, st)) != cudaSuccess) return err;
   if (rsums && (err = cudaMemcpyAsync(p.d_sums + SUM_WR, rsums, sizeof(double) * 3, cudaMemcpyDeviceToDevice, st)))
     return err;
-  auto blocks = [](int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + THREADS - 1) / THREADS, 152 * 16)); };
-  const ys_catalog* cats[2] = {&gal, &ran};
-  // counting: shared-memory histograms while the tile counters fit (a few CTAs per SM)
-  constexpr int HT = 1024;
-  const size_t hist_bytes = sizeof(unsigned) * (size_t)p.ntiles;
-  const bool hist = hist_bytes <= 160u * 1024u;
-  int hist_grid = 0;
-  if (hist) {
-    int dev = 0, sms = 0, per = 0;
-    if ((err = cudaGetDevice(&dev)) || (err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)))
-      return err;
-    if ((err = cudaFuncSetAttribute(k_particles<KIND, M, true, HT>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hist_bytes)))
-      return err;
-    if ((err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_particles<KIND, M, true, HT>, HT,
-                                                             hist_bytes)))
-      return err;
-    hist_grid = std::max(1, per) * sms;
-  }
-  for (int c = 0; c < 2; ++c) {
-    const ys_catalog& k = *cats[c];
-    if (k.n == 0) continue;
-    LaunchScope ls(p, 0);
-    if (hist) {
-      const int grid = (int)std::min<int64_t>(hist_grid, (k.n + HT - 1) / HT);
-      k_particles<KIND, M, true, HT><<<grid, HT, hist_bytes, st>>>(k.x, k.y, k.z, k.w, k.nbar, k.n, c, p.geom,
-                                                                  p.d_nodes, p.d_tile_count, p.d_sums, p.ntiles);
-    } else {
-      k_particles<KIND, M, false><<<blocks(k.n), THREADS, 0, st>>>(k.x, k.y, k.z, k.w, k.nbar, k.n, c, p.geom,
-                                                                   p.d_nodes, p.d_tile_count, p.d_sums, p.ntiles);
-    }
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
-  }
+  int dev = 0, sms = 0;
+  if ((err = cudaGetDevice(&dev)) || (err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)))
+    return err;
+  const int64_t total = gal.n + ran.n;
+  // CTAs of 1024 threads share one histogram; a catalogue that would leave most of them
+  // idle takes CTAs of 256 (shorter sums at their end)
+  if (total > 0 && (err = total >= (int64_t)sms * 1024 ? run_count<KIND, M, 1024>(p, gal, ran, sms)
+                                                       : run_count<KIND, M, 256>(p, gal, ran, sms)))
+    return err;
   {
     LaunchScope ls(p, 1);
-    k_scan<<<1, 1024, 0, st>>>(p.d_tile_count, p.ntiles, p.d_tile_off, p.d_tile_cur);
+    k_scan<<<(p.ntiles + 1023) / 1024, 1024, 0, st>>>(p.d_tile_count, p.ntiles, p.d_tile_off, p.d_tile_cur);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
   }
-  for (int c = 0; c < 2; ++c) {
-    const ys_catalog& k = *cats[c];
-    if (k.n == 0) continue;
+  if (total > 0 && p.ntiles <= BIN_AGG_TILES) {
+    // chunks of up to 16 particles per thread, in whole waves of three CTAs per SM
+    const int64_t wave = (int64_t)BIN_AGG_NT * sms * 3, waves = (total + 16 * wave - 1) / (16 * wave);
+    const int per_thread = (int)((total + wave * waves - 1) / (wave * waves));
+    const int chunk = BIN_AGG_NT * per_thread;
+    int grid = 1;
+    Cats cats = make_cats(gal, ran, grid);
+    cats.blocks0 = (int)((gal.n + chunk - 1) / chunk);
+    grid = cats.blocks0 + (int)((ran.n + chunk - 1) / chunk);
+    const size_t smem = 2 * sizeof(unsigned) * (size_t)p.ntiles;
     LaunchScope ls(p, 2);
+    k_bin_agg<KIND, M><<<grid, BIN_AGG_NT, smem, st>>>(cats, per_thread, p.geom, p.d_nodes, p.ntiles, p.d_tile_off,
+                                                       p.d_tile_count, p.d_tile_cur, p.d_rec, p.d_sums, p.cfg.alpha);
+    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  } else if (total > 0) {
     constexpr int U = 2;
-    k_bin<KIND, M, U><<<blocks((k.n + U - 1) / U), THREADS, 0, st>>>(
-        k.x, k.y, k.z, k.w, k.n, c, p.geom, p.d_nodes, p.d_tile_count, p.d_tile_cur, p.d_rec, p.d_sums, p.cfg.alpha);
+    int grid = blocks_for(total, U * THREADS, sms * 16);
+    const Cats cats = make_cats(gal, ran, grid);
+    LaunchScope ls(p, 2);
+    k_bin<KIND, M, U><<<grid, THREADS, 0, st>>>(cats, p.geom, p.d_nodes, p.d_tile_off, p.d_tile_count, p.d_tile_cur,
+                                                p.d_rec, p.d_sums, p.cfg.alpha);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
   }
   const int tvol = p.geom.tdim[0] * p.geom.tdim[1] * p.geom.tdim[2];
-  int dev = 0, optin = 0;
-  if ((err = cudaGetDevice(&dev)) ||
-      (err = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)))
-    return err;
+  int optin = 0;
+  if ((err = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev))) return err;
   // fixed-point sums need two words per node; a tile that cannot hold them sums in float
   const size_t words = (size_t)M * tvol + 32;  // nodes and one trash word per lane
   const size_t smem_fixed = 2 * sizeof(float) * words;
   const bool fixed = smem_fixed + 64 <= (size_t)optin;
   const size_t smem = fixed ? smem_fixed : sizeof(float) * words;
-  auto kern = fixed ? k_deposit<KIND, M, true> : k_deposit<KIND, M, false>;
+  const int cl = deposit_cluster(p.ntiles, total, sms);
+  auto kern = cl > 1 ? (fixed ? k_deposit<KIND, M, true, true> : k_deposit<KIND, M, false, true>)
+                     : (fixed ? k_deposit<KIND, M, true, false> : k_deposit<KIND, M, false, false>);
   if ((err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
     return err;
   LaunchScope ls(p, 3);
-  kern<<<p.ntiles, THREADS, smem, st>>>(p.geom, p.d_nodes, p.d_tile_off, p.d_tile_cur, p.d_rec, p.d_mesh, rmesh,
-                                        p.d_sums, p.cfg.alpha);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr{};
+  cfg.gridDim = dim3((unsigned)p.ntiles * cl);
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  if (cl > 1) {
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)cl;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+  }
+  return cudaLaunchKernelEx(&cfg, kern, p.geom, (const float2*)p.d_nodes, (const unsigned*)p.d_tile_off,
+                            (const unsigned*)p.d_tile_cur, (const float4*)p.d_rec, p.d_mesh, rmesh,
+                            (const double*)p.d_sums, p.cfg.alpha);
 }
 
 }  // namespace
@@ -788,7 +1002,7 @@ cudaError_t launch_assign(Plan& p, const ys_catalog& gal, const ys_catalog& ran,
 cudaError_t launch_random_sums(Plan& p, const ys_catalog& ran, double* out) {
   cudaError_t e = cudaMemsetAsync(out, 0, sizeof(double) * 3, p.stream);
   if (e || ran.n == 0) return e;
-  const unsigned blocks = (unsigned)std::min<int64_t>(152 * 8, (ran.n + THREADS - 1) / THREADS);
+  const int blocks = blocks_for(ran.n, THREADS, 152 * 8);
   k_ran_sums<<<blocks, THREADS, 0, p.stream>>>(ran.w, ran.nbar, ran.n, out);
   return cudaGetLastError();
 }

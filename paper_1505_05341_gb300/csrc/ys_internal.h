@@ -45,7 +45,8 @@ struct Geom {
   float inv_h;      // 1 / H
   float bmin[3];    // box_min (float) for the first guess of the cell index
   int tiles[3];     // tiles per axis
-  int tdim[3];      // tile extent per axis
+  int tdim[3];      // tile extent per axis, a power of two
+  int tshift[3];    // its logarithm
 };
 
 // Nodes with |r|^2 (r from the observer, in units of the mesh's largest |r| component
@@ -108,9 +109,9 @@ struct Plan {
   double* d_acc = nullptr;       // [4][n_bins] shell sums (slot 3 for l_max = 6)
   double* d_sums = nullptr;      // [SUM_COUNT]
   double* d_result = nullptr;    // [5 n_bins + 3]
-  unsigned* d_tile_count = nullptr;  // [ntiles]
-  unsigned* d_tile_off = nullptr;    // [ntiles + 1]
-  unsigned* d_tile_cur = nullptr;    // [ntiles]
+  unsigned* d_tile_count = nullptr;  // [ntiles] records per tile, counted down as border records are placed
+  unsigned* d_tile_off = nullptr;    // [ntiles + 1] first record of each tile's list
+  unsigned* d_tile_cur = nullptr;    // [ntiles] front cursors; after binning the ends of the interior records
   float4* d_rec = nullptr;       // [rec_cap] (x, y, z, signed weight) per (particle, tile)
   // shared randoms (ys_randoms_cache): sum_ran w W per mesh node, and its FP64 sums
   float* d_rmesh = nullptr;      // [m][n][n][n]
