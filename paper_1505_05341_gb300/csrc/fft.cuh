@@ -5,8 +5,9 @@
 //   y,z stage: lines walked by consecutive threads, 16 (12) elements per thread, two
 //     large radices and a small last one done by the reader (LineFft, below).
 //   x stage: interleaved lines, a Stockham autosort transform with 8 (12) elements per
-//     thread: radix-8 stages, then one radix-4 or radix-2; for 3 * 2^a radix-4 stages, an
-//     optional radix-2, then radix-3.  The data go through shared memory between stages.
+//     thread: radix-8 stages, then one radix-4 or radix-2; for 3 * 2^a a radix-12 stage,
+//     then radix-4 stages and an optional radix-2.  The data go through shared memory
+//     between stages.
 // Twiddles come from tables computed in FP64 on the host and rounded to float.
 #pragma once
 #include <cuda_runtime.h>
@@ -29,28 +30,24 @@ __device__ __forceinline__ void line_group_sync() {
   }
 }
 
-// Number of stages of the x stage's transform and the radix of stage s.
-__host__ __device__ constexpr int fft_nstages(int n) {
-  if (is_pow2(n)) {
-    int s = 0, m = n;
-    while (m >= 8) { m /= 8; ++s; }
-    return s + (m > 1 ? 1 : 0);
+// Radix of stage s of the x stage's transform, and the number of stages.
+__host__ __device__ constexpr int fft_radix(int n, int stage) {
+  int m = n, big = 8;
+  if (!is_pow2(n)) {
+    if (stage == 0) return 12;
+    m = n / 12;
+    big = 4;
+    --stage;
   }
-  int s = 0, m = n / 3;
-  while (m % 4 == 0) { m /= 4; ++s; }
-  return s + (m == 2 ? 1 : 0) + 1;
+  for (; m >= big; m /= big, --stage)
+    if (stage == 0) return big;
+  return m;
 }
 
-__host__ __device__ constexpr int fft_radix(int n, int stage) {
-  if (is_pow2(n)) {
-    int m = n, s = 0;
-    while (m >= 8) { if (s == stage) return 8; m /= 8; ++s; }
-    return m;
-  }
-  int m = n / 3, s = 0;
-  while (m % 4 == 0) { if (s == stage) return 4; m /= 4; ++s; }
-  if (m == 2) { if (s == stage) return 2; ++s; }
-  return 3;
+__host__ __device__ constexpr int fft_nstages(int n) {
+  int s = 0;
+  for (int m = n; m > 1; ++s) m /= fft_radix(n, s);
+  return s;
 }
 
 __host__ __device__ constexpr int fft_ns_before(int n, int stage) {
@@ -230,9 +227,12 @@ struct LineFft {
 // are TPL apart, so that the groups' elements fall on different banks (LINE is odd).
 template <int TPL>
 __device__ __forceinline__ int line_of_group(int g) {
-  if constexpr (TPL >= 16) return g;
-  constexpr int G = 16 / TPL;
-  return (g % G) * TPL + (g / G) % TPL + (g / 16) * 16;
+  if constexpr (TPL >= 16) {
+    return g;
+  } else {
+    constexpr int G = 16 / TPL;
+    return (g % G) * TPL + (g / G) % TPL + (g / 16) * 16;
+  }
 }
 
 // exp(-2 pi i q / 32), q < 16
@@ -357,109 +357,102 @@ __host__ __device__ constexpr int fft_tw_offset(int n, int stage) {
   return off;
 }
 
-// Padded buffers of interleaved lines (x stage: element x of line p at x P + p):
-// PADP > 0 inserts PADP elements after every 8 PADP, so that the stores of a radix-8
-// first stage, 8 P apart across a warp, land on distinct bank pairs.
-template <int PADP>
-__host__ __device__ constexpr int lf_pad(int i) {
-  return PADP > 0 ? i + (i / (8 * PADP)) * PADP : i;
-}
+// ---------------------------------------------------------------------------
+// x stage: P interleaved lines, element i of line p at (i + pad) P + p, thread
+// (p, tl = tid / P) with E elements of line p.  Where the first radix is 8, one element
+// of padding follows every 8, so that the first stage's stores, 8 elements apart
+// across a warp, land on distinct bank pairs.
+// ---------------------------------------------------------------------------
+template <int N>
+__host__ __device__ constexpr bool lf_padded() { return fft_radix(N, 0) == 8; }
+template <int N, int P>
+__host__ __device__ constexpr int lf_elems() { return (lf_padded<N>() ? N + N / 8 : N) * P; }
+// Offset of element i; separable (pos(a + c) = pos(a) + pos(c)) for c a multiple of 8.
+template <int N, int P>
+__host__ __device__ constexpr int lf_pos(int i) { return (lf_padded<N>() ? i + (i >> 3) : i) * P; }
 
-// Out-of-place stage over nl interleaved lines (element i of line l at l ls + i es;
-// consecutive threads take consecutive lines): reads src and writes dst (no barrier
-// inside; the caller synchronises before dst is read).  With two buffers a stage
-// needs one barrier instead of the two an in-place stage needs.  PIN / POUT: the
-// padding (lf_pad) of src / dst.
-template <int N, int S, int PIN = 0, int POUT = 0>
-__device__ __forceinline__ void fft_stage_oop(const float2* src, float2* dst, int es, int ls, int nl,
-                                              const float2* tw) {
-  constexpr int R = fft_radix(N, S);
-  constexpr int E = fft_elems(N);
-  constexpr int TPL = N / E;
-  constexpr int NB = E / R;
-  constexpr int NS = fft_ns_before(N, S);
-  constexpr int STRIDE = N / R;
-  const float2* tws = tw + fft_tw_offset(N, S);
-  const int tid = threadIdx.x;
-  const int lpp = blockDim.x / TPL;
-  const bool in_pass = tid < lpp * TPL;
-  const int lane_line = tid % lpp, tl = tid / lpp;
-#pragma unroll 1
-  for (int base_line = 0; base_line < nl; base_line += lpp) {
-    const int line = base_line + lane_line;
-    if (!in_pass || line >= nl) continue;
-    const int lo = line * ls;
-    float2 v[E];
+// First stage (no twiddles): from the unpadded tile src into the work buffer dst.
+template <int N, int P>
+__device__ __forceinline__ void lf_first_stage(const float2* src, float2* dst, int p, int tl) {
+  constexpr int R = fft_radix(N, 0), E = fft_elems(N), TPL = N / E, STRIDE = N / R;
+  const float2* s = src + tl * P + p;
+  float2* d = dst + lf_pos<N, P>(R * tl) + p;
+  float2 v[E];
 #pragma unroll
-    for (int q = 0; q < NB; ++q) {
-      const int j = tl + q * TPL;
+  for (int q = 0; q < E / R; ++q)
 #pragma unroll
-      for (int r = 0; r < R; ++r) v[q * R + r] = src[lf_pad<PIN>(lo + (j + r * STRIDE) * es)];
-    }
+    for (int r = 0; r < R; ++r) v[q * R + r] = s[(q * TPL + r * STRIDE) * P];
 #pragma unroll
-    for (int q = 0; q < NB; ++q) {
-      const int j = tl + q * TPL;
-      const int k = j % NS;
-      if (NS > 1) {
-        const float2* tk = tws + k * (R - 1);
+  for (int q = 0; q < E / R; ++q) {
+    Dft<R>::run(&v[q * R]);
 #pragma unroll
-        for (int r = 1; r < R; ++r) v[q * R + r] = cmul(v[q * R + r], tk[r - 1]);
-      }
-      Dft<R>::run(&v[q * R]);
-      const int outb = (j / NS) * NS * R + k;
-#pragma unroll
-      for (int r = 0; r < R; ++r) dst[lf_pad<POUT>(lo + (outb + r * NS) * es)] = v[q * R + r];
-    }
+    for (int r = 0; r < R; ++r) d[lf_pos<N, P>(R * q * TPL) + r * P] = v[q * R + r];  // R | 8 or no pad
   }
 }
 
-// Stages [S, END) alternating between buffers a and b (CTA-wide barrier after each);
-// the result sits in a when END - S is even, else in b.  PA / PB: their padding.
-template <int N, int S, int END, int PA = 0, int PB = 0, bool Done = (S >= END)>
-struct FftPingPong {
-  __device__ static __forceinline__ void run(float2* a, float2* b, int es, int ls, int nl, const float2* tw) {
-    fft_stage_oop<N, S, PA, PB>(a, b, es, ls, nl, tw);
-    __syncthreads();
-    FftPingPong<N, S + 1, END, PB, PA>::run(b, a, es, ls, nl, tw);
-  }
-};
-template <int N, int S, int END, int PA, int PB>
-struct FftPingPong<N, S, END, PA, PB, true> {
-  __device__ static __forceinline__ void run(float2*, float2*, int, int, int, const float2*) {}
-};
-
-// Last stage into registers: stages 0 .. S-2 must already have run on the lines.
-// Each thread loads its butterfly inputs from line `line` of buf (element i at
-// line + i es, padded by lf_pad<PADL>), applies twiddles and the DFT, and keeps the
-// outputs: v[q * R + r] is element (tl + q * TPL) + r * (N / R).
-template <int N, int PADL = 0>
-__device__ __forceinline__ void fft_last_stage_regs(const float2* buf, int line, int es, int tl, const float2* tw,
-                                                    float2 (&v)[fft_elems(N)]) {
-  constexpr int S = fft_nstages(N) - 1;
-  constexpr int R = fft_radix(N, S);
-  constexpr int E = fft_elems(N);
-  constexpr int TPL = N / E;
-  constexpr int NB = E / R;
-  constexpr int NS = fft_ns_before(N, S);
-  constexpr int STRIDE = N / R;
-  const float2* tws = tw + fft_tw_offset(N, S);
+// The inputs of stage S of the thread's butterflies.
+template <int N, int P, int S>
+__device__ __forceinline__ void lf_load(const float2* buf, int p, int tl, float2 (&v)[fft_elems(N)]) {
+  constexpr int R = fft_radix(N, S), E = fft_elems(N), TPL = N / E, STRIDE = N / R;
+  constexpr bool SEP = !lf_padded<N>() || (TPL % 8 == 0 && STRIDE % 8 == 0);
+  const float2* s = buf + (SEP ? lf_pos<N, P>(tl) : 0) + p;
 #pragma unroll
-  for (int q = 0; q < NB; ++q) {
-    const int j = tl + q * TPL;
+  for (int q = 0; q < E / R; ++q)
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[q * R + r] = buf[lf_pad<PADL>(line + (j + r * STRIDE) * es)];
-  }
-#pragma unroll
-  for (int q = 0; q < NB; ++q) {
-    const int j = tl + q * TPL;
-    const int k = j % NS;
-    if (NS > 1) {
-      const float2* tk = tws + k * (R - 1);
-#pragma unroll
-      for (int r = 1; r < R; ++r) v[q * R + r] = cmul(v[q * R + r], tk[r - 1]);
+    for (int r = 0; r < R; ++r) {
+      const int c = q * TPL + r * STRIDE;
+      v[q * R + r] = s[SEP ? lf_pos<N, P>(c) : lf_pos<N, P>(tl + c)];
     }
+}
+
+// Twiddles and butterflies of stage S on the loaded inputs.
+template <int N, int S>
+__device__ __forceinline__ void lf_butterflies(float2 (&v)[fft_elems(N)], int tl, const float2* tw) {
+  constexpr int R = fft_radix(N, S), E = fft_elems(N), TPL = N / E, NS = fft_ns_before(N, S);
+#pragma unroll
+  for (int q = 0; q < E / R; ++q) {
+    const float2* tk = tw + fft_tw_offset(N, S) + ((tl + q * TPL) % NS) * (R - 1);
+#pragma unroll
+    for (int r = 1; r < R; ++r) v[q * R + r] = cmul(v[q * R + r], tk[r - 1]);
     Dft<R>::run(&v[q * R]);
   }
+}
+
+// Stages S .. last - 1 in place, two CTA barriers each.
+template <int N, int P, int S, bool Done = (S >= fft_nstages(N) - 1)>
+struct LfMiddle {
+  __device__ static __forceinline__ void run(float2* buf, int p, int tl, const float2* tw) {
+    constexpr int R = fft_radix(N, S), E = fft_elems(N), TPL = N / E, NS = fft_ns_before(N, S);
+    static_assert(!lf_padded<N>() || NS % 8 == 0, "separable stores");
+    float2 v[E];
+    lf_load<N, P, S>(buf, p, tl, v);
+    lf_butterflies<N, S>(v, tl, tw);
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < E / R; ++q) {
+      const int j = tl + q * TPL, outb = (j / NS) * NS * R + j % NS;
+      float2* d = buf + lf_pos<N, P>(outb) + p;
+#pragma unroll
+      for (int r = 0; r < R; ++r) d[lf_pos<N, P>(r * NS)] = v[q * R + r];
+    }
+    __syncthreads();
+    LfMiddle<N, P, S + 1>::run(buf, p, tl, tw);
+  }
+};
+template <int N, int P, int S>
+struct LfMiddle<N, P, S, true> {
+  __device__ static __forceinline__ void run(float2*, int, int, const float2*) {}
+};
+
+// Last stage into registers: v[q R + r] is frequency tl + q TPL + r N / R.  The CTA is
+// past its loads when this returns.
+template <int N, int P>
+__device__ __forceinline__ void lf_last_stage(const float2* buf, int p, int tl, const float2* tw,
+                                              float2 (&v)[fft_elems(N)]) {
+  constexpr int S = fft_nstages(N) - 1;
+  lf_load<N, P, S>(buf, p, tl, v);
+  __syncthreads();
+  lf_butterflies<N, S>(v, tl, tw);
 }
 
 }  // namespace ys

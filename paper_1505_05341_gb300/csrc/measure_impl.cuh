@@ -101,7 +101,7 @@ cudaError_t run_x_p(Plan* const* lanes, int W) {
   int dev0 = 0, smem_max = 0;
   if ((err = cudaGetDevice(&dev0))) return err;
   if ((err = cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev0))) return err;
-  // Float-bin copies: several per warp (lanes spread over them) while that costs no
+  // Float-bin copies: several per warp (pencils spread over them) while that costs no
   // resident CTA, else one per warp while it fits, else one shared copy (many shells).
   auto occupancy = [&](int nwb, int* per) -> cudaError_t {
     const size_t sm = XC::smem(nbins, nwb);
@@ -118,8 +118,9 @@ cudaError_t run_x_p(Plan* const* lanes, int W) {
   if (per_warp > 0) {
     nwb = XC::NW;
     per = per_warp;
-    for (int c : {8, 4, 2}) {
+    for (int c : {4, 2}) {
       int pc = 0;
+      if (c > XC::P) continue;
       if ((err = occupancy(XC::NW * c, &pc))) return err;
       if (pc >= per_warp) {
         nwb = XC::NW * c;

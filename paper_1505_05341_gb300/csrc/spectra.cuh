@@ -597,24 +597,22 @@ struct XMulti {
   int nlanes;
 };
 
-// First group of the multipole that group g belongs to (groups: A_0 | l = 2, powers
-// 0..2 of k_x | l = 4, powers 0..4 | l = 6, powers 0..6), and its last.
-__host__ __device__ constexpr int group_first(int g) { return g == 0 ? 0 : (g <= 3 ? 1 : (g <= 8 ? 4 : 9)); }
-__host__ __device__ constexpr int group_last(int g) { return g == 0 ? 0 : (g <= 3 ? 3 : (g <= 8 ? 8 : 15)); }
-
-// Group transformed at tile position q of a pencil block.  With HORNER the powers of
-// k_x of each multipole come highest first, so that the x stage can sum them by
-// Horner's rule (see k_x_combine); otherwise in table order.
-template <bool HORNER>
+// First group of multipole slot s (groups: A_0 | l = 2, powers 0..2 of k_x | l = 4,
+// powers 0..4 | l = 6, powers 0..6): s^2; its last is s^2 + 2 s.
+//
+// Group transformed at tile position q of a pencil block: the powers of k_x of each
+// multipole come highest first, so that they are summed by Horner's rule.
+__host__ __device__ constexpr int group_slot(int g) { return g == 0 ? 0 : (g <= 3 ? 1 : (g <= 8 ? 2 : 3)); }
 __host__ __device__ constexpr int tile_group(int q) {
-  return HORNER ? group_first(q) + group_last(q) - q : q;
+  const int s = group_slot(q);
+  return 2 * s * s + 2 * s - q;
 }
 
-// Whether the x stage sums the k_x powers of each multipole by the compensated
-// Horner scheme (see k_x_combine): always for l_max = 6, and for l_max = 2, 4 except
-// at 256^3 and 512^3, where the x stage is held to 80 registers for three CTAs per SM
-// and the extra error terms would spill (shells there hold many modes, and the
-// plain sums meet the parity bar with a wide margin).
+// Whether the x stage carries the rounding errors of the Horner sums of each multipole
+// (see k_x_combine): always for l_max = 6, and for l_max = 2, 4 except at 256^3 and
+// 512^3, where the x stage is held to 80 registers for three CTAs per SM and the extra
+// error terms would spill (shells there hold many modes, and the plain sums meet the
+// parity bar with a wide margin).
 template <int N, int ELL>
 __host__ __device__ constexpr bool x_horner() { return ELL == 6 || (ELL >= 2 && N != 256 && N != 512); }
 
@@ -622,12 +620,17 @@ __host__ __device__ constexpr bool x_horner() { return ELL == 6 || (ELL >= 2 && 
 // x stage: FFT along x of every (mesh, group) tile of P pencils, fed by TMA.
 // The grouped y,z transforms are a 2D tensor [m NG N rows][np_pad pencils] of
 // float2; one tile (all N rows x P pencils) arrives by BOXES 2D bulk-tensor copies
-// into one of two shared buffers (mbarrier completion), so the copy of the next
-// tile overlaps the FFT of this one.  The last FFT stage stays in registers: each
-// thread owns E modes (one pencil, E values of k_x) for the whole pencil block and
-// accumulates A_0 and k^n A_n there; the per-mode terms of the shell sums go to
-// compensated per-warp float bins in shared memory (add_compensated), folded into
-// the FP64 accumulators when the CTA ends.
+// in one shared buffer (mbarrier completion).  Its first FFT stage moves it to the work
+// buffer, and the copy of the next tile overlaps the other stages, which run in
+// place there.  The last FFT stage stays in registers: each thread owns E modes (one
+// pencil, E values of k_x) for the whole pencil block.
+//
+// Per multipole and mesh the powers of k_x are summed by Horner's rule, one FMA per
+// component and tile; the interlacing phase, the window and the mean over the two meshes
+// are common to all powers and applied once, when the multipole is complete.  A_0 waits
+// in shared memory for the other multipoles.  The per-mode terms of the shell sums go to
+// compensated per-warp float bins in shared memory, folded into the FP64 accumulators
+// when the CTA ends.
 // ---------------------------------------------------------------------------
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
@@ -649,10 +652,9 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
       : "memory");
 }
 
-// Bounded wait for the given phase parity of an mbarrier; false on timeout.
-// Wait for an mbarrier phase for at most limit_ns nanoseconds.
+// Wait for an mbarrier phase (by parity) for at most limit_ns nanoseconds; false on timeout.
 __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity, long long limit_ns) {
-  const unsigned long long t0 = globaltimer_ns();
+  unsigned long long t0 = 0;
   for (;;) {
     unsigned ok;
     asm volatile(
@@ -661,7 +663,9 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned pari
         : "r"(smem_u32(bar)), "r"(parity)
         : "memory");
     if (ok) return true;
-    if ((long long)(globaltimer_ns() - t0) > limit_ns) return false;
+    const unsigned long long t = globaltimer_ns();
+    if (t0 == 0) t0 = t;
+    else if ((long long)(t - t0) > limit_ns) return false;
   }
 }
 
@@ -680,6 +684,12 @@ __device__ __forceinline__ float two_sum_err(float a, float b) {
   return (a - (s - bb)) + (b - bb);
 }
 
+// The same for both components of a complex sum s = a + b.
+__device__ __forceinline__ float2 two_sum_err2(float2 a, float2 b, float2 s) {
+  const float2 bb = csub(s, a);
+  return cadd(csub(a, csub(s, bb)), csub(b, bb));
+}
+
 template <int N, int ELL, int M, int PX = k3_pencils(N)>
 struct XCombine {
   static constexpr int P = PX;  // pencils per CTA
@@ -689,30 +699,30 @@ struct XCombine {
   static constexpr int NW = THREADS / 32;
   static constexpr int NG = GroupTable<ELL>::NG;
   // shell-sum slots: |A_0|^2, Re A_0 A_2^*, Re A_0 A_4^* (and Re A_0 A_6^* for l = 6)
-  static constexpr int SLOTS = ELL == 6 ? 4 : 3;
+  static constexpr int SLOTS = ELL / 2 + 1;
   static constexpr int TILES = NG * M;
   static constexpr int BOX_ROWS = x_box_rows(N);
   static constexpr int BOXES = N / BOX_ROWS;
   static_assert(BOXES * BOX_ROWS == N, "boxes must tile the x axis");
   static constexpr unsigned TILE_BYTES = (unsigned)(N * P * sizeof(float2));
-  // work buffer padded (lf_pad) where the first stage is radix 8
-  static constexpr int PADW = fft_radix(N, 0) == 8 ? P : 0;
-  static constexpr int WK_ELEMS = lf_pad<PADW>(N * P);
-  static constexpr int RL = fft_radix(N, fft_nstages(N) - 1);  // last radix
-  // resident CTAs per SM the register budget is set for (3 x 256 threads at 256^3, 512^3)
-  static constexpr int MIN_BLOCKS = ((N == 256 || N == 512) && ELL <= 4 && THREADS == 256) ? 3 : 1;
+  static constexpr int STAGES = fft_nstages(N);
+  static constexpr int WK_ELEMS = lf_elems<N, P>();
+  static constexpr int RL = fft_radix(N, STAGES - 1);  // last radix
+  // resident CTAs per SM the register budget is set for (3 x 256 threads at 256^3, 512^3;
+  // 2 where the sums' errors are carried)
+  static constexpr int MIN_BLOCKS = THREADS != 256 || E != 8 ? 1 : (x_horner<N, ELL>() ? 2 : 3);
   static_assert(THREADS % 32 == 0, "threads");
   // nwb copies of the compensated float shell bins: a sum and an error term per shell
-  // and slot.  With nwb = NW c (c copies per warp) lane l = p + P j of warp w adds into
-  // copy w c + j mod c, which divides the lanes of one pencil (neighbouring k_x, mostly
-  // one shell) that would hit one address in one instruction (same-address shared
-  // atomics are served one after another); with fewer copies warp w adds into copy
-  // w mod nwb.
+  // and slot.  With nwb = NW c (c copies per warp) the lanes of pencil p add into copy
+  // p mod c of their warp's: the run-reduced sums of different pencils, which often fall
+  // in one shell, then never meet in one instruction (same-address shared atomics are
+  // served one after another); with fewer copies warp w adds into copy w mod nwb.
   static size_t smem(int nbins, int nwb) {
-    size_t b = 2 * (size_t)TILE_BYTES + sizeof(float2) * WK_ELEMS;  // two tile buffers and a work buffer
-    b += sizeof(float2) * 2 * N + sizeof(float) * N;         // twiddles, phases, windows
-    b += sizeof(float) * 2 * nwb * SLOTS * nbins;            // float bins and their error terms
-    return b + 128;                                          // alignment slack
+    size_t b = TILE_BYTES + sizeof(float2) * WK_ELEMS;  // tile and work buffer
+    if (ELL > 0) b += TILE_BYTES;                       // A_0
+    b += sizeof(float2) * 2 * N + sizeof(float) * N;    // twiddles, phases, windows
+    b += sizeof(float) * 2 * nwb * SLOTS * nbins;       // float bins and their error terms
+    return b;
   }
 };
 
@@ -723,34 +733,30 @@ k_x_combine(const __grid_constant__ XMulti pm, int np_pad, const short2* __restr
             const short* __restrict__ lut, int n2_hi, int nbins, int nwb) {
   // lane blockIdx.y: its grouped transforms (tensor map), shell accumulators, error flag
   const CUtensorMap* gmap = &pm.map[blockIdx.y];
-  double* __restrict__ acc = pm.acc[blockIdx.y];
-  int* __restrict__ err = pm.err[blockIdx.y];
   using XC = XCombine<N, ELL, M, PX>;
-  constexpr int P = XC::P, E = XC::E, TPL = XC::TPL, TILES = XC::TILES, RL = XC::RL;
-  constexpr bool HORNER = x_horner<N, ELL>();
-  constexpr int NBL = E / RL;
-  extern __shared__ unsigned char smem_raw[];
-  __shared__ __align__(8) unsigned long long bar[2];
+  constexpr int P = XC::P, E = XC::E, TPL = XC::TPL, TILES = XC::TILES, RL = XC::RL, SLOTS = XC::SLOTS;
+  constexpr int THREADS = XC::THREADS;
+  constexpr bool COMP = x_horner<N, ELL>();
+  extern __shared__ __align__(128) float2 smem_x[];
+  __shared__ __align__(8) unsigned long long bar;
   __shared__ int s_fail;
-  unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
-  float2* T0 = reinterpret_cast<float2*>(base);
-  float2* Wk = T0 + 2 * N * P;  // second buffer of the out-of-place stages (padded)
-  float2* tw = Wk + XC::WK_ELEMS;
+  float2* T = smem_x;
+  float2* Wk = T + N * P;
+  float2* sA0 = Wk + XC::WK_ELEMS;
+  float2* tw = sA0 + (ELL > 0 ? N * P : 0);
   float2* phs = tw + N;
   float* invw = reinterpret_cast<float*>(phs + N);
-  constexpr int SLOTS = XC::SLOTS;
   float* wbin = invw + N;                    // [nwb][SLOTS][nbins] sums
   float* wcmp = wbin + nwb * SLOTS * nbins;  // [nwb][SLOTS][nbins] their rounding errors
   const int tid = threadIdx.x, warp = tid >> 5;
-  for (int k = tid; k < N; k += blockDim.x) {
+  for (int k = tid; k < N; k += THREADS) {
     tw[k] = tw_g[k];
     phs[k] = phase_g[k];
     invw[k] = invw_g[k];
   }
-  for (int k = tid; k < 2 * nwb * SLOTS * nbins; k += blockDim.x) wbin[k] = 0.f;
+  for (int k = tid; k < 2 * nwb * SLOTS * nbins; k += THREADS) wbin[k] = 0.f;
   if (tid == 0) {
-    mbar_init(&bar[0], 1);
-    mbar_init(&bar[1], 1);
+    mbar_init(&bar, 1);
     s_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -758,142 +764,124 @@ k_x_combine(const __grid_constant__ XMulti pm, int np_pad, const short2* __restr
   const int npb = np_pad / P;
   const int mine = blockIdx.x < npb ? (npb - 1 - blockIdx.x) / gridDim.x + 1 : 0;
   const int total = mine * TILES;
-  auto issue = [&](int s) {
+  auto issue = [&](int s) {  // thread 0: the copy of tile s
     const int k = s / TILES, t = s - k * TILES;
-    const int gi = tile_group<HORNER>(t / M), mj = t - (t / M) * M;
+    const int gi = tile_group(t / M), mj = t % M;
     const int pb = blockIdx.x + k * gridDim.x;
-    float2* dst = T0 + (s & 1) * N * P;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    mbar_expect_tx(&bar[s & 1], XC::TILE_BYTES);
+    mbar_expect_tx(&bar, XC::TILE_BYTES);
 #pragma unroll
     for (int bx = 0; bx < XC::BOXES; ++bx)
-      tma_load_2d(dst + bx * XC::BOX_ROWS * P, gmap, pb * P * 2, (mj * XC::NG + gi) * N + bx * XC::BOX_ROWS, &bar[s & 1]);
+      tma_load_2d(T + bx * XC::BOX_ROWS * P, gmap, pb * P * 2, (mj * XC::NG + gi) * N + bx * XC::BOX_ROWS, &bar);
   };
   if (tid == 0 && total > 0) issue(0);
   const int p = tid % P, tl = tid / P;
-  float2 a0[E], ga[E];
-  float2 gl[HORNER ? E : 1];  // rounding errors of the Horner sums in ga
-  int bins[E];  // shell of each of this thread's modes in the current pencil (-1: none)
-  int ky = 0, kz = -1, iyk = 0;
-  float cf_pen = 0.f;
-  float2 ph_pen = make_float2(1.f, 0.f);
-  int s_stop = total;  // step whose wait ran out (copies s_stop and s_stop + 1 may be in flight)
-  for (int s = 0; s < total; ++s) {
-    if (tid == 0 && s + 1 < total) issue(s + 1);
-    if (!mbar_wait(&bar[s & 1], (s >> 1) & 1, 1000000000LL)) s_fail = 1;  // 1 s
-    __syncthreads();
-    if (s_fail) {
-      s_stop = s;
-      break;
+  const float m0 = (float)tl;
+  // mode e of this thread: k_x = tl + koff(e), as a signed frequency tl + koff(e) - N past N / 2
+  auto koff = [](int e) { return (e / RL) * TPL + (e % RL) * (N / RL); };
+  auto msign = [&](int e) { return koff(e) < N / 2 ? koff(e) : koff(e) - N; };
+  const int copy = nwb >= XC::NW ? warp * (nwb / XC::NW) + p % (nwb / XC::NW) : warp % nwb;
+  float* wb0 = wbin + copy * SLOTS * nbins;
+  const int cmp_off = nwb * SLOTS * nbins;
+  int s = 0;
+  bool failed = false;
+  for (int k = 0; k < mine && !failed; ++k) {
+    const short2 pc = pencil[(blockIdx.x + k * gridDim.x) * P + p];
+    const int ky = pc.x, kz = pc.y;  // kz < 0: a padding pencil, no shell
+    const int iyk = ky < 0 ? ky + N : ky, kzc = kz < 0 ? 0 : kz;
+    const int kyz2 = ky * ky + kz * kz;
+    const float cf_pen = invw[iyk] * invw[kzc] * (M == 2 ? 0.5f : 1.f);
+    const float2 ph_pen = cmul(phs[iyk], phs[kzc]);
+    const float wgt = kz == 0 ? 1.f : 2.f;
+    unsigned keys[(E + 1) / 2];  // shells of this thread's modes (16 bits each; 0xffff: none)
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int mx = tl + msign(e), n2 = mx * mx + kyz2;
+      const unsigned key = (kz >= 0 && n2 < n2_hi) ? (unsigned short)lut[n2] : 0xffffu;
+      if (e & 1) keys[e / 2] |= key << 16;
+      else keys[e / 2] = key;
     }
-    const int k = s / TILES, t = s - k * TILES;
-    const int gi = tile_group<HORNER>(t / M), mj = t - (t / M) * M;
-    if (t == 0) {
-      const short2 pc = pencil[(blockIdx.x + k * gridDim.x) * P + p];
-      ky = pc.x;
-      kz = pc.y;
-      iyk = ky < 0 ? ky + N : ky;
-      const int kzc = kz < 0 ? 0 : kz;
-      cf_pen = invw[iyk] * invw[kzc] * (M == 2 ? 0.5f : 1.f);
-      ph_pen = cmul(phs[iyk], phs[kzc]);
+#pragma unroll 1
+    for (int slot = 0; slot < SLOTS && !failed; ++slot) {
+      float2 H[M][E];               // Horner sums of each mesh
+      float2 C[COMP ? M : 1][COMP ? E : 1];  // and their rounding errors
 #pragma unroll
-      for (int q = 0; q < NBL; ++q)
-#pragma unroll
-        for (int r = 0; r < RL; ++r) {
-          const int kx = tl + q * TPL + r * (N / RL);
-          const int mx = kx <= N / 2 ? kx : kx - N;
-          const int n2 = mx * mx + ky * ky + kz * kz;
-          bins[q * RL + r] = (kz >= 0 && n2 < n2_hi) ? lut[n2] : -1;
-        }
-    }
-    float2* Tb = T0 + (s & 1) * N * P;
-    constexpr int SM_STAGES = fft_nstages(N) - 1;  // stages through shared memory
-    FftPingPong<N, 0, SM_STAGES, 0, XC::PADW>::run(Tb, Wk, P, 1, P, tw);
-    const float2* Tf = (SM_STAGES % 2 == 0) ? Tb : Wk;
-    constexpr int PADF = (SM_STAGES % 2 == 0) ? 0 : XC::PADW;
-    float2 v[E];
-    fft_last_stage_regs<N, PADF>(Tf, p, P, tl, tw, v);
-    const int first = group_first(gi);
-    const int pw = gi - first;  // power of k_x
-#pragma unroll
-    for (int q = 0; q < NBL; ++q)
-#pragma unroll
-      for (int r = 0; r < RL; ++r) {
-        const int e = q * RL + r;
-        const int kx = tl + q * TPL + r * (N / RL);
-        const int mx = kx <= N / 2 ? kx : kx - N;
-        float2 X = v[e];
-        if (M == 2 && mj == 1) X = cmul(X, cmul(phs[kx], ph_pen));
-        if (HORNER && gi != 0) {
-          // sum_p m_x^p X_p by Horner's rule (highest power first), every step
-          // error-free: the product by the integer m_x is split exactly with an FMA
-          // and the add with TwoSum, and both errors go to gl.  The window and the
-          // interlacing mean, common to all powers, are applied at completion.
-          if (mj == 0 && gi == group_last(gi)) {
-            ga[e] = X;
-            gl[e] = make_float2(0.f, 0.f);
-          } else {
-            const float m = mj == 0 ? (float)mx : 1.f;
-            const float pr = ga[e].x * m, pi = ga[e].y * m;
-            const float er = fmaf(ga[e].x, m, -pr), ei = fmaf(ga[e].y, m, -pi);
-            ga[e].x = pr + X.x;
-            ga[e].y = pi + X.y;
-            gl[e].x = fmaf(gl[e].x, m, er) + two_sum_err(pr, X.x);
-            gl[e].y = fmaf(gl[e].y, m, ei) + two_sum_err(pi, X.y);
-          }
-          continue;
-        }
-        float kp = cf_pen * invw[kx];
-        for (int u = 0; u < pw; ++u) kp *= (float)mx;
-        if (gi == 0) {
-          if (mj == 0) a0[e] = make_float2(kp * X.x, kp * X.y);
-          else { a0[e].x = fmaf(kp, X.x, a0[e].x); a0[e].y = fmaf(kp, X.y, a0[e].y); }
-        } else if (gi == first && mj == 0) {
-          ga[e] = make_float2(kp * X.x, kp * X.y);
-        } else {
-          ga[e].x = fmaf(kp, X.x, ga[e].x);
-          ga[e].y = fmaf(kp, X.y, ga[e].y);
-        }
-      }
-    // a multipole is complete after its last tile (for l = 6 its power-0 group)
-    const bool complete = (mj == M - 1) && (HORNER ? gi == group_first(gi) : gi == group_last(gi));
-    if (complete) {
-      const int slot = gi == 0 ? 0 : (gi <= 3 ? 1 : (gi <= 8 ? 2 : 3));
-      if (HORNER && slot > 0) {
+      for (int mj = 0; mj < M; ++mj)
 #pragma unroll
         for (int e = 0; e < E; ++e) {
-          const int kx = tl + (e / RL) * TPL + (e % RL) * (N / RL);
-          const float c = cf_pen * invw[kx];
-          ga[e] = make_float2(c * (ga[e].x + gl[e].x), c * (ga[e].y + gl[e].y));
+          H[mj][e] = make_float2(0.f, 0.f);
+          if constexpr (COMP) C[mj][e] = make_float2(0.f, 0.f);
+        }
+#pragma unroll 1
+      for (int q = 0; q <= 2 * slot && !failed; ++q) {
+#pragma unroll
+        for (int mj = 0; mj < M; ++mj) {
+          float2 v[E];
+          if (!mbar_wait(&bar, s & 1, 1000000000LL)) s_fail = 1;  // 1 s
+          lf_first_stage<N, P>(T, Wk, p, tl);
+          __syncthreads();
+          if (s_fail) {
+            failed = true;
+            break;
+          }
+          if (tid == 0 && s + 1 < total) issue(s + 1);
+          LfMiddle<N, P, 1>::run(Wk, p, tl, tw);
+          lf_last_stage<N, P>(Wk, p, tl, tw, v);  // (a barrier after its loads)
+          ++s;
+#pragma unroll
+          for (int e = 0; e < E; ++e) {
+            const float m = m0 + (float)msign(e);
+            if constexpr (COMP) {
+              // every step error-free: the product by the integer m is split exactly with
+              // an FMA and the add with TwoSum, and both errors go to C
+              const float2 mm = make_float2(m, m);
+              const float2 pr = __fmul2_rn(H[mj][e], mm);
+              const float2 er = __ffma2_rn(H[mj][e], mm, make_float2(-pr.x, -pr.y));
+              H[mj][e] = cadd(pr, v[e]);
+              C[mj][e] = cadd(__ffma2_rn(C[mj][e], mm, er), two_sum_err2(pr, v[e], H[mj][e]));
+            } else {
+              H[mj][e].x = fmaf(H[mj][e].x, m, v[e].x);
+              H[mj][e].y = fmaf(H[mj][e].y, m, v[e].y);
+            }
+          }
         }
       }
-      // the lanes of one pencil (lane = p + P j) hold neighbouring k_x, mostly in one
-      // shell: spread them over the warp's copies by j
-      const int copy = nwb >= XC::NW ? warp * (nwb / XC::NW) + ((tid & 31) / P) % (nwb / XC::NW) : warp % nwb;
-      float* wb = wbin + (copy * SLOTS + slot) * nbins;
-      float* wc = wb + nwb * SLOTS * nbins;
-      const float wgt = kz == 0 ? 1.f : 2.f;
+      if (failed) break;
       // The lanes of one pencil (lane = p + P j, j < 32 / P) hold neighbouring k_x and
       // mostly share a shell: each run of equal shells (cut wherever neighbouring lanes
       // differ) is first summed across its lanes by a segmented suffix scan with
       // compensated adds, and only the run's first lane adds it to the bins.
-      const int lane = tid & 31, jl = lane / P;
+      const int jl = (tid & 31) / P;
       constexpr int LG = 32 / P;
+      float* wb = wb0 + slot * nbins;
 #pragma unroll
       for (int e = 0; e < E; ++e) {
-        const int kx = tl + (e / RL) * TPL + (e % RL) * (N / RL);
-        const int mx = kx <= N / 2 ? kx : kx - N;
+        const int kx = tl + koff(e);
+        float2 A = H[0][e];
+        if constexpr (COMP) A = cadd(A, C[0][e]);
+        if constexpr (M == 2) {
+          float2 B = H[M - 1][e];
+          if constexpr (COMP) B = cadd(B, C[M - 1][e]);
+          B = cmul(B, cmul(phs[kx], ph_pen));
+          A = cadd(A, B);
+        }
+        const float c = cf_pen * invw[kx];
+        A = make_float2(c * A.x, c * A.y);
         float val;
         if (slot == 0) {
-          val = wgt * (a0[e].x * a0[e].x + a0[e].y * a0[e].y);
+          if (ELL > 0) sA0[e * THREADS + tid] = A;
+          val = wgt * (A.x * A.x + A.y * A.y);
         } else {
-          const float inv = 1.f / (float)(mx * mx + ky * ky + kz * kz);
+          const float2 a0 = sA0[e * THREADS + tid];
+          const int mx = tl + msign(e);
+          const float inv = 1.f / (float)(mx * mx + kyz2);
           const float ik = slot == 1 ? inv : (slot == 2 ? inv * inv : inv * inv * inv);  // 1 / k^(2 slot)
-          val = wgt * ik * (a0[e].x * ga[e].x + a0[e].y * ga[e].y);
+          val = wgt * ik * (a0.x * A.x + a0.y * A.y);
         }
-        const int key = bins[e];
-        const int key_next = __shfl_down_sync(0xffffffffu, key, P);
-        const int key_prev = __shfl_up_sync(0xffffffffu, key, P);
+        const unsigned key = (e & 1) ? keys[e / 2] >> 16 : keys[e / 2] & 0xffffu;
+        if (__all_sync(0xffffffffu, key == 0xffffu)) continue;  // no lane's mode is in a shell
+        const unsigned key_next = __shfl_down_sync(0xffffffffu, key, P);
+        const unsigned key_prev = __shfl_up_sync(0xffffffffu, key, P);
         int end = (jl == LG - 1 || key_next != key) ? 1 : 0;  // this lane's run stops here
         float cmp = 0.f;
 #pragma unroll
@@ -907,27 +895,27 @@ k_x_combine(const __grid_constant__ XMulti pm, int np_pad, const short2* __restr
             end = en;
           }
         }
-        if (key >= 0 && (jl == 0 || key_prev != key)) {
+        if (key != 0xffffu && (jl == 0 || key_prev != key)) {
           const float old = atomicAdd(wb + key, val);
           const float err = cmp + two_sum_err(old, val);
-          if (err != 0.f) atomicAdd(wc + key, err);
+          if (err != 0.f) atomicAdd(wb + cmp_off + key, err);
         }
       }
     }
-    __syncthreads();
   }
-  if (s_fail) {
+  if (failed) {
     if (tid == 0) {
-      atomicExch(err, 2);
-      // Copies s_stop and s_stop + 1 (if issued) are the last ones issued into their
-      // buffers: wait for each by its own phase parity before the CTA's shared memory
-      // is released (bounded; every earlier copy has completed).
-      for (int s = s_stop; s < s_stop + 2 && s < total; ++s) mbar_wait(&bar[s & 1], (s >> 1) & 1, 100000000LL);
+      atomicExch(pm.err[blockIdx.y], 2);
+      // Copy s is the last one issued: wait for it by its own phase parity before the
+      // CTA's shared memory is released (bounded; every earlier copy has completed).
+      mbar_wait(&bar, s & 1, 100000000LL);
     }
     return;
   }
+  __syncthreads();
   // FP64 fold of every warp copy's sum and error term, once per CTA.
-  for (int b = tid; b < SLOTS * nbins; b += blockDim.x) {
+  double* __restrict__ acc = pm.acc[blockIdx.y];
+  for (int b = tid; b < SLOTS * nbins; b += THREADS) {
     double v = 0.0;
     for (int w = 0; w < nwb; ++w) v += (double)wbin[w * SLOTS * nbins + b] + (double)wcmp[w * SLOTS * nbins + b];
     if (v != 0.0) atomicAdd(&acc[b], v);

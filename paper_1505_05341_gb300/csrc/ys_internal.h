@@ -34,9 +34,10 @@ constexpr int YZ_MAX_LANES = 8;
 // Pencils per CTA of the x stage (its FFT tile): the default for mesh size n and the
 // alternative the autotuner also times.  Both are powers of two; the plan pads its
 // pencil list to a multiple of the larger.
-__host__ __device__ constexpr int k3_pencils(int n) { return n <= 32 ? 32 : (n >= 512 ? 4 : 8); }
+// (At 16^3 and 32^3 a CTA is one warp, so that the few pencils spread over the SMs.)
+__host__ __device__ constexpr int k3_pencils(int n) { return n <= 16 ? 16 : (n >= 512 ? 4 : 8); }
 __host__ __device__ constexpr int k3_pencils_alt(int n) {
-  return n <= 32 ? 16 : (n >= 1024 ? 2 : (n >= 512 ? 8 : 4));
+  return n <= 32 ? 32 : (n >= 1024 ? 2 : (n >= 512 ? 8 : 4));
 }
 constexpr int kTileCandidates[5][3] = {{16, 16, 32}, {8, 16, 32}, {16, 16, 16}, {32, 16, 32}, {8, 8, 32}};
 
