@@ -5,12 +5,10 @@
 // shot-noise subtraction.
 //
 // Weights are kept in bfloat16 for the forward and backward passes (FP32 master copy
-// and Adam moments); activations and every accumulation are FP32.  A CTA handles
-// MLP_ROWS rows: per-row phases run one row per thread with activations in shared
-// memory laid out [feature][row] (odd row stride, so a warp's rows hit distinct
-// banks), the weight-gradient contractions run one weight per thread over the CTA's
-// rows, and each CTA adds its partial gradient to the global FP32 gradient with
-// atomics.
+// and Adam moments); activations and every accumulation are FP32.  A CTA walks tiles of
+// MLP_ROWS rows with all weights and the tile's activations in shared memory; every
+// 64 x 64 product of a tile is a register-blocked FP32 product (4 x 4 per thread), the
+// activations' derivatives and the weight gradients stay in registers.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -25,8 +23,10 @@
 namespace ys {
 namespace {
 
-constexpr int MLP_ROWS = 64;   // rows (and threads) per CTA
-constexpr int RS = MLP_ROWS + 1;  // padded row stride of the [feature][row] buffers
+constexpr int MLP_ROWS = 64;      // rows per tile
+constexpr int MLP_THREADS = 256;  // 16 x 16 threads, a 4 x 4 block of every 64 x 64 product each
+constexpr int RS = 68;            // row stride of the [feature][row] and weight buffers: a multiple of 4
+                                  // floats, and 17 units of 16 bytes, so that 8 rows fall on distinct banks
 constexpr int H = 64;
 constexpr int IN = 5, OUT = 3;
 constexpr int OFF_W1 = 0, OFF_B1 = OFF_W1 + H * IN, OFF_W2 = OFF_B1 + H, OFF_B2 = OFF_W2 + H * H;
@@ -34,162 +34,350 @@ constexpr int OFF_W3 = OFF_B2 + H, OFF_B3 = OFF_W3 + H * H, OFF_W4 = OFF_B3 + H,
 constexpr int NP = OFF_B4 + OUT;
 static_assert(NP == YS_MLP_PARAMS, "parameter count");
 
+// GELU (erf form) of x, and its derivative.
 __device__ __forceinline__ float gelu(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_grad(float x) {
-  return 0.5f * (1.f + erff(x * 0.70710678118654752f)) + x * expf(-0.5f * x * x) * 0.39894228040143268f;
+__device__ __forceinline__ float gelu_both(float x, float& grad) {
+  const float cdf = 0.5f * (1.f + erff(x * 0.70710678118654752f));
+  grad = cdf + x * expf(-0.5f * x * x) * 0.39894228040143268f;
+  return x * cdf;
 }
 
 struct MlpSmem {
-  float w[NP];
+  float w1[IN * H];       // [input][hidden]
+  float w2[H * RS], w3[H * RS];
+  float w4[OUT * RS];
+  float b[3 * H + 4];     // biases of the hidden layers, then of the output
   float x[IN * RS];
-  float z[3][H * RS];   // pre-activations of the hidden layers (overwritten by deltas)
-  float h[3][H * RS];   // post-activations
-  float d4[OUT * RS];
+  float y[OUT * RS];      // outputs, then their deltas
+  float h[3][H * RS];     // post-activations; h[2] later holds the second layer's deltas
+  float d[H * RS];        // deltas of the third, then of the first layer
 };
 
-__device__ __forceinline__ void load_weights(float* w, const __nv_bfloat16* __restrict__ w16) {
-  for (int k = threadIdx.x; k < NP; k += blockDim.x) w[k] = __bfloat162float(w16[k]);
-}
-
-// One dense layer for this thread's row r: out[o][r] = b[o] + sum_i W[o][i] in[i][r].
-__device__ __forceinline__ void dense_row(const float* W, const float* b, const float* in, int nin, float* out,
-                                          int nout, int r) {
-  for (int o = 0; o < nout; ++o) {
-    float acc = b[o];
-    const float* wr = W + o * nin;
-    for (int i = 0; i < nin; ++i) acc = fmaf(wr[i], in[i * RS + r], acc);
-    out[o * RS + r] = acc;
+__device__ __forceinline__ void load_weights(MlpSmem& s, const __nv_bfloat16* __restrict__ w16) {
+  for (int k = threadIdx.x; k < H * H; k += MLP_THREADS) {
+    const int o = k / H, i = k % H;
+    s.w2[o * RS + i] = __bfloat162float(w16[OFF_W2 + k]);
+    s.w3[o * RS + i] = __bfloat162float(w16[OFF_W3 + k]);
   }
+  for (int k = threadIdx.x; k < H * IN; k += MLP_THREADS) s.w1[(k % IN) * H + k / IN] = __bfloat162float(w16[OFF_W1 + k]);
+  if (threadIdx.x < OUT * H)
+    s.w4[threadIdx.x / H * RS + threadIdx.x % H] = __bfloat162float(w16[OFF_W4 + threadIdx.x]);
+  if (threadIdx.x < H) {
+    s.b[threadIdx.x] = __bfloat162float(w16[OFF_B1 + threadIdx.x]);
+    s.b[H + threadIdx.x] = __bfloat162float(w16[OFF_B2 + threadIdx.x]);
+    s.b[2 * H + threadIdx.x] = __bfloat162float(w16[OFF_B3 + threadIdx.x]);
+  }
+  if (threadIdx.x < OUT) s.b[3 * H + threadIdx.x] = __bfloat162float(w16[OFF_B4 + threadIdx.x]);
 }
 
-// Forward pass of the CTA's rows; keeps z and h for the backward pass.
-__device__ __forceinline__ void forward_rows(MlpSmem& s, int rows, float (&y)[OUT]) {
-  const int r = threadIdx.x;
-  const bool ok = r < rows;
-  if (ok) {
-    dense_row(s.w + OFF_W1, s.w + OFF_B1, s.x, IN, s.z[0], H, r);
-    for (int o = 0; o < H; ++o) s.h[0][o * RS + r] = gelu(s.z[0][o * RS + r]);
-    dense_row(s.w + OFF_W2, s.w + OFF_B2, s.h[0], H, s.z[1], H, r);
-    for (int o = 0; o < H; ++o) s.h[1][o * RS + r] = gelu(s.z[1][o * RS + r]);
-    dense_row(s.w + OFF_W3, s.w + OFF_B3, s.h[1], H, s.z[2], H, r);
-    for (int o = 0; o < H; ++o) s.h[2][o * RS + r] = gelu(s.z[2][o * RS + r]);
-    for (int o = 0; o < OUT; ++o) {
-      float acc = s.w[OFF_B4 + o];
-      for (int i = 0; i < H; ++i) acc = fmaf(s.w[OFF_W4 + o * H + i], s.h[2][i * RS + r], acc);
-      y[o] = acc;
+// This thread's block of a layer's outputs: hidden units a + 16 k (k < 4) of rows
+// 4 c .. 4 c + 3.
+struct Block {
+  int a, c;
+  __device__ Block() {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    a = (lane & 7) + 8 * (warp & 1);
+    c = (lane >> 3) + 4 * (warp >> 1);
+  }
+};
+
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ void st4(float* p, const float (&v)[4]) {
+  *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void axpy4(float (&acc)[4], float w, const float4& v) {
+  acc[0] = fmaf(w, v.x, acc[0]);
+  acc[1] = fmaf(w, v.y, acc[1]);
+  acc[2] = fmaf(w, v.z, acc[2]);
+  acc[3] = fmaf(w, v.w, acc[3]);
+}
+
+// acc[k][.] = bias[a + 16 k] + sum_i W[a + 16 k][i] in[i][4 c ..]: 8 shared loads of 16
+// bytes per 64 FMAs.
+__device__ __forceinline__ void dense(const float* W, const float* bias, const float* in, const Block& t,
+                                      float (&acc)[4][4]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) acc[k][r] = bias[t.a + 16 * k];
+#pragma unroll 2
+  for (int i = 0; i < H; i += 4) {
+    float4 v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = ld4(in + (i + j) * RS + 4 * t.c);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float4 w = ld4(W + (t.a + 16 * k) * RS + i);
+      axpy4(acc[k], w.x, v[0]);
+      axpy4(acc[k], w.y, v[1]);
+      axpy4(acc[k], w.z, v[2]);
+      axpy4(acc[k], w.w, v[3]);
     }
   }
 }
 
-__global__ void __launch_bounds__(MLP_ROWS) k_mlp_forward(const __nv_bfloat16* __restrict__ w16,
-                                                          const float* __restrict__ X, int64_t rows,
-                                                          float* __restrict__ Y) {
-  extern __shared__ __align__(16) unsigned char raw[];
-  MlpSmem& s = *reinterpret_cast<MlpSmem*>(raw);
-  load_weights(s.w, w16);
-  const int64_t r0 = (int64_t)blockIdx.x * MLP_ROWS;
-  const int nr = rows - r0 < MLP_ROWS ? (int)(rows - r0) : MLP_ROWS;
-  for (int k = threadIdx.x; k < IN * MLP_ROWS; k += blockDim.x) {
-    const int f = k / MLP_ROWS, r = k % MLP_ROWS;
-    s.x[f * RS + r] = r < nr ? X[(r0 + r) * IN + f] : 0.f;
+// acc[k][.] = sum_o W[o][a + 16 k] D[o][4 c ..]
+__device__ __forceinline__ void dense_t(const float* W, const float* D, const Block& t, float (&acc)[4][4]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) acc[k][r] = 0.f;
+#pragma unroll 4
+  for (int o = 0; o < H; ++o) {
+    const float4 v = ld4(D + o * RS + 4 * t.c);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) axpy4(acc[k], W[o * RS + t.a + 16 * k], v);
+  }
+}
+
+// g[k][l] += sum_r D[a + 16 k][r] A[c + 16 l][r] over the tile's rows
+__device__ __forceinline__ void outer(const float* D, const float* A, const Block& t, float (&g)[4][4]) {
+#pragma unroll 2
+  for (int r = 0; r < MLP_ROWS; r += 4) {
+    float4 v[4];
+#pragma unroll
+    for (int l = 0; l < 4; ++l) v[l] = ld4(A + (t.c + 16 * l) * RS + r);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float4 d = ld4(D + (t.a + 16 * k) * RS + r);
+#pragma unroll
+      for (int l = 0; l < 4; ++l)
+        g[k][l] = fmaf(d.x, v[l].x, fmaf(d.y, v[l].y, fmaf(d.z, v[l].z, fmaf(d.w, v[l].w, g[k][l]))));
+    }
+  }
+}
+
+// sum_r A[r] B[r] (B == nullptr: sum_r A[r]) over the tile's rows
+__device__ __forceinline__ float row_dot(const float* A, const float* B) {
+  float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+  for (int r = 0; r < MLP_ROWS; r += 4) {
+    const float4 a = ld4(A + r), b = B ? ld4(B + r) : make_float4(1.f, 1.f, 1.f, 1.f);
+    s[0] = fmaf(a.x, b.x, s[0]);
+    s[1] = fmaf(a.y, b.y, s[1]);
+    s[2] = fmaf(a.z, b.z, s[2]);
+    s[3] = fmaf(a.w, b.w, s[3]);
+  }
+  return (s[0] + s[1]) + (s[2] + s[3]);
+}
+
+// Forward pass of the tile of nr rows from r0: outputs to s.y, post-activations in s.h and,
+// with GRAD, the activations' derivatives of this thread's blocks in gp.  The caller has
+// synchronised after the last use of s.x, s.h and s.y.
+template <bool GRAD>
+__device__ __forceinline__ void forward_tile(MlpSmem& s, const float* __restrict__ X, int64_t r0, int nr,
+                                             const Block& t, float (&gp)[3][4][4]) {
+  for (int k = threadIdx.x; k < IN * MLP_ROWS; k += MLP_THREADS) {
+    const int r = k / IN, f = k % IN;
+    s.x[f * RS + r] = r < nr ? X[r0 * IN + k] : 0.f;
   }
   __syncthreads();
-  float y[OUT];
-  forward_rows(s, nr, y);
-  if ((int)threadIdx.x < nr)
-    for (int o = 0; o < OUT; ++o) Y[(r0 + threadIdx.x) * OUT + o] = y[o];
+  float acc[4][4];
+#pragma unroll
+  for (int layer = 0; layer < 3; ++layer) {
+    if (layer == 0) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[k][r] = s.b[t.a + 16 * k];
+#pragma unroll
+      for (int i = 0; i < IN; ++i) {
+        const float4 v = ld4(s.x + i * RS + 4 * t.c);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) axpy4(acc[k], s.w1[i * H + t.a + 16 * k], v);
+      }
+    } else {
+      dense(layer == 1 ? s.w2 : s.w3, s.b + layer * H, s.h[layer - 1], t, acc);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r) acc[k][r] = GRAD ? gelu_both(acc[k][r], gp[layer][k][r]) : gelu(acc[k][r]);
+      st4(s.h[layer] + (t.a + 16 * k) * RS + 4 * t.c, acc[k]);
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x < OUT * MLP_ROWS) {
+    const int o = threadIdx.x / MLP_ROWS, r = threadIdx.x % MLP_ROWS;
+    float y = s.b[3 * H + o];
+#pragma unroll 16
+    for (int i = 0; i < H; ++i) y = fmaf(s.w4[o * RS + i], s.h[2][i * RS + r], y);
+    s.y[o * RS + r] = y;
+  }
 }
 
-// dW[o][i] += sum_r D[o][r] A[i][r] and db[o] += sum_r D[o][r] over the CTA's rows.
-__device__ __forceinline__ void weight_grad(const float* D, const float* A, int nout, int nin, int rows,
-                                            float* __restrict__ gW, float* __restrict__ gb) {
-  for (int k = threadIdx.x; k < nout * nin; k += blockDim.x) {
-    const int o = k / nin, i = k % nin;
-    float acc = 0.f;
-    for (int r = 0; r < rows; ++r) acc = fmaf(D[o * RS + r], A[i * RS + r], acc);
-    atomicAdd(&gW[k], acc);
-  }
-  for (int o = threadIdx.x; o < nout; o += blockDim.x) {
-    float acc = 0.f;
-    for (int r = 0; r < rows; ++r) acc += D[o * RS + r];
-    atomicAdd(&gb[o], acc);
-  }
-}
-
-// Delta of a hidden layer for this thread's row: Z[i][r] <- (sum_o W[o][i] D[o][r]) gelu'(Z[i][r]).
-__device__ __forceinline__ void back_row(const float* W, const float* D, int nout, float* Z, int nin, int r) {
-  for (int i = 0; i < nin; ++i) {
-    float acc = 0.f;
-    for (int o = 0; o < nout; ++o) acc = fmaf(W[o * nin + i], D[o * RS + r], acc);
-    Z[i * RS + r] = acc * gelu_grad(Z[i * RS + r]);
-  }
-}
-
-// Gradient of loss = sum (y - t)^2 / (rows_total * 3) accumulated into grad; the
-// summed squared error goes to sse.
-__global__ void __launch_bounds__(MLP_ROWS) k_mlp_backward(const __nv_bfloat16* __restrict__ w16,
-                                                           const float* __restrict__ X, const float* __restrict__ T,
-                                                           int64_t rows, float* __restrict__ grad,
-                                                           double* __restrict__ sse) {
+__global__ void __launch_bounds__(MLP_THREADS, 2) k_mlp_forward(const __nv_bfloat16* __restrict__ w16,
+                                                                const float* __restrict__ X, int64_t rows,
+                                                                float* __restrict__ Y) {
   extern __shared__ __align__(16) unsigned char raw[];
   MlpSmem& s = *reinterpret_cast<MlpSmem*>(raw);
-  __shared__ double red[MLP_ROWS / 32];
-  load_weights(s.w, w16);
-  const int64_t r0 = (int64_t)blockIdx.x * MLP_ROWS;
-  const int nr = rows - r0 < MLP_ROWS ? (int)(rows - r0) : MLP_ROWS;
-  for (int k = threadIdx.x; k < IN * MLP_ROWS; k += blockDim.x) {
-    const int f = k / MLP_ROWS, r = k % MLP_ROWS;
-    s.x[f * RS + r] = r < nr ? X[(r0 + r) * IN + f] : 0.f;
+  load_weights(s, w16);
+  const Block t;
+  const int64_t tiles = (rows + MLP_ROWS - 1) / MLP_ROWS;
+  for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const int64_t r0 = tile * MLP_ROWS;
+    const int nr = rows - r0 < MLP_ROWS ? (int)(rows - r0) : MLP_ROWS;
+    float gp[3][4][4];
+    forward_tile<false>(s, X, r0, nr, t, gp);
+    __syncthreads();
+    for (int k = threadIdx.x; k < nr * OUT; k += MLP_THREADS) Y[r0 * OUT + k] = s.y[(k % OUT) * RS + k / OUT];
   }
-  __syncthreads();
-  float y[OUT];
-  forward_rows(s, nr, y);
-  const int r = threadIdx.x;
+}
+
+// Gradient of loss = sum (y - t)^2 / (rows_total * 3): each CTA walks its tiles with the
+// weight gradients in registers (a 4 x 4 block of each 64 x 64 layer per thread) and
+// writes its sums to partial[blockIdx.x] (k_mlp_reduce adds them); the CTA's summed
+// squared error goes to sse_part[blockIdx.x].
+//
+// What bounds it: FP32 FMA issue.  158 000 rows, 8.25 GFLOP: 2.00 ms with one row per
+// thread of 64-thread CTAs (137 KB of shared memory, two warps per SM) and one atomic
+// per weight and CTA, against 0.28 ms now
+// (41 % of the FMA rate; erff and expf of the activations are a quarter of the instructions).
+__global__ void __launch_bounds__(MLP_THREADS, 2) k_mlp_backward(const __nv_bfloat16* __restrict__ w16,
+                                                                 const float* __restrict__ X,
+                                                                 const float* __restrict__ T, int64_t rows,
+                                                                 float* __restrict__ partial,
+                                                                 double* __restrict__ sse_part) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  MlpSmem& s = *reinterpret_cast<MlpSmem*>(raw);
+  load_weights(s, w16);
+  const Block t;
+  const int tid = threadIdx.x;
   const float scale = 2.f / (float)(rows * OUT);
+  float g2[4][4] = {}, g3[4][4] = {};   // layers 2 and 3
+  float g1[2] = {}, g4 = 0.f;           // layer 1: weights tid and tid + 256; layer 4: weight tid
+  float gb = 0.f;                       // biases: 64 per hidden layer, then the output's
   double e2 = 0.0;
-  for (int o = 0; o < OUT; ++o) {
-    float d = 0.f;
-    if (r < nr) {
-      const float diff = y[o] - T[(r0 + r) * OUT + o];
-      e2 += (double)diff * diff;
-      d = scale * diff;
+  const int64_t tiles = (rows + MLP_ROWS - 1) / MLP_ROWS;
+  for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const int64_t r0 = tile * MLP_ROWS;
+    const int nr = rows - r0 < MLP_ROWS ? (int)(rows - r0) : MLP_ROWS;
+    float gp[3][4][4];
+    forward_tile<true>(s, X, r0, nr, t, gp);
+    // this thread wrote these outputs itself; rows past the end get zero deltas
+    if (tid < OUT * MLP_ROWS) {
+      const int o = tid / MLP_ROWS, r = tid % MLP_ROWS;
+      float d = 0.f;
+      if (r < nr) {
+        const float diff = s.y[o * RS + r] - T[(r0 + r) * OUT + o];
+        e2 += (double)diff * diff;
+        d = scale * diff;
+      }
+      s.y[o * RS + r] = d;
     }
-    s.d4[o * RS + r] = d;
+    __syncthreads();
+    // layer 4, and the deltas of layer 3
+    if (tid < OUT * H) g4 += row_dot(s.y + tid / H * RS, s.h[2] + tid % H * RS);
+    if (tid >= 3 * H && tid < 3 * H + OUT) gb += row_dot(s.y + (tid - 3 * H) * RS, nullptr);
+    float acc[4][4] = {};
+#pragma unroll
+    for (int o = 0; o < OUT; ++o) {
+      const float4 v = ld4(s.y + o * RS + 4 * t.c);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) axpy4(acc[k], s.w4[o * RS + t.a + 16 * k], v);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r) acc[k][r] *= gp[2][k][r];
+      st4(s.d + (t.a + 16 * k) * RS + 4 * t.c, acc[k]);
+    }
+    __syncthreads();
+    // layer 3, and the deltas of layer 2 (into h[2], which nothing reads any more)
+    outer(s.d, s.h[1], t, g3);
+    if (tid >= 2 * H && tid < 3 * H) gb += row_dot(s.d + (tid - 2 * H) * RS, nullptr);
+    dense_t(s.w3, s.d, t, acc);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r) acc[k][r] *= gp[1][k][r];
+      st4(s.h[2] + (t.a + 16 * k) * RS + 4 * t.c, acc[k]);
+    }
+    __syncthreads();
+    // layer 2, and the deltas of layer 1
+    outer(s.h[2], s.h[0], t, g2);
+    if (tid >= H && tid < 2 * H) gb += row_dot(s.h[2] + (tid - H) * RS, nullptr);
+    dense_t(s.w2, s.h[2], t, acc);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r) acc[k][r] *= gp[0][k][r];
+      st4(s.d + (t.a + 16 * k) * RS + 4 * t.c, acc[k]);
+    }
+    __syncthreads();
+    // layer 1
+    if (tid < H) gb += row_dot(s.d + tid * RS, nullptr);
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int k = tid + u * MLP_THREADS;
+      if (k < H * IN) g1[u] += row_dot(s.d + k / IN * RS, s.x + k % IN * RS);
+    }
+    __syncthreads();
   }
-  // rows beyond nr contribute zero deltas; their activations are zeroed too
-  if (r >= nr)
-    for (int l = 0; l < 3; ++l)
-      for (int i = 0; i < H; ++i) s.h[l][i * RS + r] = 0.f;
-  __syncthreads();
-  weight_grad(s.d4, s.h[2], OUT, H, MLP_ROWS, grad + OFF_W4, grad + OFF_B4);
-  __syncthreads();
-  if (r < nr) back_row(s.w + OFF_W4, s.d4, OUT, s.z[2], H, r);
-  else for (int i = 0; i < H; ++i) s.z[2][i * RS + r] = 0.f;
-  __syncthreads();
-  weight_grad(s.z[2], s.h[1], H, H, MLP_ROWS, grad + OFF_W3, grad + OFF_B3);
-  __syncthreads();
-  if (r < nr) back_row(s.w + OFF_W3, s.z[2], H, s.z[1], H, r);
-  else for (int i = 0; i < H; ++i) s.z[1][i * RS + r] = 0.f;
-  __syncthreads();
-  weight_grad(s.z[1], s.h[0], H, H, MLP_ROWS, grad + OFF_W2, grad + OFF_B2);
-  __syncthreads();
-  if (r < nr) back_row(s.w + OFF_W2, s.z[1], H, s.z[0], H, r);
-  else for (int i = 0; i < H; ++i) s.z[0][i * RS + r] = 0.f;
-  __syncthreads();
-  weight_grad(s.z[0], s.x, H, IN, MLP_ROWS, grad + OFF_W1, grad + OFF_B1);
+  float* out = partial + (size_t)blockIdx.x * NP;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+      const int w = (t.a + 16 * k) * H + t.c + 16 * l;
+      out[OFF_W2 + w] = g2[k][l];
+      out[OFF_W3 + w] = g3[k][l];
+    }
+  for (int u = 0; u < 2; ++u)
+    if (tid + u * MLP_THREADS < H * IN) out[OFF_W1 + tid + u * MLP_THREADS] = g1[u];
+  if (tid < OUT * H) out[OFF_W4 + tid] = g4;
+  if (tid < 3 * H + OUT) {
+    const int layer = tid / H;
+    out[(layer == 0 ? OFF_B1 : layer == 1 ? OFF_B2 : layer == 2 ? OFF_B3 : OFF_B4) + tid % H] = gb;
+  }
   // squared error
+  __shared__ double red[MLP_THREADS / 32];
   for (int o = 16; o > 0; o >>= 1) e2 += __shfl_xor_sync(0xffffffffu, e2, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = e2;
+  if ((tid & 31) == 0) red[tid >> 5] = e2;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0;
-    for (int k = 0; k < MLP_ROWS / 32; ++k) t += red[k];
-    atomicAdd(sse, t);
+  if (tid == 0) {
+    double v = 0;
+    for (int k = 0; k < MLP_THREADS / 32; ++k) v += red[k];
+    sse_part[blockIdx.x] = v;
   }
 }
 
-// Adam on the FP32 master weights, refresh of the bfloat16 copy, gradient reset.
-__global__ void k_mlp_adam(float* __restrict__ w, __nv_bfloat16* __restrict__ w16, float* __restrict__ grad,
+// grad[k] (and copy[k]) = sum over the n partial gradients, in one fixed order: 32
+// parameters per CTA, 8 threads each.  The last CTA adds the squared errors.
+__global__ void __launch_bounds__(256) k_mlp_reduce(const float* __restrict__ partial,
+                                                    const double* __restrict__ sse_part, int n,
+                                                    float* __restrict__ grad, float* __restrict__ copy,
+                                                    double* __restrict__ sse, double* __restrict__ sse_copy) {
+  if (blockIdx.x == gridDim.x - 1) {
+    if (threadIdx.x < 32) {
+      double v = 0.0;
+      for (int q = threadIdx.x; q < n; q += 32) v += sse_part[q];
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (threadIdx.x == 0) {
+        *sse = v;
+        if (sse_copy) *sse_copy = v;
+      }
+    }
+    return;
+  }
+  __shared__ float part[8][32];
+  const int p = threadIdx.x & 31, slice = threadIdx.x >> 5, k = blockIdx.x * 32 + p;
+  float v = 0.f;
+  if (k < NP) {
+#pragma unroll 8
+    for (int q = slice; q < n; q += 8) v += partial[(size_t)q * NP + k];
+  }
+  part[slice][p] = v;
+  __syncthreads();
+  if (slice == 0 && k < NP) {
+    for (int q = 1; q < 8; ++q) v += part[q][p];
+    grad[k] = v;
+    if (copy) copy[k] = v;
+  }
+}
+
+// Adam on the FP32 master weights, refresh of the bfloat16 copy.
+__global__ void k_mlp_adam(float* __restrict__ w, __nv_bfloat16* __restrict__ w16, const float* __restrict__ grad,
                            float* __restrict__ m, float* __restrict__ v, float lr, float b1, float b2, float eps,
                            float c1, float c2) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -202,7 +390,6 @@ __global__ void k_mlp_adam(float* __restrict__ w, __nv_bfloat16* __restrict__ w1
   const float wk = w[k] - lr * (mk / c1) / (sqrtf(vk / c2) + eps);
   w[k] = wk;
   w16[k] = __float2bfloat16_rn(wk);
-  grad[k] = 0.f;
 }
 
 // Per-shell features of result rows (layout of ys_measure_multipoles_async) and,
@@ -263,12 +450,16 @@ __global__ void k_mlp_apply(const double* __restrict__ rows, int64_t stride, int
 }  // namespace ys
 
 struct ys_mlp_s {
+  unsigned char* slab = nullptr;  // one allocation; everything down to fcount but the features lies in it
   float* w = nullptr;            // FP32 master weights
   __nv_bfloat16* w16 = nullptr;  // bfloat16 copy used by the kernels
   float* grad = nullptr;
   float* m = nullptr;
   float* v = nullptr;
   double* sse = nullptr;
+  float* partial = nullptr;      // [grid_max][NP] gradients of the CTAs
+  double* sse_part = nullptr;    // [grid_max]
+  int grid_max = 0;              // CTAs that are resident at once
   float* fx = nullptr;           // feature scratch for ys_mlp_correct
   float* fy = nullptr;
   int* fsrc = nullptr;
@@ -287,8 +478,7 @@ ys_status fail(cudaError_t e) {
 }
 
 void free_mlp(ys_mlp* m) {
-  for (void* p : {(void*)m->w, (void*)m->w16, (void*)m->grad, (void*)m->m, (void*)m->v, (void*)m->sse,
-                  (void*)m->fx, (void*)m->fy, (void*)m->fsrc, (void*)m->fcount})
+  for (void* p : {(void*)m->slab, (void*)m->fx, (void*)m->fy, (void*)m->fsrc})
     if (p) cudaFree(p);
   delete m;
 }
@@ -297,6 +487,13 @@ cudaError_t set_attrs() {
   cudaError_t e = cudaFuncSetAttribute(ys::k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes());
   if (!e) e = cudaFuncSetAttribute(ys::k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes());
   return e;
+}
+
+// CTAs of the tile kernels: the tiles shared evenly among at most grid_max.
+unsigned grid_for(const ys_mlp* m, int64_t rows) {
+  const int64_t tiles = (rows + ys::MLP_ROWS - 1) / ys::MLP_ROWS;
+  const int64_t per = (tiles + m->grid_max - 1) / m->grid_max;
+  return (unsigned)((tiles + per - 1) / per);
 }
 
 }  // namespace
@@ -316,12 +513,35 @@ ys_status ys_mlp_create(const float* h_params, ys_mlp** out) {
   if (!m) return YS_ERR_OOM;
   cudaError_t e;
   const size_t n = ys::NP;
-  if ((e = cudaMalloc(&m->w, n * 4)) || (e = cudaMalloc(&m->w16, n * 2)) || (e = cudaMalloc(&m->grad, n * 4)) ||
-      (e = cudaMalloc(&m->m, n * 4)) || (e = cudaMalloc(&m->v, n * 4)) || (e = cudaMalloc(&m->sse, 8)) ||
-      (e = cudaMalloc(&m->fcount, 4))) {
+  int dev = 0, sms = 0;
+  if ((e = cudaGetDevice(&dev)) || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) {
     free_mlp(m);
     return fail(e);
   }
+  m->grid_max = 2 * sms;
+  // one allocation for everything whose size is known
+  size_t bytes = 0;
+  auto part = [&](size_t size) {
+    const size_t at = bytes;
+    bytes += (size + 255) & ~size_t(255);
+    return at;
+  };
+  const size_t at_w = part(n * 4), at_w16 = part(n * 2), at_grad = part(n * 4), at_m = part(n * 4), at_v = part(n * 4),
+               at_sse = part(8), at_count = part(4), at_ssep = part((size_t)m->grid_max * 8),
+               at_partial = part((size_t)m->grid_max * n * 4);
+  if ((e = cudaMalloc(&m->slab, bytes))) {
+    free_mlp(m);
+    return fail(e);
+  }
+  m->w = reinterpret_cast<float*>(m->slab + at_w);
+  m->w16 = reinterpret_cast<__nv_bfloat16*>(m->slab + at_w16);
+  m->grad = reinterpret_cast<float*>(m->slab + at_grad);
+  m->m = reinterpret_cast<float*>(m->slab + at_m);
+  m->v = reinterpret_cast<float*>(m->slab + at_v);
+  m->sse = reinterpret_cast<double*>(m->slab + at_sse);
+  m->fcount = reinterpret_cast<int*>(m->slab + at_count);
+  m->sse_part = reinterpret_cast<double*>(m->slab + at_ssep);
+  m->partial = reinterpret_cast<float*>(m->slab + at_partial);
   std::vector<__nv_bfloat16> h16(n);
   for (size_t k = 0; k < n; ++k) h16[k] = __float2bfloat16_rn(h_params[k]);
   if ((e = cudaMemcpy(m->w, h_params, n * 4, cudaMemcpyHostToDevice)) ||
@@ -363,8 +583,7 @@ ys_status ys_mlp_set_state(ys_mlp* m, const float* h_params, const float* h_m, c
 ys_status ys_mlp_forward(ys_mlp* m, const float* d_x, int64_t rows, float* d_y, void* stream) {
   if (!m || rows < 0 || (rows > 0 && (!d_x || !d_y))) return YS_ERR_ARG;
   if (rows == 0) return YS_OK;
-  const int64_t blocks = (rows + ys::MLP_ROWS - 1) / ys::MLP_ROWS;
-  ys::k_mlp_forward<<<(unsigned)blocks, ys::MLP_ROWS, smem_bytes(), static_cast<cudaStream_t>(stream)>>>(
+  ys::k_mlp_forward<<<grid_for(m, rows), ys::MLP_THREADS, smem_bytes(), static_cast<cudaStream_t>(stream)>>>(
       m->w16, d_x, rows, d_y);
   cudaError_t e = cudaGetLastError();
   return e ? fail(e) : YS_OK;
@@ -375,12 +594,12 @@ ys_status ys_mlp_gradient(ys_mlp* m, const float* d_x, const float* d_t, int64_t
   if (!m || rows <= 0 || !d_x || !d_t) return YS_ERR_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t e;
-  if ((e = cudaMemsetAsync(m->grad, 0, ys::NP * 4, st)) || (e = cudaMemsetAsync(m->sse, 0, 8, st))) return fail(e);
-  const int64_t blocks = (rows + ys::MLP_ROWS - 1) / ys::MLP_ROWS;
-  ys::k_mlp_backward<<<(unsigned)blocks, ys::MLP_ROWS, smem_bytes(), st>>>(m->w16, d_x, d_t, rows, m->grad, m->sse);
+  const unsigned grid = grid_for(m, rows);
+  ys::k_mlp_backward<<<grid, ys::MLP_THREADS, smem_bytes(), st>>>(m->w16, d_x, d_t, rows, m->partial, m->sse_part);
   if ((e = cudaGetLastError())) return fail(e);
-  if (d_grad && (e = cudaMemcpyAsync(d_grad, m->grad, ys::NP * 4, cudaMemcpyDeviceToDevice, st))) return fail(e);
-  if (d_loss && (e = cudaMemcpyAsync(d_loss, m->sse, 8, cudaMemcpyDeviceToDevice, st))) return fail(e);
+  ys::k_mlp_reduce<<<(ys::NP + 31) / 32 + 1, 256, 0, st>>>(m->partial, m->sse_part, (int)grid, m->grad, d_grad, m->sse,
+                                                           d_loss);
+  if ((e = cudaGetLastError())) return fail(e);
   return YS_OK;
 }
 
