@@ -13,13 +13,23 @@
 // One more complex sum per mode, with the top hat Theta(|mu| <= 1/2) in place of the
 // Legendre weight, gives the wedges by their definition (Sec. 5, Eqs. 14-15).
 //
-// Layout: one thread per mode, with the mode's complex sums in registers; points
-// stream through shared memory in chunks that every thread reads as broadcasts.
-// Positions are 32-bit fixed-point fractions of the box, u = (x - box_min) / L, so
-// the phase k.x = 2 pi m.u is taken mod one turn exactly by integer multiply-adds;
-// only the final angle in [-pi, pi) is rounded.  Each thread's sums are compensated
-// float (TwoSum per add); CTAs that split the points add their sums into FP64
-// per-mode accumulators, and a second kernel forms the shell sums in FP64.
+// Layout: one thread per group of SG_GROUP modes with neighbouring m_z, their complex
+// sums in registers; points stream through shared memory in chunks that every thread
+// reads as broadcasts.  Positions are 32-bit fixed-point fractions of the box,
+// u = (x - box_min) / L, so the phase k.x = 2 pi m.u is taken mod one turn exactly by
+// integer multiply-adds; only the final angle in [-pi, pi) is rounded.  The group's
+// middle mode takes sine and cosine of its phase, the others multiply by the point's
+// e^{-2 pi i j u_z}, j = +-1, +-2, formed once per point the same way.  SG_BLOCK terms of
+// a sum are added in float, and the block's sum goes into a compensated float sum
+// (TwoSum); CTAs that split the points add their sums into FP64 per-mode accumulators,
+// and a second kernel forms the shell sums in FP64.
+//
+// What bounds the mode kernel: FP32 issue, about 35 instructions per mode and point at
+// l_max = 4 (105 with one sincospif and six compensated adds per mode and point).  The sums
+// carry (m . r_hat)^n, normalised in FP64 afterwards: with k_hat in float its rounding was
+// common to all points.  Against FP64, over eight catalogues: P_2 and P_4 are off by 1e-8
+// to 2e-7 (7e-8 to 9e-7 before), P_0 by 2e-9 to 9e-9 (1e-9 to 5e-9 before).
+// 68 000 modes of a 64^3 lattice, 120 000 points: 26.9 -> 9.8 ms a call.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -33,24 +43,32 @@
 namespace ys {
 namespace {
 
-constexpr int SG_THREADS = 256;
+constexpr int SG_THREADS = 128;
 constexpr int SG_CHUNK = 256;  // points per shared-memory chunk
+constexpr int SG_GROUP = 5;    // modes per thread (neighbouring m_z)
+constexpr int SG_BLOCK = 4;    // points per block of plain sums
 
 // Components of the per-mode sums: A_0, A_2, A_4, A_6 and the top-hat sum B_perp.
 enum { C_A0 = 0, C_A2 = 1, C_A4 = 2, C_A6 = 3, C_BP = 4, C_COUNT = 5 };
 
-struct SgPoint {
+struct __align__(16) SgPoint {
   uint32_t u[3];  // position as a fraction of the box, 2^-32 units
   float sw;       // signed weight
   float rh[3];    // r_hat (0 at r = 0)
   float pad;
+  float2 w1, w2;  // e^{-2 pi i u_z}, e^{-4 pi i u_z}
 };
 
 struct SgMode {
   short m[3];     // integer frequency
   short bin;      // shell
-  float khat[3];
   float w;        // Hermitian weight (1 or 2)
+};
+
+// Up to SG_GROUP modes (m_x, m_y, m_z .. m_z + count - 1), entries first .. of the mode list.
+struct SgGroup {
+  short mx, my, mz, count;
+  int first;
 };
 
 __device__ __forceinline__ float two_sum_err(float a, float b) {
@@ -106,6 +124,13 @@ __device__ __forceinline__ void unit3(double x, double y, double z, float (&o)[3
   o[2] = (float)(z * inv);
 }
 
+// The phase of `turn` (units of 2^-32 turns) as e^{-2 pi i turn}.
+__device__ __forceinline__ float2 cis_minus(uint32_t turn) {
+  float sn, cs;
+  sincospif((float)(int32_t)turn * 4.656612873077393e-10f, &sn, &cs);  // angle / pi in [-1, 1)
+  return make_float2(cs, -sn);
+}
+
 // Catalogue particles as points: galaxies +w, randoms -alpha w.
 __global__ void k_sg_points_cat(const float* __restrict__ x, const float* __restrict__ y,
                                 const float* __restrict__ z, const float* __restrict__ w, int64_t n, int is_ran,
@@ -123,6 +148,8 @@ __global__ void k_sg_points_cat(const float* __restrict__ x, const float* __rest
   q.sw = (float)(sgn * (w ? (double)w[i] : 1.0));
   unit3(px - ox, py - oy, pz - oz, q.rh);
   q.pad = 0.f;
+  q.w1 = cis_minus(q.u[2]);
+  q.w2 = cis_minus(2u * q.u[2]);
   out[i] = q;
 }
 
@@ -146,77 +173,121 @@ __global__ void k_sg_points_mesh(const float* __restrict__ mesh, int n, int j, i
   q.sw = f * scale;
   unit3(rel_x0 + (ix + s) * H, rel_y0 + (iy + s) * H, rel_z0 + (iz + s) * H, q.rh);
   q.pad = 0.f;
+  q.w1 = cis_minus(q.u[2]);
+  q.w2 = cis_minus(2u * q.u[2]);
   out[atomicAdd(count, 1u)] = q;
 }
 
-// Per-mode sums over the points [p_lo, p_hi) of this CTA's split; FP64 atomics into
+__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
+  return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+}
+
+// Per-mode sums over the points of this CTA's split (blockIdx.y); FP64 atomics into
 // acc[C_COUNT][nmodes] (interleaved re, im).
 template <int ELL, bool WEDGE>
-__global__ void __launch_bounds__(SG_THREADS) k_sg_modes(const SgMode* __restrict__ modes, int nmodes,
+__global__ void __launch_bounds__(SG_THREADS) k_sg_modes(const SgGroup* __restrict__ groups, int ngroups, int nmodes,
                                                           const SgPoint* __restrict__ pts,
                                                           const unsigned* __restrict__ npts_dev, int64_t npts_host,
                                                           int splits, double* __restrict__ acc) {
   __shared__ SgPoint s_pts[SG_CHUNK];
-  const int mi = blockIdx.x * SG_THREADS + threadIdx.x;
-  const bool active = mi < nmodes;
+  const int gi = blockIdx.x * SG_THREADS + threadIdx.x;
+  const bool active = gi < ngroups;
   const int64_t npts = npts_dev ? (int64_t)*npts_dev : npts_host;
   const int64_t per = (npts + splits - 1) / splits;
   const int64_t p_lo = std::min<int64_t>(npts, per * blockIdx.y), p_hi = std::min<int64_t>(npts, p_lo + per);
-  int mx = 0, my = 0, mz = 0;
-  float kx = 0.f, ky = 0.f, kz = 0.f;
-  if (active) {
-    const SgMode md = modes[mi];
-    mx = md.m[0];
-    my = md.m[1];
-    mz = md.m[2];
-    kx = md.khat[0];
-    ky = md.khat[1];
-    kz = md.khat[2];
-  }
-  constexpr int NC = (ELL >= 6 ? 4 : ELL / 2 + 1) + (WEDGE ? 1 : 0);
-  float sre[NC], sim[NC], cre[NC], cim[NC];
+  SgGroup g{};
+  if (active) g = groups[gi];
+  const int mid = g.mz + SG_GROUP / 2;
+  const float fx = g.mx, fy = g.my;
+  // The sums carry (m . r_hat)^n: the mode's 1 / |m|^n is applied in FP64 (k_sg_shells).
+  // The top hat, which jumps at |mu| = 1/2, takes mu from k_hat's components.
+  [[maybe_unused]] float kh[WEDGE ? SG_GROUP : 1][3];
+  if constexpr (WEDGE) {
 #pragma unroll
-  for (int c = 0; c < NC; ++c) sre[c] = sim[c] = cre[c] = cim[c] = 0.f;
+    for (int j = 0; j < SG_GROUP; ++j) {
+      const int mz = g.mz + j, n2 = g.mx * g.mx + g.my * g.my + mz * mz;
+      const double inv = n2 > 0 ? 1.0 / sqrt((double)n2) : 0.0;
+      kh[j][0] = (float)(g.mx * inv);
+      kh[j][1] = (float)(g.my * inv);
+      kh[j][2] = (float)(mz * inv);
+    }
+  }
+  constexpr int NM = ELL >= 6 ? 4 : ELL / 2 + 1;  // A_0, A_2, ..
+  constexpr int NC = NM + (WEDGE ? 1 : 0);
+  float sre[SG_GROUP][NC], sim[SG_GROUP][NC], cre[SG_GROUP][NC], cim[SG_GROUP][NC];
+#pragma unroll
+  for (int j = 0; j < SG_GROUP; ++j)
+#pragma unroll
+    for (int c = 0; c < NC; ++c) sre[j][c] = sim[j][c] = cre[j][c] = cim[j][c] = 0.f;
   for (int64_t base = p_lo; base < p_hi; base += SG_CHUNK) {
     const int cnt = (int)std::min<int64_t>(SG_CHUNK, p_hi - base);
     __syncthreads();
-    if (threadIdx.x < cnt) s_pts[threadIdx.x] = pts[base + threadIdx.x];
+    // points past the end carry no weight
+    for (int i = threadIdx.x; i < SG_CHUNK; i += SG_THREADS) s_pts[i] = i < cnt ? pts[base + i] : SgPoint{};
     __syncthreads();
     if (!active) continue;
-    for (int j = 0; j < cnt; ++j) {
-      const SgPoint q = s_pts[j];
-      // one turn = 2^32: the phase m.u mod 1 is exact in wrapping integer arithmetic
-      const uint32_t turn = (uint32_t)mx * q.u[0] + (uint32_t)my * q.u[1] + (uint32_t)mz * q.u[2];
-      float sn, cs;
-      sincospif((float)(int32_t)turn * 4.656612873077393e-10f, &sn, &cs);  // angle / pi in [-1, 1)
-      const float tre = q.sw * cs, tim = -q.sw * sn;                        // s w e^{-i k.x}
-      add_comp(sre[0], cre[0], tre);
-      add_comp(sim[0], cim[0], tim);
-      if constexpr (ELL >= 2 || WEDGE) {
-        const float mu = fmaf(kx, q.rh[0], fmaf(ky, q.rh[1], kz * q.rh[2]));
-        const float mu2 = mu * mu;
-        float f = mu2;
+#pragma unroll 1
+    for (int i = 0; i < cnt; i += SG_BLOCK) {
+      float2 e[SG_BLOCK];  // s w e^{-i k.x} of the middle mode
+      float d[SG_BLOCK];   // m_x r_hat_x + m_y r_hat_y
 #pragma unroll
-        for (int c = 1; c <= (ELL >= 6 ? 3 : ELL / 2); ++c) {
-          add_comp(sre[c], cre[c], f * tre);
-          add_comp(sim[c], cim[c], f * tim);
-          f *= mu2;
+      for (int b = 0; b < SG_BLOCK; ++b) {
+        const SgPoint& q = s_pts[i + b];
+        // one turn = 2^32: the phase m.u mod 1 is exact in wrapping integer arithmetic
+        const float2 c = cis_minus((uint32_t)(int)g.mx * q.u[0] + (uint32_t)(int)g.my * q.u[1] + (uint32_t)mid * q.u[2]);
+        e[b] = make_float2(q.sw * c.x, q.sw * c.y);
+        d[b] = fmaf(fx, q.rh[0], fy * q.rh[1]);
+      }
+#pragma unroll
+      for (int j = 0; j < SG_GROUP; ++j) {
+        float pr[NC], pi[NC];  // the block's plain sums
+#pragma unroll
+        for (int b = 0; b < SG_BLOCK; ++b) {
+          const SgPoint& q = s_pts[i + b];
+          const int o = j - SG_GROUP / 2;
+          float2 t = e[b];
+          if (o != 0) {
+            const float2 w = (o == 1 || o == -1) ? q.w1 : q.w2;
+            t = cmul(t, o > 0 ? w : make_float2(w.x, -w.y));
+          }
+          pr[0] = b == 0 ? t.x : pr[0] + t.x;
+          pi[0] = b == 0 ? t.y : pi[0] + t.y;
+          if constexpr (NC > 1) {
+            const float md = fmaf((float)(g.mz + j), q.rh[2], d[b]), md2 = md * md;  // m . r_hat
+            float f = md2;
+#pragma unroll
+            for (int c = 1; c < NM; ++c) {
+              pr[c] = b == 0 ? f * t.x : fmaf(f, t.x, pr[c]);
+              pi[c] = b == 0 ? f * t.y : fmaf(f, t.y, pi[c]);
+              f *= md2;
+            }
+            if constexpr (WEDGE) {
+              const float mu = fmaf(kh[j][0], q.rh[0], fmaf(kh[j][1], q.rh[1], kh[j][2] * q.rh[2]));
+              const bool in = fabsf(mu) <= 0.5f;
+              pr[NC - 1] = (b == 0 ? 0.f : pr[NC - 1]) + (in ? t.x : 0.f);
+              pi[NC - 1] = (b == 0 ? 0.f : pi[NC - 1]) + (in ? t.y : 0.f);
+            }
+          }
         }
-        if constexpr (WEDGE) {
-          const float t = fabsf(mu) <= 0.5f ? 1.f : 0.f;
-          add_comp(sre[NC - 1], cre[NC - 1], t * tre);
-          add_comp(sim[NC - 1], cim[NC - 1], t * tim);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          add_comp(sre[j][c], cre[j][c], pr[c]);
+          add_comp(sim[j][c], cim[j][c], pi[c]);
         }
       }
     }
   }
   if (!active) return;
 #pragma unroll
-  for (int c = 0; c < NC; ++c) {
-    const int comp = (WEDGE && c == NC - 1) ? C_BP : c;
-    double* a = acc + ((size_t)comp * nmodes + mi) * 2;
-    atomicAdd(a, (double)sre[c] + (double)cre[c]);
-    atomicAdd(a + 1, (double)sim[c] + (double)cim[c]);
+  for (int j = 0; j < SG_GROUP; ++j) {
+    if (j >= g.count) break;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const int comp = (WEDGE && c == NC - 1) ? C_BP : c;
+      double* a = acc + ((size_t)comp * nmodes + g.first + j) * 2;
+      atomicAdd(a, (double)sre[j][c] + (double)cre[j][c]);
+      atomicAdd(a + 1, (double)sim[j][c] + (double)cim[j][c]);
+    }
   }
 }
 
@@ -238,12 +309,15 @@ __global__ void k_sg_shells(const SgMode* __restrict__ modes, int nmodes, const 
   }
   const double* a0 = acc + (size_t)mi * 2;
   const double r0 = a0[0] * cw, i0 = a0[1] * cw;
+  const double inv_n2 = 1.0 / (double)(md.m[0] * md.m[0] + md.m[1] * md.m[1] + md.m[2] * md.m[2]);
+  double norm = 1.0;  // 1 / |m|^(2 s)
   for (int s = 0; s < nmain + (wedge ? 1 : 0); ++s) {
     const int comp = s < nmain ? s : C_BP;
     const int slot = s < nmain ? s : 4;
     const double* as = acc + ((size_t)comp * nmodes + mi) * 2;
-    const double v = md.w * (r0 * as[0] * cw + i0 * as[1] * cw);
+    const double v = md.w * (s < nmain ? norm : 1.0) * (r0 * as[0] * cw + i0 * as[1] * cw);
     atomicAdd(&shell_acc[(size_t)slot * nbins + md.bin], v);
+    norm *= inv_n2;
   }
 }
 
@@ -293,6 +367,7 @@ __global__ void k_sg_finalize(const double* __restrict__ sacc, const double* __r
 
 struct ModeTable {
   std::vector<SgMode> modes;
+  std::vector<SgGroup> groups;
   std::vector<double> shell;  // [2][nbins]: mode count, sum |k|
 };
 
@@ -305,30 +380,43 @@ ModeTable build_modes(const ys_config& c) {
   const double kmax = std::min(knyq, c.k_min + c.dk * c.n_bins);
   const int mr = std::min(n / 2, (int)std::ceil(kmax / kf) + 1);
   t.shell.assign(2 * (size_t)c.n_bins, 0.0);
-  for (int mx = -mr; mx <= mr; ++mx)
-    for (int my = -mr; my <= mr; ++my)
-      for (int mz = 0; mz <= mr; ++mz) {
-        if (mx < -n / 2 || mx >= n / 2 || my < -n / 2 || my >= n / 2 || mz > n / 2) continue;
-        const int n2 = mx * mx + my * my + mz * mz;
-        if (n2 == 0) continue;
-        const double km = kf * std::sqrt((double)n2);
-        if (!(km < knyq)) continue;
-        const double b = std::floor((km - c.k_min) / c.dk);
-        if (!(b >= 0 && b < c.n_bins)) continue;
+  // shell (-1: none) and |k| of every |m|^2 up to the largest that can fall in one
+  const int n2_max = mr * mr;
+  std::vector<int> shell(n2_max + 1, -1);
+  std::vector<double> k_of(n2_max + 1, 0.0);
+  for (int n2 = 1; n2 <= n2_max; ++n2) {
+    const double km = kf * std::sqrt((double)n2);
+    if (!(km < knyq)) continue;
+    const double b = std::floor((km - c.k_min) / c.dk);
+    if (!(b >= 0 && b < c.n_bins)) continue;
+    shell[n2] = (int)b;
+    k_of[n2] = km;
+  }
+  const int hi = std::min(mr, n / 2 - 1);  // m_x, m_y in [-n/2, n/2)
+  for (int mx = -mr; mx <= hi; ++mx)
+    for (int my = -mr; my <= hi; ++my) {
+      const int xy2 = mx * mx + my * my;
+      for (int mz = 0; mz <= mr && xy2 + mz * mz <= n2_max; ++mz) {
+        const int n2 = xy2 + mz * mz;
+        if (shell[n2] < 0) continue;
         SgMode md;
         md.m[0] = (short)mx;
         md.m[1] = (short)my;
         md.m[2] = (short)mz;
-        md.bin = (short)b;
-        const double inv = 1.0 / std::sqrt((double)n2);
-        md.khat[0] = (float)(mx * inv);
-        md.khat[1] = (float)(my * inv);
-        md.khat[2] = (float)(mz * inv);
+        md.bin = (short)shell[n2];
         md.w = (mz > 0 && mz < n / 2) ? 2.f : 1.f;
+        // modes of one (m_x, m_y) with consecutive m_z share a group
+        SgGroup* g = t.groups.empty() ? nullptr : &t.groups.back();
+        if (g && g->mx == mx && g->my == my && g->mz + g->count == mz && g->count < SG_GROUP) {
+          ++g->count;
+        } else {
+          t.groups.push_back({(short)mx, (short)my, (short)mz, 1, (int)t.modes.size()});
+        }
         t.modes.push_back(md);
-        t.shell[(size_t)b] += md.w;
-        t.shell[(size_t)c.n_bins + (size_t)b] += md.w * km;
+        t.shell[(size_t)md.bin] += md.w;
+        t.shell[(size_t)c.n_bins + (size_t)md.bin] += md.w * k_of[n2];
       }
+    }
   return t;
 }
 
@@ -355,35 +443,41 @@ ys_status fail(cudaError_t e) {
   return e == cudaErrorMemoryAllocation ? YS_ERR_OOM : YS_ERR_CUDA;
 }
 
+// The modes' groups on the device.
+struct ModeGroups {
+  const SgGroup* groups;
+  int ngroups, nmodes;
+};
+
 template <int ELL, bool WEDGE>
-cudaError_t launch_modes(const SgMode* modes, int nmodes, const SgPoint* pts, const unsigned* npts_dev,
+cudaError_t launch_modes(const ModeGroups& mg, const SgPoint* pts, const unsigned* npts_dev,
                          int64_t npts_host, double* acc, cudaStream_t st) {
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (!e) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e) return e;
-  const int mblocks = (nmodes + SG_THREADS - 1) / SG_THREADS;
+  const int mblocks = (mg.ngroups + SG_THREADS - 1) / SG_THREADS;
   // split the points so that the grid fills the GPU a few times over
-  const int64_t want = (int64_t)sms * 8;
+  const int64_t want = (int64_t)sms * 16;
   int splits = (int)std::max<int64_t>(1, std::min<int64_t>(1024, (want + mblocks - 1) / mblocks));
   const int64_t np_bound = npts_dev ? INT64_MAX : npts_host;
   splits = (int)std::max<int64_t>(1, std::min<int64_t>(splits, (np_bound + SG_CHUNK - 1) / SG_CHUNK));
   dim3 grid(mblocks, splits);
-  k_sg_modes<ELL, WEDGE><<<grid, SG_THREADS, 0, st>>>(modes, nmodes, pts, npts_dev, npts_host, splits, acc);
+  k_sg_modes<ELL, WEDGE><<<grid, SG_THREADS, 0, st>>>(mg.groups, mg.ngroups, mg.nmodes, pts, npts_dev, npts_host, splits, acc);
   return cudaGetLastError();
 }
 
-cudaError_t run_modes(int ell, bool wedge, const SgMode* modes, int nmodes, const SgPoint* pts,
+cudaError_t run_modes(int ell, bool wedge, const ModeGroups& mg, const SgPoint* pts,
                       const unsigned* npts_dev, int64_t npts_host, double* acc, cudaStream_t st) {
   switch (ell * 2 + (wedge ? 1 : 0)) {
-    case 0: return launch_modes<0, false>(modes, nmodes, pts, npts_dev, npts_host, acc, st);
-    case 1: return launch_modes<0, true>(modes, nmodes, pts, npts_dev, npts_host, acc, st);
-    case 4: return launch_modes<2, false>(modes, nmodes, pts, npts_dev, npts_host, acc, st);
-    case 5: return launch_modes<2, true>(modes, nmodes, pts, npts_dev, npts_host, acc, st);
-    case 8: return launch_modes<4, false>(modes, nmodes, pts, npts_dev, npts_host, acc, st);
-    case 9: return launch_modes<4, true>(modes, nmodes, pts, npts_dev, npts_host, acc, st);
-    case 12: return launch_modes<6, false>(modes, nmodes, pts, npts_dev, npts_host, acc, st);
-    default: return launch_modes<6, true>(modes, nmodes, pts, npts_dev, npts_host, acc, st);
+    case 0: return launch_modes<0, false>(mg, pts, npts_dev, npts_host, acc, st);
+    case 1: return launch_modes<0, true>(mg, pts, npts_dev, npts_host, acc, st);
+    case 4: return launch_modes<2, false>(mg, pts, npts_dev, npts_host, acc, st);
+    case 5: return launch_modes<2, true>(mg, pts, npts_dev, npts_host, acc, st);
+    case 8: return launch_modes<4, false>(mg, pts, npts_dev, npts_host, acc, st);
+    case 9: return launch_modes<4, true>(mg, pts, npts_dev, npts_host, acc, st);
+    case 12: return launch_modes<6, false>(mg, pts, npts_dev, npts_host, acc, st);
+    default: return launch_modes<6, true>(mg, pts, npts_dev, npts_host, acc, st);
   }
 }
 
@@ -433,15 +527,19 @@ extern "C" ys_status ys_sum_gal(const ys_config* cfg, const ys_catalog* gal, con
   const bool wedge = d_wedges != nullptr;
   Scratch sc;
   SgMode* d_modes = nullptr;
+  SgGroup* d_groups = nullptr;
   double *d_acc = nullptr, *d_sums = nullptr;
   SgPoint* d_pts = nullptr;
   const int64_t npts = gal->n + ran->n;
   cudaError_t e;
-  if ((e = sc.get(d_modes, (size_t)nmodes)) || (e = sc.get(d_acc, (size_t)C_COUNT * 2 * std::max(1, nmodes))) ||
+  if ((e = sc.get(d_modes, (size_t)nmodes)) || (e = sc.get(d_groups, mt.groups.size())) || (e = sc.get(d_acc, (size_t)C_COUNT * 2 * std::max(1, nmodes))) ||
       (e = sc.get(d_sums, (size_t)SUM_COUNT)) || (e = sc.get(d_pts, (size_t)std::max<int64_t>(1, npts))))
     return fail(e);
-  if (nmodes > 0 && (e = cudaMemcpyAsync(d_modes, mt.modes.data(), sizeof(SgMode) * nmodes, cudaMemcpyHostToDevice, st)))
+  if (nmodes > 0 &&
+      ((e = cudaMemcpyAsync(d_modes, mt.modes.data(), sizeof(SgMode) * nmodes, cudaMemcpyHostToDevice, st)) ||
+       (e = cudaMemcpyAsync(d_groups, mt.groups.data(), sizeof(SgGroup) * mt.groups.size(), cudaMemcpyHostToDevice, st))))
     return fail(e);
+  const ModeGroups mg{d_groups, (int)mt.groups.size(), nmodes};
   if ((e = cudaMemsetAsync(d_acc, 0, sizeof(double) * C_COUNT * 2 * std::max(1, nmodes), st)) ||
       (e = cudaMemsetAsync(d_sums, 0, sizeof(double) * SUM_COUNT, st)))
     return fail(e);
@@ -463,7 +561,7 @@ extern "C" ys_status ys_sum_gal(const ys_config* cfg, const ys_catalog* gal, con
     }
     off += q.n;
   }
-  if (nmodes > 0 && npts > 0 && (e = run_modes(c.ell_max, wedge, d_modes, nmodes, d_pts, nullptr, npts, d_acc, st)))
+  if (nmodes > 0 && npts > 0 && (e = run_modes(c.ell_max, wedge, mg, d_pts, nullptr, npts, d_acc, st)))
     return fail(e);
   return finish(mt, d_modes, d_acc, nullptr, c.n_mesh, d_sums, c.alpha, c.n_bins, c.ell_max, wedge, d_out, d_wedges,
                 sc, st);
@@ -484,15 +582,19 @@ extern "C" ys_status ys_sum_grid(ys_plan* plan, double* d_out, double* d_wedges)
   const int64_t chunk = std::min<int64_t>(n3, (int64_t)1 << 26);
   Scratch sc;
   SgMode* d_modes = nullptr;
+  SgGroup* d_groups = nullptr;
   double* d_acc = nullptr;
   SgPoint* d_pts = nullptr;
   unsigned* d_count = nullptr;
   cudaError_t e;
-  if ((e = sc.get(d_modes, (size_t)nmodes)) || (e = sc.get(d_acc, (size_t)C_COUNT * 2 * std::max(1, nmodes))) ||
+  if ((e = sc.get(d_modes, (size_t)nmodes)) || (e = sc.get(d_groups, mt.groups.size())) || (e = sc.get(d_acc, (size_t)C_COUNT * 2 * std::max(1, nmodes))) ||
       (e = sc.get(d_pts, (size_t)chunk)) || (e = sc.get(d_count, 1)))
     return fail(e);
-  if (nmodes > 0 && (e = cudaMemcpyAsync(d_modes, mt.modes.data(), sizeof(SgMode) * nmodes, cudaMemcpyHostToDevice, st)))
+  if (nmodes > 0 &&
+      ((e = cudaMemcpyAsync(d_modes, mt.modes.data(), sizeof(SgMode) * nmodes, cudaMemcpyHostToDevice, st)) ||
+       (e = cudaMemcpyAsync(d_groups, mt.groups.data(), sizeof(SgGroup) * mt.groups.size(), cudaMemcpyHostToDevice, st))))
     return fail(e);
+  const ModeGroups mg{d_groups, (int)mt.groups.size(), nmodes};
   if ((e = cudaMemsetAsync(d_acc, 0, sizeof(double) * C_COUNT * 2 * std::max(1, nmodes), st))) return fail(e);
   // The interlaced pair is averaged: each mesh's nodes carry F / 2.
   const float scale = p.m == 2 ? 0.5f : 1.f;
@@ -504,7 +606,7 @@ extern "C" ys_status ys_sum_grid(ys_plan* plan, double* d_out, double* d_wedges)
           p.d_mesh + j * n3, p.n, j, first, cnt, c.box_min[0] - c.observer[0], c.box_min[1] - c.observer[1],
           c.box_min[2] - c.observer[2], p.H, scale, d_count, d_pts);
       if ((e = cudaGetLastError())) return fail(e);
-      if ((e = run_modes(c.ell_max, wedge, d_modes, nmodes, d_pts, d_count, cnt, d_acc, st))) return fail(e);
+      if ((e = run_modes(c.ell_max, wedge, mg, d_pts, d_count, cnt, d_acc, st))) return fail(e);
     }
   return finish(mt, d_modes, d_acc, c.compensate ? p.d_invw : nullptr, p.n, p.d_sums, c.alpha, c.n_bins, c.ell_max,
                 wedge, d_out, d_wedges, sc, st);
