@@ -130,8 +130,8 @@ size_t x_smem_for(int n, int nbins, int nwb, int ell) {
   }
 }
 
-// 2D tensor map over the grouped transforms d_g: rows = (mesh, group, x), columns =
-// 2 np_pad floats (np_pad float2 pencils); box = (2 P floats, x_box_rows(N) rows, a
+// 2D tensor map over the grouped transforms d_g: rows = (mesh, group, pencil block, x),
+// columns = 2 gw floats (gw float2 pencils); box = (2 P floats, x_box_rows(N) rows, a
 // divisor of N of at most 256).
 ys_status make_gmap(Plan& p) {
   void* fn = nullptr;
@@ -146,8 +146,8 @@ ys_status make_gmap(Plan& p) {
                                               CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
                                               CUtensorMapFloatOOBfill)>(fn);
   const int P = p.x_pencils;
-  const cuuint64_t dims[2] = {(cuuint64_t)2 * p.np_pad, (cuuint64_t)p.m * p.ng * p.n};
-  const cuuint64_t strides[1] = {(cuuint64_t)2 * p.np_pad * sizeof(float)};
+  const cuuint64_t dims[2] = {(cuuint64_t)2 * p.gw, (cuuint64_t)p.m * p.ng * p.ngb * p.n};
+  const cuuint64_t strides[1] = {(cuuint64_t)2 * p.gw * sizeof(float)};
   const cuuint32_t box[2] = {(cuuint32_t)(2 * P), (cuuint32_t)x_box_rows(p.n)};
   const cuuint32_t estr[2] = {1, 1};
   CUresult r = encode(&p.gmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, p.d_g, dims, strides, box, estr,
@@ -226,6 +226,8 @@ ys_status build_tables(Plan& p) {
   p.x_pencils = k3_pencils(n);
   p.np_pad = std::max(xp, (p.np + xp - 1) / xp * xp);
   while ((int)pen.size() < p.np_pad) pen.push_back(make_short2(0, -1));
+  p.gw = std::min(p.np_pad, GROUP_BLOCK);
+  p.ngb = (p.np_pad + p.gw - 1) / p.gw;
   // mode count and sum |k| per shell (half grid, weight 2 for 0 < k_z < n/2)
   std::vector<double> shell(2 * c.n_bins, 0.0);
   for (int kz = 0; kz < nzc; ++kz) {
@@ -593,7 +595,7 @@ ys_status ys_plan_create(const ys_config* cfg, ys_plan** out) {
   const size_t slot = (size_t)p.nf * std::max(1, p.nzc) * n;
   if ((e = ys::dalloc(p, p.d_mesh, p.m * n3)) || (e = ys::dalloc(p, p.d_z, slot * p.ring_slots_cap)) ||
       (e = ys::dalloc(p, p.d_sync, (size_t)2 * p.m * n + 2)) ||
-      (e = ys::dalloc(p, p.d_g, (size_t)p.m * p.ng * n * std::max(1, p.np_pad))) ||
+      (e = ys::dalloc(p, p.d_g, (size_t)p.m * p.ng * p.ngb * n * p.gw)) ||
       (e = ys::dalloc(p, p.d_acc, (size_t)4 * c.n_bins)) || (e = ys::dalloc(p, p.d_sums, (size_t)ys::SUM_COUNT)) ||
       (e = ys::dalloc(p, p.d_result, (size_t)p.row_len)) ||
       (e = ys::dalloc(p, p.d_tile_count, (size_t)p.ntiles_max)) ||

@@ -72,7 +72,8 @@ cudaError_t run_yz(Plan* const* lanes, int W) {
     prm.ticket = p.d_sync + 2 * p.m * N;
     prm.err = p.d_sync + 2 * p.m * N + 1;
     prm.nzc = p.nzc;
-    prm.np = p.np_pad;
+    prm.gw = p.gw;
+    prm.ngb = p.ngb;
     prm.m = p.m;
     prm.S = p.ring_slots;
     prm.D = p.ring_lead;
@@ -149,7 +150,7 @@ cudaError_t run_x_p(Plan* const* lanes, int W) {
   const int resident = std::max(1, per) * sms;
   const int grid = std::max(1, std::min(npb, (resident + W - 1) / W));
   LaunchScope ls(p, 6);
-  k_x_combine<N, ELL, M, PX><<<dim3(grid, W), XC::THREADS, smem, p.stream>>>(pm, p.np_pad, p.d_pencil, p.d_tw, p.d_invw,
+  k_x_combine<N, ELL, M, PX><<<dim3(grid, W), XC::THREADS, smem, p.stream>>>(pm, p.np_pad, p.ngb, p.d_pencil, p.d_tw, p.d_invw,
                                                                          p.d_phase, p.d_lut, p.n2_hi, nbins, nwb);
   return cudaGetLastError();
 }

@@ -11,7 +11,7 @@
 //                  transformed along y, folded with k_y, k_z polynomial weights into
 //                  the groups G_{n,p} (power p of k_x; GroupTable); only the pencils
 //                  (k_y, k_z) with k_y^2 + k_z^2 < n2_hi are written, layout
-//                  [mesh][group][x][pencil].
+//                  [mesh][group][pencil block][x][pencil].
 //  k_x_combine  P pencils per CTA, tiles loaded by TMA: FFT along x of every group of
 //             every mesh, interlacing phase and window compensation per mode, A_0
 //             and k^n A_n = sum_p k_x^p G_{n,p}, then w |A_0|^2, w Re A_0 A_2^*,
@@ -98,13 +98,13 @@ struct YZParams {
   const float2* rel;     // [m][3][N] node - observer v, and 2^-floor(log2 |v|) (at most 2^30)
   const float2* tw;      // [TWN] twiddles of the line transforms (LineFft<N>)
   float2* ring;          // [S][nzc][NF][N]
-  float2* gout;          // [m][NG][N][np]
+  float2* gout;          // [m][NG][ngb][N][gw] (GROUP_BLOCK)
   const int* col_off;    // [nzc + 1]
   int* done_z;           // [m N]
   int* done_y;           // [m N]
   int* ticket;           // [1]
   int* err;              // [1]
-  int nzc, np, m, S, D;
+  int nzc, gw, ngb, m, S, D;
   int org[2][3];         // node at r = 0 of each mesh (x < 0: none)
   long long spin_limit;  // ns
   int skip_plane;        // >= 0: that plane's row items withhold their completion (test hook)
@@ -311,7 +311,7 @@ __device__ __forceinline__ void row_item(float2* S, const float2* tws, const flo
 // value times its phase.
 template <int N, int ELL>
 __device__ __forceinline__ void column_fold(const float2* S, int kz, const int* __restrict__ col_off,
-                                            float2* __restrict__ gout, int j, int ix, int np, const int* org,
+                                            float2* __restrict__ gout, int j, int ix, int gw, int ngb, const int* org,
                                             const float* __restrict__ mesh, int tid, int nthr) {
   using Y = YZ<N, ELL>;
   using L = typename Y::L;
@@ -320,8 +320,8 @@ __device__ __forceinline__ void column_fold(const float2* S, int kz, const int* 
   const int p0 = col_off[kz];
   const int cnt = col_off[kz + 1] - p0;
   const int kymax = (cnt - 1) / 2;
-  const size_t gstep = (size_t)N * np;  // between groups
-  float2* g0 = gout + ((size_t)j * NG * N + ix) * np + p0 + kymax;
+  const size_t gstep = (size_t)ngb * N * gw;  // between groups
+  float2* g0 = gout + j * NG * gstep + (size_t)ix * gw;
   const bool at_org = ELL > 0 && ix == org[0];
   float f0 = 0.f;
   if (at_org) f0 = mesh[((size_t)ix * N + org[1]) * N + org[2]];
@@ -337,7 +337,8 @@ __device__ __forceinline__ void column_fold(const float2* S, int kz, const int* 
     }
     float2 gr[NG];
     GroupTable<ELL>::combine([&](int f) { return f == 0 ? F0 : (f == 1 ? Fp : line(f - 1)); }, (float)ky, (float)kz, gr);
-    float2* gp = g0 + ky;
+    const int pen = p0 + kymax + ky;
+    float2* gp = g0 + (size_t)(pen / GROUP_BLOCK) * N * gw + pen % GROUP_BLOCK;
 #pragma unroll
     for (int gi = 0; gi < NG; ++gi) gp[gi * gstep] = gr[gi];
   };
@@ -493,7 +494,7 @@ __device__ __forceinline__ void column_item(float2* S, const float2* tws, const 
   constexpr int NTHR = Y::THREADS / KC;
   const int c = threadIdx.x / NTHR;
   if (c < ncol)
-    column_fold<N, ELL>(S + c * NL * LINE, kz0 + c, prm.col_off, prm.gout, j, ix, prm.np, prm.org[j],
+    column_fold<N, ELL>(S + c * NL * LINE, kz0 + c, prm.col_off, prm.gout, j, ix, prm.gw, prm.ngb, prm.org[j],
                         prm.mesh + (size_t)j * N * N * N, threadIdx.x % NTHR, NTHR);
 }
 
@@ -618,7 +619,7 @@ __host__ __device__ constexpr bool x_horner() { return ELL == 6 || (ELL >= 2 && 
 
 // ---------------------------------------------------------------------------
 // x stage: FFT along x of every (mesh, group) tile of P pencils, fed by TMA.
-// The grouped y,z transforms are a 2D tensor [m NG N rows][np_pad pencils] of
+// The grouped y,z transforms are a 2D tensor [m NG ngb N rows][gw pencils] of
 // float2; one tile (all N rows x P pencils) arrives by BOXES 2D bulk-tensor copies
 // in one shared buffer (mbarrier completion).  Its first FFT stage moves it to the work
 // buffer, and the copy of the next tile overlaps the other stages, which run in
@@ -728,7 +729,7 @@ struct XCombine {
 
 template <int N, int ELL, int M, int PX>
 __global__ void __launch_bounds__(XCombine<N, ELL, M, PX>::THREADS, XCombine<N, ELL, M, PX>::MIN_BLOCKS)
-k_x_combine(const __grid_constant__ XMulti pm, int np_pad, const short2* __restrict__ pencil,
+k_x_combine(const __grid_constant__ XMulti pm, int np_pad, int ngb, const short2* __restrict__ pencil,
             const float2* __restrict__ tw_g, const float* __restrict__ invw_g, const float2* __restrict__ phase_g,
             const short* __restrict__ lut, int n2_hi, int nbins, int nwb) {
   // lane blockIdx.y: its grouped transforms (tensor map), shell accumulators, error flag
@@ -767,12 +768,13 @@ k_x_combine(const __grid_constant__ XMulti pm, int np_pad, const short2* __restr
   auto issue = [&](int s) {  // thread 0: the copy of tile s
     const int k = s / TILES, t = s - k * TILES;
     const int gi = tile_group(t / M), mj = t % M;
-    const int pb = blockIdx.x + k * gridDim.x;
+    const int pen = (blockIdx.x + k * gridDim.x) * P;  // a block of P pencils lies in one pencil block
+    const int row = ((mj * XC::NG + gi) * ngb + pen / GROUP_BLOCK) * N;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     mbar_expect_tx(&bar, XC::TILE_BYTES);
 #pragma unroll
     for (int bx = 0; bx < XC::BOXES; ++bx)
-      tma_load_2d(T + bx * XC::BOX_ROWS * P, gmap, pb * P * 2, (mj * XC::NG + gi) * N + bx * XC::BOX_ROWS, &bar);
+      tma_load_2d(T + bx * XC::BOX_ROWS * P, gmap, pen % GROUP_BLOCK * 2, row + bx * XC::BOX_ROWS, &bar);
   };
   if (tid == 0 && total > 0) issue(0);
   const int p = tid % P, tl = tid / P;

@@ -56,6 +56,13 @@ struct Geom {
 // that near.
 constexpr float YZ_R2_MIN = 8.673617379884035e-19f;
 
+// Pencils per block of the grouped transforms d_g: pencil p of plane x sits in row
+// (block p / GROUP_BLOCK, x) at p % GROUP_BLOCK.  An x-stage tile (a few pencils, every x)
+// then touches rows 8 KB apart; in rows of all 412 000 pencils of a full 1024^3 mesh they
+// were 3.3 MB apart, one page each, and the tiles arrived at 1.2 TB/s (2.3 TB/s in rows of
+// 44 000 pencils).  With at most GROUP_BLOCK pencils there is one block of that many.
+constexpr int GROUP_BLOCK = 1024;
+
 // Launch shape of the y,z kernel for one mesh size and l_max.
 struct YzShape {
   int grid = 0;             // resident CTAs
@@ -78,6 +85,7 @@ struct Plan {
   // pencils (k_y, k_z) kept for the x transform: k_y^2 + k_z^2 < n2_hi
   int n2_hi = 0, nzc = 0, np = 0;
   int np_pad = 0;                // np rounded up to whole x-stage pencil blocks (of either size)
+  int gw = 1, ngb = 1;           // pencils per row and pencil blocks of d_g (GROUP_BLOCK)
   int x_pencils = 0;             // pencils per x-stage CTA in use (k3_pencils or k3_pencils_alt)
   int ring_slots = 1;            // S: planes held by the y,z-stage ring
   int ring_lead = 1;             // D: column items trail row items by D planes
@@ -105,7 +113,7 @@ struct Plan {
   float* d_mesh = nullptr;       // [m][n][n][n]
   float2* d_z = nullptr;         // [S][nzc][nf][n] y,z-stage ring of z-transformed planes
   int* d_sync = nullptr;         // [2 m n + 2] per-plane counters, ticket, error flag
-  float2* d_g = nullptr;         // [m][ng][n][np_pad] grouped y,z transforms
+  float2* d_g = nullptr;         // [m][ng][ngb][n][gw] grouped y,z transforms
   CUtensorMap gmap;              // 2D tensor map of d_g for the x-stage TMA loads
   double* d_acc = nullptr;       // [4][n_bins] shell sums (slot 3 for l_max = 6)
   double* d_sums = nullptr;      // [SUM_COUNT]
