@@ -52,7 +52,7 @@ void dfree(T*& ptr) {
 }
 
 void free_all(Plan& p) {
-  dfree(p.d_tw); dfree(p.d_twl); dfree(p.d_nodes); dfree(p.d_rel); dfree(p.d_invw); dfree(p.d_phase);
+  dfree(p.d_tw); dfree(p.d_twl); dfree(p.d_nodes); dfree(p.d_rel); dfree(p.d_relz); dfree(p.d_invw); dfree(p.d_phase);
   dfree(p.d_col_off); dfree(p.d_pencil); dfree(p.d_lut); dfree(p.d_shell);
   dfree(p.d_mesh); dfree(p.d_z); dfree(p.d_sync); dfree(p.d_g); dfree(p.d_acc); dfree(p.d_sums); dfree(p.d_result);
   dfree(p.d_tile_count); dfree(p.d_tile_off); dfree(p.d_tile_cur); dfree(p.d_rec);
@@ -263,6 +263,8 @@ ys_status build_tables(Plan& p) {
   };
   for (int k = 1; k < r1; ++k)
     for (int t = 0; t < tpl; ++t) twl[(size_t)(k - 1) * tpl + t] = unit_root((double)t * k / n);
+  if (n == 2 * e2_max)  // E2 = 2, R2 = 16
+    for (int q = 0; q < 16; ++q) twl.push_back(unit_root(q / 32.0));
   if (n == 4 * e2_max)  // E2 = 4, R2 = 16
     for (int e = 0; e < 4; ++e)
       for (int q = 0; q < 17; ++q) twl.push_back(unit_root((double)e * q / 64.0));
@@ -334,7 +336,14 @@ ys_status build_tables(Plan& p) {
   YS_UP(p.d_tw, tw);
   YS_UP(p.d_twl, twl);
   YS_UP(p.d_nodes, nodes);
-  YS_UP(p.d_rel, rel);
+  std::vector<float2> rel_xy;
+  std::vector<float> rel_z;
+  for (int j = 0; j < p.m; ++j) {
+    rel_xy.insert(rel_xy.end(), rel.begin() + (size_t)j * 3 * n, rel.begin() + (size_t)(j * 3 + 2) * n);
+    for (int i = 0; i < n; ++i) rel_z.push_back(rel[(size_t)(j * 3 + 2) * n + i].x);
+  }
+  YS_UP(p.d_rel, rel_xy);
+  YS_UP(p.d_relz, rel_z);
 #undef YS_UP
   return YS_OK;
 }
@@ -397,9 +406,15 @@ int ring_lead_for(const Plan& p, int grid, int pct) {
 void set_yz_grid(Plan& p, int grid, int lead_pct) {
   p.yz_grid = std::max(1, std::min(grid, p.yz_grid_max));
   if (lead_pct > 0) p.ring_lead_pct = lead_pct;
+  // Slots: row items of plane p reuse the slot of plane p - S, whose column items are claimed
+  // S - D steps earlier; those steps must hold more than one grid of items, or row items
+  // wait for columns still in flight (256^3 interlaced, about 126 items per plane:
+  // 1.40 ms with S = D + 2, 0.97 ms now; 192^3 400 and 191 us).
+  const int per_plane = p.n / p.yz_rows + std::max(1, (p.nzc + p.yz_cols - 1) / p.yz_cols);
+  const int gap = 2 + (p.yz_grid + per_plane - 1) / per_plane;
   const int slots_max = p.ring_slots_cap > 0 ? p.ring_slots_cap : p.m * p.n;
-  p.ring_lead = std::min(ring_lead_for(p, p.yz_grid, p.ring_lead_pct), std::max(1, slots_max - 2));
-  p.ring_slots = std::min(p.m * p.n, p.ring_lead + 2);
+  p.ring_lead = std::min(ring_lead_for(p, p.yz_grid, p.ring_lead_pct), std::max(1, slots_max - gap));
+  p.ring_slots = std::min(p.m * p.n, p.ring_lead + gap);
 }
 
 LaunchScope::LaunchScope(Plan& plan, int c) : p(plan), cls(c) {
@@ -575,7 +590,7 @@ ys_status ys_plan_create(const ys_config* cfg, ys_plan** out) {
   }
   const size_t n3 = (size_t)n * n * n;
   // y,z-stage ring: the column items of a plane trail its row items by D planes, and a
-  // slot is rewritten S = D + 2 planes later; D covers one grid's worth of items.
+  // slot is rewritten S planes later (set_yz_grid).
   const ys::YzShape shape = ys::yz_shape_for(p, &e);
   p.yz_grid_max = shape.grid;
   p.yz_rows = shape.rows;

@@ -192,11 +192,12 @@ template <> struct Dft<1> {
 //   1. Thread t holds x[t + TPL r] and does one radix-R1 butterfly in registers,
 //      multiplies by exp(-2 pi i t k1 / N) and stores element (k1, t) at k1 P + t.
 //   2. Butterfly (k1, e), e < E2, takes (k1, e + E2 s), s < R2, through a radix-R2
-//      butterfly, multiplies by exp(-2 pi i e q / (R2 E2)) and puts the results back
-//      where its inputs were.
+//      butterfly, multiplies by exp(-2 pi i e q / (R2 E2)) (E2 = 4) and puts the results
+//      back where its inputs were.
 //   3. The reader does the last radix E2 (1, 2 or 4) on the E2 neighbouring elements
 //      of a slot: frequency kappa + (N / E2) h, kappa = k1 + R1 q, is
-//      sum_e exp(-2 pi i e h / E2) element[slot(kappa) + e].
+//      sum_e exp(-2 pi i e h / E2) element[slot(kappa) + e], the second element of an
+//      E2 = 2 slot times exp(-2 pi i q / (2 R2)) (in step 2 half of the lanes would idle).
 // A line thus crosses shared memory twice (three times with radix-8 stages of 8
 // elements per thread at N = 512), and its twiddles stay in registers.  The pitch P
 // and the line length LINE keep every access conflict-free: the E2 elements of a slot
@@ -216,9 +217,10 @@ struct LineFft {
   static constexpr int LINE = E2 == 1 ? ((R1 * P) | 1) : R1 * P + (6 - (R1 * P) % 4) % 4;
   static constexpr int M = N / E2;
   static constexpr int HALF_ITEMS = E2 == 1 ? N / 2 : M / 2;  // items of line_halves
-  // Twiddle table: exp(-2 pi i t k / N) at (k - 1) TPL + t, 1 <= k < R1, then for E2 = 4
-  // exp(-2 pi i e q / (4 R2)) at 17 e + q.
-  static constexpr int TWN = (R1 - 1) * TPL + (E2 == 4 ? 4 * 17 : 0);
+  // Twiddle table: exp(-2 pi i t k / N) at (k - 1) TPL + t, 1 <= k < R1, then for E2 = 2
+  // exp(-2 pi i q / (2 R2)) at q, for E2 = 4 exp(-2 pi i e q / (4 R2)) at 17 e + q.
+  static constexpr int TW2 = (R1 - 1) * TPL;
+  static constexpr int TWN = TW2 + (E2 == 4 ? 4 * 17 : (E2 == 2 ? R2 : 0));
   static_assert(R1 * R2 * E2 == N && TPL * R1 == N, "factors");
   __host__ __device__ static constexpr int slot(int kappa) { return (kappa % R1) * P + (kappa / R1) * E2; }
 };
@@ -235,25 +237,6 @@ __device__ __forceinline__ int line_of_group(int g) {
   }
 }
 
-// exp(-2 pi i q / 32), q < 16
-__device__ constexpr float kW32[16][2] = {
-      {1.000000000000000000e+00f, -0.000000000000000000e+00f},
-      {9.807852804032304306e-01f, -1.950903220161282481e-01f},
-      {9.238795325112867385e-01f, -3.826834323650897818e-01f},
-      {8.314696123025452357e-01f, -5.555702330196021776e-01f},
-      {7.071067811865475727e-01f, -7.071067811865474617e-01f},
-      {5.555702330196022887e-01f, -8.314696123025452357e-01f},
-      {3.826834323650898373e-01f, -9.238795325112867385e-01f},
-      {1.950903220161283314e-01f, -9.807852804032304306e-01f},
-      {6.123233995736766036e-17f, -1.000000000000000000e+00f},
-      {-1.950903220161281926e-01f, -9.807852804032304306e-01f},
-      {-3.826834323650897263e-01f, -9.238795325112867385e-01f},
-      {-5.555702330196019556e-01f, -8.314696123025454577e-01f},
-      {-7.071067811865474617e-01f, -7.071067811865475727e-01f},
-      {-8.314696123025453467e-01f, -5.555702330196021776e-01f},
-      {-9.238795325112867385e-01f, -3.826834323650898928e-01f},
-      {-9.807852804032304306e-01f, -1.950903220161286089e-01f}};
-
 // The twiddles of thread t of a line, from the table.
 template <int N>
 __device__ __forceinline__ void load_twiddles(float2 (&tw)[LineFft<N>::R1 - 1], const float2* table, int t) {
@@ -263,7 +246,7 @@ __device__ __forceinline__ void load_twiddles(float2 (&tw)[LineFft<N>::R1 - 1], 
 
 // Steps 1 and 2 for the line at `line`; v: the thread's R1 elements.  Every thread of a
 // warp calls this (ok: whether its line exists); tw: exp(-2 pi i t k / N), k = 1..R1 - 1;
-// wE: the table's part for E2 = 4.
+// wE: the table's part from TW2.
 template <int N>
 __device__ __forceinline__ void line_fft(float2 (&v)[LineFft<N>::R1], float2* line, int t,
                                          const float2 (&tw)[LineFft<N>::R1 - 1], const float2* wE, bool ok) {
@@ -287,13 +270,7 @@ __device__ __forceinline__ void line_fft(float2 (&v)[LineFft<N>::R1], float2* li
 #pragma unroll
         for (int s = 0; s < R2; ++s) b[s] = q[E2 * s];
         Dft<R2>::run(b);
-        if constexpr (E2 == 2) {
-          static_assert(E2 != 2 || R2 == 16, "w32 twiddles");
-          if (e) {
-#pragma unroll
-            for (int s = 1; s < R2; ++s) b[s] = cmul(b[s], make_float2(kW32[s][0], kW32[s][1]));
-          }
-        } else if constexpr (E2 == 4) {
+        if constexpr (E2 == 4) {
 #pragma unroll
           for (int s = 1; s < R2; ++s) b[s] = cmul(b[s], wE[17 * e + s]);
         }
@@ -304,16 +281,18 @@ __device__ __forceinline__ void line_fft(float2 (&v)[LineFft<N>::R1], float2* li
   }
 }
 
-// The two half spectra of a line that holds real lines a + i b: emit(k, A_k, B_k) for
+// The two half spectra of a line that holds real lines (a + i b) / 2: emit(k, A_k, B_k) for
 // the k < nk of item i (0 <= i < HALF_ITEMS covers every k < N / 2 once).  With
-// C_k the line's transform, A_k = (C_k + C_{N-k}^*) / 2, B_k = (C_k - C_{N-k}^*) / (2 i).
+// C_k the line's transform, A_k = C_k + C_{N-k}^*, B_k = (C_k - C_{N-k}^*) / i.
 template <int N, class Emit>
-__device__ __forceinline__ void line_halves(const float2* line, int i, int nk, Emit&& emit) {
+__device__ __forceinline__ void line_halves(const float2* line, const float2* wE, int i, int nk, Emit&& emit) {
   using L = LineFft<N>;
   constexpr int M = L::M;
   auto out = [&](int k, float2 c, float2 m) {
-    if (k < nk)
-      emit(k, make_float2(0.5f * (c.x + m.x), 0.5f * (c.y - m.y)), make_float2(0.5f * (c.y + m.y), -0.5f * (c.x - m.x)));
+    if (k < nk) {
+      const float2 s = __ffma2_rn(m, make_float2(1.f, -1.f), c), d = __ffma2_rn(m, make_float2(-1.f, 1.f), c);
+      emit(k, s, make_float2(d.y, -d.x));
+    }
   };
   if constexpr (L::E2 == 1) {
     if (i >= nk) return;
@@ -326,9 +305,11 @@ __device__ __forceinline__ void line_halves(const float2* line, int i, int nk, E
     const float4* s0 = reinterpret_cast<const float4*>(line + L::slot(k0));
     const float4* s1 = reinterpret_cast<const float4*>(line + L::slot(k1));
     const float4 p = s0[0], q = s1[0];
-    const float2 p0 = make_float2(p.x, p.y), p1 = make_float2(p.z, p.w);
-    const float2 q0 = make_float2(q.x, q.y), q1 = make_float2(q.z, q.w);
+    float2 p0 = make_float2(p.x, p.y), p1 = make_float2(p.z, p.w);
+    float2 q0 = make_float2(q.x, q.y), q1 = make_float2(q.z, q.w);
     if constexpr (L::E2 == 2) {
+      p1 = cmul(p1, wE[k0 / L::R1]);
+      q1 = cmul(q1, wE[k1 / L::R1]);
       const float2 a0 = cadd(p0, p1), a1 = csub(p0, p1), b0 = cadd(q0, q1), b1 = csub(q0, q1);
       out(k0, a0, i ? b1 : a0);
       out(k1, b0, i ? a1 : b1);

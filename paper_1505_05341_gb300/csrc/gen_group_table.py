@@ -107,6 +107,9 @@ def emit(ell_max):
     lines.append("    kyp[0] = 1.f; kzp[0] = 1.f;")
     lines.append("    #pragma unroll")
     lines.append(f"    for (int i = 1; i < {npow}; ++i) {{ kyp[i] = kyp[i - 1] * ky; kzp[i] = kzp[i - 1] * kz; }}")
+    monos = sorted({m for poly in tab.values() for m in poly if m[0] and m[1]})
+    for b, c in monos:  # each product of powers once
+        lines.append(f"    [[maybe_unused]] const float m{b}{c} = kyp[{b}] * kzp[{c}];")
     by_beta = {}
     for (gi, beta), poly in sorted(tab.items()):
         by_beta.setdefault(beta, []).append((gi, poly))
@@ -116,7 +119,8 @@ def emit(ell_max):
             terms = []
             for (b, c), v in sorted(poly.items()):
                 assert v.denominator == 1
-                terms.append(f"({float(v.numerator)!r}f * kyp[{b}] * kzp[{c}])")
+                mono = f"m{b}{c}" if b and c else (f"kyp[{b}]" if b else f"kzp[{c}]")
+                terms.append(f"({float(v.numerator)!r}f * {mono})")
             lines.append(f"      {{ const float w = {' + '.join(terms)};")
             lines.append(f"        g[{gi}].x = fmaf(w, ps.x, g[{gi}].x); g[{gi}].y = fmaf(w, ps.y, g[{gi}].y); }}")
         lines.append("    }")

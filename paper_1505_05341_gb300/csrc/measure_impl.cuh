@@ -63,6 +63,7 @@ cudaError_t run_yz(Plan* const* lanes, int W) {
     YZParams& prm = pm.lane[l];
     prm.mesh = p.d_mesh;
     prm.rel = p.d_rel;
+    prm.relz = p.d_relz;
     prm.tw = p.d_twl;
     prm.ring = p.d_z;
     prm.gout = p.d_g;

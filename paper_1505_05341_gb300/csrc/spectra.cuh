@@ -86,16 +86,18 @@ template <int ELL> __constant__ constexpr YLines<ELL> kYLines{};
 // per-plane completion counters (release / acquire), bounded in time; a CTA only
 // ever waits on items claimed before its own, so the list cannot deadlock.
 //
-// What bounds it (512^3, l_max = 4, one mesh): instruction issue (51 % of the slots; 30 %
-// of the instructions are packed or scalar float arithmetic) and barriers, with
-// 16 warps per SM (128 registers); shared memory 57 % busy.  12.1 -> 6.5 ms for the
-// interlaced pair against transforming every basis field along z (16 real lines per
-// row instead of 5) with radix-8 stages; l_max = 6 30.8 -> 13.9 ms, 1024^3 87 -> 40 ms.
+// What bounds it: instruction issue (512^3, l_max = 4: about half of the slots, 16 warps
+// per SM at 128 registers; shared memory 57 % busy).  The interlaced pair at 512^3 took
+// 12.1 ms when every basis field was transformed along z (16 real lines per row instead of
+// 5) with radix-8 stages, 6.5 ms with source fields and line transforms, 5.7 ms with two
+// barriers per item and the radix-2 twiddles left to the readers; l_max = 6 30.8, 13.9,
+// 11.6 ms; 1024^3 87, 40, 35 ms; 256^3 interlaced 1.76, 1.19, 0.97 ms.
 // ---------------------------------------------------------------------------
 
 struct YZParams {
   const float* mesh;     // [m][N][N][N]
-  const float2* rel;     // [m][3][N] node - observer v, and 2^-floor(log2 |v|) (at most 2^30)
+  const float2* rel;     // [m][2][N] x, y of node - observer v, and 2^-floor(log2 |v|) (at most 2^30)
+  const float* relz;     // [m][N] z of node - observer
   const float2* tw;      // [TWN] twiddles of the line transforms (LineFft<N>)
   float2* ring;          // [S][nzc][NF][N]
   float2* gout;          // [m][NG][ngb][N][gw] (GROUP_BLOCK)
@@ -184,6 +186,8 @@ struct YZ {
   static constexpr int KC = kc();
   static constexpr int CLINES = NL * KC;
   static constexpr int LPG = (CLINES + GROUPS - 1) / GROUPS;  // lines per thread group
+  // whether the last warp has less to transform than the others in a column item
+  static constexpr bool SLACK = TPL >= 32 && GROUPS * LPG > CLINES;
   static constexpr int LINES = (RLINES > CLINES ? RLINES : CLINES) * LINE;  // elements of the line buffers
   static constexpr int TWN = L::TWN;                                         // and of the twiddles
   static constexpr size_t smem = sizeof(float2) * (LINES + TWN);
@@ -207,17 +211,19 @@ __device__ __forceinline__ float recip_nr(float x) {
 // the item stay in shared memory, so one barrier separates the transforms from the
 // split into half spectra, which writes runs of R rows to the ring slot
 // [k_z][source][y].
-template <int N, int ELL>
-__device__ __forceinline__ void row_item(float2* S, const float2* tws, const float* __restrict__ plane, float2 X,
-                                         const float2* __restrict__ rely, const float2* __restrict__ relz, int row0,
-                                         float2* __restrict__ zslot, int nzc, int* ticket, int& next) {
+// before_mid() is called by every thread between the transforms and the barrier before the
+// split (it elects the threads that claim and wait); false after that barrier: give up.
+template <int N, int ELL, class Mid>
+__device__ __forceinline__ bool row_item(float2* S, const float2* tws, const float* __restrict__ plane, float2 X,
+                                         const float2* __restrict__ rely, const float* __restrict__ relz, int row0,
+                                         float2* __restrict__ zslot, int nzc, Mid&& before_mid, const int& ok_flag) {
   using Y = YZ<N, ELL>;
   using L = typename Y::L;
   constexpr int R = Y::R, LINE = L::LINE, R1 = L::R1, TPL = L::TPL, GROUPS = Y::GROUPS, ND = Y::ND, NF = Y::NF;
   const int t = threadIdx.x % TPL, g = line_of_group<TPL>(threadIdx.x / TPL);
   float2 tw[R1 - 1];
   load_twiddles<N>(tw, tws, t);
-  const float2* wE = tws + (R1 - 1) * TPL;
+  const float2* wE = tws + L::TW2;
   if constexpr (ND > 0) {
 #pragma unroll 1
     for (int r0 = 0; r0 < R; r0 += GROUPS) {
@@ -228,17 +234,17 @@ __device__ __forceinline__ void row_item(float2* S, const float2* tws, const flo
       float f[R1], i2[R1], irho = 1.f;
       if (ok) {
         const float2 Yc = rely[row0 + r];
-        const float xy2 = fmaf(X.x, X.x, Yc.x * Yc.x);
-        irho = fminf(X.y, Yc.y);  // a power of two, as 1 / irho: exact
-        const float rho2 = 1.f / (irho * irho);
+        irho = fminf(X.y, Yc.y);  // a power of two: every product with it is exact
+        const float xs = X.x * irho, ys = Yc.x * irho, xy2 = fmaf(xs, xs, ys * ys);
+        const float r2_min = YZ_R2_MIN * irho * irho;
         const float* frow = plane + (size_t)(row0 + r) * N + t;
 #pragma unroll
         for (int k = 0; k < R1; ++k) f[k] = frow[k * TPL];
 #pragma unroll
         for (int k = 0; k < R1; ++k) {
-          const float Zc = relz[t + k * TPL].x;
-          const float r2 = fmaf(Zc, Zc, xy2);
-          i2[k] = r2 > YZ_R2_MIN ? rho2 * recip_nr(r2) : 0.f;
+          const float zs = relz[t + k * TPL] * irho, r2 = fmaf(zs, zs, xy2);  // (|r| / rho)^2
+          i2[k] = r2 > r2_min ? recip_nr(r2) : 0.f;
+          f[k] *= 0.5f;  // for line_halves
         }
       }
 #pragma unroll
@@ -248,7 +254,7 @@ __device__ __forceinline__ void row_item(float2* S, const float2* tws, const flo
 #pragma unroll
           for (int k = 0; k < R1; ++k) {
             f[k] *= i2[k];
-            v[k] = make_float2(f[k], f[k] * (relz[t + k * TPL].x * irho));
+            v[k] = make_float2(f[k], f[k] * (relz[t + k * TPL] * irho));
           }
         }
         if (Y::SPLIT && (d >= Y::DSPLIT) != upper) continue;
@@ -265,13 +271,14 @@ __device__ __forceinline__ void row_item(float2* S, const float2* tws, const flo
     if (ok) {
       const float* frow = plane + (size_t)(row0 + 2 * p) * N + t;
 #pragma unroll
-      for (int k = 0; k < R1; ++k) v[k] = make_float2(frow[k * TPL], frow[N + k * TPL]);
+      for (int k = 0; k < R1; ++k) v[k] = make_float2(0.5f * frow[k * TPL], 0.5f * frow[N + k * TPL]);
     }
     line_fft<N>(v, S + (ND * R + p) * LINE, t, tw, wE, ok);
   }
-  if (threadIdx.x == 0) next = atomicAdd(ticket, 1);  // see k_yz
+  before_mid();
   __syncthreads();
-  // Two real lines a + i b: A_k = (C_k + C_{N-k}^*)/2, B_k = (C_k - C_{N-k}^*)/(2i).
+  if (!ok_flag) return false;
+  // Two real lines per complex line: their half spectra.
   if constexpr (ND > 0) {
     constexpr int RL = R < 16 ? R : 16, KS = Y::THREADS / RL;
 #pragma unroll 1
@@ -282,7 +289,7 @@ __device__ __forceinline__ void row_item(float2* S, const float2* tws, const flo
         const float2* line = S + (d * R + r) * LINE;
         float2* out = zslot + (size_t)(1 + 2 * d) * N + row0 + r;
         for (int i = threadIdx.x / RL; i < L::HALF_ITEMS; i += KS)
-          line_halves<N>(line, i, nzc, [&](int kz, float2 A, float2 B) {
+          line_halves<N>(line, wE, i, nzc, [&](int kz, float2 A, float2 B) {
             float2* o = out + (size_t)kz * NF * N;
             o[0] = A;
             o[N] = B;
@@ -298,11 +305,12 @@ __device__ __forceinline__ void row_item(float2* S, const float2* tws, const flo
       const float2* line = S + (ND * R + p) * LINE;
       float2* out = zslot + row0 + 2 * p;
       for (int i = threadIdx.x / PL; i < L::HALF_ITEMS; i += KS)
-        line_halves<N>(line, i, nzc, [&](int kz, float2 A, float2 B) {
+        line_halves<N>(line, wE, i, nzc, [&](int kz, float2 A, float2 B) {
           *reinterpret_cast<float4*>(out + (size_t)kz * NF * N) = make_float4(A.x, A.y, B.x, B.y);
         });
     }
   }
+  return true;
 }
 
 // Fold of one column (k_z): the y transforms of the basis fields at k_y become the
@@ -310,7 +318,7 @@ __device__ __forceinline__ void row_item(float2* S, const float2* tws, const flo
 // F' at the plane of the node at r = 0 (org): the transform of F less that node's
 // value times its phase.
 template <int N, int ELL>
-__device__ __forceinline__ void column_fold(const float2* S, int kz, const int* __restrict__ col_off,
+__device__ __forceinline__ void column_fold(const float2* S, const float2* wE, int kz, const int* __restrict__ col_off,
                                             float2* __restrict__ gout, int j, int ix, int gw, int ngb, const int* org,
                                             const float* __restrict__ mesh, int tid, int nthr) {
   using Y = YZ<N, ELL>;
@@ -358,12 +366,13 @@ __device__ __forceinline__ void column_fold(const float2* S, int kz, const int* 
       const bool up = kap <= kymax, dn = M - kap <= kymax;
       if (!up && !dn) continue;
       const float2* sp = S + L::slot(kap);
+      const float2 w = wE[kap / L::R1];
       if constexpr (HOLD) {
         float2 Ta[NL], Tb[NL];
 #pragma unroll
         for (int l = 0; l < NL; ++l) {
           const float4 q = *reinterpret_cast<const float4*>(sp + l * LINE);
-          const float2 x = make_float2(q.x, q.y), y = make_float2(q.z, q.w);
+          const float2 x = make_float2(q.x, q.y), y = cmul(make_float2(q.z, q.w), w);
           Ta[l] = cadd(x, y);
           Tb[l] = csub(x, y);
         }
@@ -376,7 +385,7 @@ __device__ __forceinline__ void column_fold(const float2* S, int kz, const int* 
           const float2 sg = half ? make_float2(-1.f, -1.f) : make_float2(1.f, 1.f);
           emit([&](int l) {
             const float4 q = *reinterpret_cast<const float4*>(sp + l * LINE);
-            return __ffma2_rn(make_float2(q.z, q.w), sg, make_float2(q.x, q.y));
+            return __ffma2_rn(cmul(make_float2(q.z, q.w), w), sg, make_float2(q.x, q.y));
           }, kap - half * M);
         }
       }
@@ -416,21 +425,21 @@ __device__ __forceinline__ void column_fold(const float2* S, int kz, const int* 
 // loads a source line, multiplies it by (X / rho)^a (Y / rho)^b and transforms it, LPG
 // lines in turn.  The exponents are uniform over the group, so the tests on their bits
 // skip whole unrolled loops where a group is a warp or more.
-template <int N, int ELL>
+template <int N, int ELL, class Mid>
 __device__ __forceinline__ void column_item(float2* S, const float2* tws, const float2* __restrict__ zslot, int kz0,
-                                            const YZParams& prm, int j, int ix, int* ticket, int& next) {
+                                            const YZParams& prm, int j, int ix, Mid&& before_mid) {
   using Y = YZ<N, ELL>;
   using L = typename Y::L;
   constexpr int LINE = L::LINE, R1 = L::R1, TPL = L::TPL, NF = Y::NF, NL = Y::NL, KC = Y::KC, LPG = Y::LPG;
   const int t = threadIdx.x % TPL, g = line_of_group<TPL>(threadIdx.x / TPL);
   const int ncol = min(KC, prm.nzc - kz0);
-  const float2* __restrict__ rel = prm.rel + (size_t)j * 3 * N;
+  const float2* __restrict__ rel = prm.rel + (size_t)j * 2 * N;
   const float2* __restrict__ rely = rel + N + t;
   const float2 X = rel[ix];
   {
     float2 tw[R1 - 1];
     load_twiddles<N>(tw, tws, t);
-    const float2* wE = tws + (R1 - 1) * TPL;
+    const float2* wE = tws + L::TW2;
 #pragma unroll 1
     for (int i = 0; i < LPG; ++i) {
       const int l = g * LPG + i, c = l / NL, ln = l - c * NL;
@@ -481,7 +490,9 @@ __device__ __forceinline__ void column_item(float2* S, const float2* tws, const 
       line_fft<N>(v, S + l * LINE, t, tw, wE, ok);
     }
   }
+  if constexpr (Y::SLACK) before_mid();
   __syncthreads();  // every ring load is done, every line transformed
+  if constexpr (!Y::SLACK) before_mid();
   // The ring lines of these columns are dead once read: drop them from L2 without a
   // write-back (the slot is rewritten only after this item's completion is
   // released).  A column is NF * N * 8 bytes, a whole number of 128-byte lines.
@@ -490,100 +501,134 @@ __device__ __forceinline__ void column_item(float2* S, const float2* tws, const 
     for (int c = threadIdx.x; c < ncol * (NF * N / 16); c += Y::THREADS)
       asm volatile("discard.global.L2 [%0], 128;" ::"l"(dead + c * 16) : "memory");
   }
-  if (threadIdx.x == 0) next = atomicAdd(ticket, 1);  // see k_yz
   constexpr int NTHR = Y::THREADS / KC;
   const int c = threadIdx.x / NTHR;
   if (c < ncol)
-    column_fold<N, ELL>(S + c * NL * LINE, kz0 + c, prm.col_off, prm.gout, j, ix, prm.gw, prm.ngb, prm.org[j],
+    column_fold<N, ELL>(S + c * NL * LINE, tws + L::TW2, kz0 + c, prm.col_off, prm.gout, j, ix, prm.gw, prm.ngb, prm.org[j],
                         prm.mesh + (size_t)j * N * N * N, threadIdx.x % NTHR, NTHR);
 }
 
-// Completion of one item: every thread's writes are ordered before thread 0's
-// release-add by the barrier (the release is cumulative over them).
-__device__ __forceinline__ void signal_release(int* counter) {
-  __syncthreads();
-  if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(counter) : "memory");
+// What a CTA does next: one item of the list, decoded from its ticket by one thread.
+struct YZItem {
+  int lane;   // -1: the list is at its end
+  int plane;  // of the row or column item; -1: nothing to do (the list's ragged ends)
+  int sub;    // row item index (< NZ), or NZ + column item index
+  int ready;  // the items it depends on were done when it was claimed
+};
+
+// The completion counter that item `it` waits on, and its target; nullptr: none.
+template <int N, int ELL>
+__device__ __forceinline__ const int* yz_dependency(const YZMulti& pm, const YZItem& it, int& target) {
+  using Y = YZ<N, ELL>;
+  if (it.lane < 0 || it.plane < 0) return nullptr;
+  const YZParams& prm = pm.lane[it.lane];
+  if (it.sub >= N / Y::R) {  // column item: the plane's row items
+    target = N / Y::R;
+    return prm.done_z + it.plane;
+  }
+  if (it.plane < prm.S) return nullptr;  // row item: the column items of the ring slot's last plane
+  target = (prm.nzc + Y::KC - 1) / Y::KC;
+  return prm.done_y + (it.plane - prm.S);
 }
 
+// Decodes a ticket and looks once whether its dependency is met.
+template <int N, int ELL>
+__device__ __forceinline__ YZItem yz_decode(const YZMulti& pm, int ticket) {
+  using Y = YZ<N, ELL>;
+  constexpr int NZ = N / Y::R;
+  YZItem it{-1, -1, 0, 0};
+  if (ticket >= pm.end[pm.nlanes - 1]) return it;
+  int l = 0;
+  while (ticket >= pm.end[l]) ++l;
+  const YZParams& prm = pm.lane[l];
+  const int item = ticket - (l > 0 ? pm.end[l - 1] : 0);
+  const int per_step = NZ + (prm.nzc + Y::KC - 1) / Y::KC;
+  const int step = item / per_step;
+  it.lane = l;
+  it.sub = item - step * per_step;
+  it.plane = it.sub < NZ ? (step < prm.m * N ? step : -1) : step - prm.D;
+  if (it.plane < 0) it.plane = -1;
+  int target = 0;
+  const int* dep = yz_dependency<N, ELL>(pm, it, target);
+  it.ready = dep == nullptr || ld_acquire(dep) >= target;
+  return it;
+}
+
+// Completion of an item: the CTA is past a barrier after its last writes, and thread 0's
+// release-add orders them (it is cumulative over the barrier).
+__device__ __forceinline__ void signal_release(int* counter) {
+  asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(counter) : "memory");
+}
+
+// One thread of the last warp, which has the least to transform, claims the next ticket
+// when its own transforms of the item are done (of a column item without SLACK: after the
+// middle barrier; the fold leaves the last warp idle first): the atomic's round trip, the
+// decoding and one look at the next item's dependency (~1400 cycles) overlap the other
+// warps' work, and the barrier that ends the item publishes the result.  Usually the dependency is met and the
+// next item starts without another barrier: two per item (five with a wait, a completion
+// and a hand-over barrier each).  A row item needs its ring slot only for the split, so
+// there a wait delays the middle barrier only.  Claiming a whole item ahead delayed the
+// items waiting on it too much.  Items wait only on items of earlier tickets, so the list
+// cannot deadlock; a CTA signals its item before it waits for the next one's dependency.
 template <int N, int ELL>
 __global__ void __launch_bounds__(YZ<N, ELL>::THREADS, YZ<N, ELL>::MIN_BLOCKS) k_yz(const __grid_constant__ YZMulti pm) {
   using Y = YZ<N, ELL>;
-  using L = typename Y::L;
-  constexpr int R = Y::R;
+  constexpr int R = Y::R, NZ = N / R;
+  constexpr int CLAIM = Y::THREADS - 32, WAIT = Y::THREADS - 64;  // the claiming and the waiting thread
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int s_item;
+  __shared__ YZItem s_item[2];  // this item and the next
   __shared__ int s_ok;
   float2* work = reinterpret_cast<float2*>(smem_raw);
   // Twiddles of the line transforms (same N: the same for every lane).
   float2* tws = work + Y::LINES;
   for (int k = threadIdx.x; k < Y::TWN; k += Y::THREADS) tws[k] = pm.lane[0].tw[k];
-  constexpr int NZ = N / R;
-  const int total = pm.end[pm.nlanes - 1];
   const size_t n3 = (size_t)N * N * N;
-  if (threadIdx.x == 0) s_item = atomicAdd(pm.ticket, 1);
+  if (threadIdx.x == CLAIM) s_item[0] = yz_decode<N, ELL>(pm, atomicAdd(pm.ticket, 1));
+  if (threadIdx.x == 0) s_ok = 1;
   __syncthreads();
-  int gitem = s_item;
-  for (;;) {
-    if (gitem >= total) break;
-    // Thread 0 claims the next ticket shortly before this item ends (before the split
-    // of a row item, before the fold of a column item), so that the atomic's round
-    // trip overlaps the item's tail.  A claimed item starts that little later;
-    // claiming a whole item ahead delayed the items waiting on it too much.  Items
-    // wait only on items of earlier tickets, so the list cannot deadlock.
-    int next = -1;
-    {  // L2 prefetch of the mesh rows of the row item one grid of tickets ahead
-      const int ahead = gitem + (int)gridDim.x;
-      if (ahead < total && threadIdx.x < R * N / 32) {
-        int la = 0;
-        while (ahead >= pm.end[la]) ++la;
-        const YZParams& pa = pm.lane[la];
-        const int ia = ahead - (la > 0 ? pm.end[la - 1] : 0);
-        const int ipa = NZ + (pa.nzc + Y::KC - 1) / Y::KC, sta = ia / ipa, sba = ia - sta * ipa;
-        if (sba < NZ && sta < pa.m * N) {
-          const int ja = sta / N, xa = sta - ja * N;
-          const float* rows = pa.mesh + ja * n3 + (size_t)xa * N * N + (size_t)sba * R * N;
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(rows + threadIdx.x * 32));  // one 128-byte line each
-        }
-      }
+  for (int turn = 0;; turn ^= 1) {
+    const YZItem it = s_item[turn];
+    if (it.lane < 0) break;
+    const YZParams& prm = pm.lane[it.lane];
+    const bool row = it.sub < NZ;
+    auto wait = [&]() {
+      int target = 0;
+      const int* dep = yz_dependency<N, ELL>(pm, it, target);
+      if (!wait_geq(dep, target, prm.err, prm.spin_limit)) s_ok = 0;
+    };
+    if (!it.ready && !row) {
+      if (threadIdx.x == WAIT) wait();
+      __syncthreads();
+      if (!s_ok) break;
     }
-    int l = 0;
-    while (gitem >= pm.end[l]) ++l;
-    const YZParams& prm = pm.lane[l];
-    const int item = gitem - (l > 0 ? pm.end[l - 1] : 0);
-    const int NY = (prm.nzc + Y::KC - 1) / Y::KC, IPS = NZ + NY;
-    const int mN = prm.m * N;
-    const size_t slot_elems = (size_t)Y::NF * prm.nzc * N;  // float2 units
-    const int step = item / IPS, sub = item - step * IPS;
-    if (sub < NZ) {
-      const int p = step;  // row item of plane p
-      if (p < mN) {
-        if (threadIdx.x == 0)
-          s_ok = (p < prm.S) ? 1 : (int)wait_geq(prm.done_y + (p - prm.S), NY, prm.err, prm.spin_limit);
-        __syncthreads();
-        if (!s_ok) break;
-        const int j = p / N, ix = p - j * N;
-        const float2* rel = prm.rel + (size_t)j * 3 * N;
-        row_item<N, ELL>(work, tws, prm.mesh + j * n3 + (size_t)ix * N * N, rel[ix], rel + N, rel + 2 * N, sub * R,
-                         prm.ring + (size_t)(p % prm.S) * slot_elems, prm.nzc, pm.ticket, next);
-        if (p != prm.skip_plane) signal_release(prm.done_z + p);
-        else __syncthreads();  // withheld: the column items of plane p wait until their limit
+    auto before_mid = [&]() {
+      if (threadIdx.x == CLAIM) s_item[turn ^ 1] = yz_decode<N, ELL>(pm, atomicAdd(pm.ticket, 1));
+      if (threadIdx.x == WAIT && !it.ready && row) wait();
+    };
+    int* done = nullptr;
+    const int p = it.plane, j = p / N, ix = p - j * N;
+    if (p >= 0) {
+      float2* slot = prm.ring + (size_t)(p % prm.S) * Y::NF * prm.nzc * N;
+      const float* plane = prm.mesh + j * n3 + (size_t)ix * N * N;
+      if (row) {
+        // L2 prefetch of the next plane's rows, about one grid of tickets ahead
+        if (p + 1 < prm.m * N && threadIdx.x < R * N / 32)
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(plane + (size_t)N * N + (size_t)it.sub * R * N +
+                                                        threadIdx.x * 32));  // one 128-byte line each
+        const float2* rel = prm.rel + (size_t)j * 2 * N;
+        if (!row_item<N, ELL>(work, tws, plane, rel[ix], rel + N, prm.relz + (size_t)j * N, it.sub * R, slot, prm.nzc,
+                              before_mid, s_ok))
+          break;
+        if (p != prm.skip_plane) done = prm.done_z + p;  // (withheld: its column items wait until their limit)
+      } else {
+        column_item<N, ELL>(work, tws, slot, (it.sub - NZ) * Y::KC, prm, j, ix, before_mid);
+        done = prm.done_y + p;
       }
     } else {
-      const int p = step - prm.D;  // column item of plane p
-      if (p >= 0) {
-        if (threadIdx.x == 0) s_ok = (int)wait_geq(prm.done_z + p, NZ, prm.err, prm.spin_limit);
-        __syncthreads();
-        if (!s_ok) break;
-        const int j = p / N, ix = p - j * N;
-        column_item<N, ELL>(work, tws, prm.ring + (size_t)(p % prm.S) * slot_elems, (sub - NZ) * Y::KC, prm, j, ix,
-                            pm.ticket, next);
-        signal_release(prm.done_y + p);
-      }
+      before_mid();
     }
-    __syncthreads();  // every thread is past this item before s_item changes
-    if (threadIdx.x == 0) s_item = next >= 0 ? next : atomicAdd(pm.ticket, 1);
-    __syncthreads();
-    gitem = s_item;
+    __syncthreads();  // every thread is past this item, and the next one is published
+    if (threadIdx.x == 0 && done) signal_release(done);
   }
 }
 

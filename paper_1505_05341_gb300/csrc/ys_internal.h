@@ -102,7 +102,8 @@ struct Plan {
   float2* d_tw = nullptr;        // [n] stage-major twiddles of the x stage (fft_tw_offset)
   float2* d_twl = nullptr;       // twiddles of the y,z stage's line transforms (LineFft)
   float2* d_nodes = nullptr;     // [3][n + 3] node positions (hi, lo), index offset 1
-  float2* d_rel = nullptr;       // [m][3][n] node - observer v in units of a power of two, 2^-floor(log2 |v|)
+  float2* d_rel = nullptr;       // [m][2][n] x, y of node - observer v in units of a power of two, 2^-floor(log2 |v|)
+  float* d_relz = nullptr;       // [m][n] z of node - observer in that unit
   float* d_invw = nullptr;       // [n] per-axis 1 / sinc^p by FFT index (1 if !compensate)
   float2* d_phase = nullptr;     // [n] per-axis exp(-i pi m / n) by FFT index
   int* d_col_off = nullptr;      // [nzc + 1] first pencil of each k_z column
