@@ -666,8 +666,8 @@ __host__ __device__ constexpr bool x_horner() { return ELL == 6 || (ELL >= 2 && 
 // x stage: FFT along x of every (mesh, group) tile of P pencils, fed by TMA.
 // The grouped y,z transforms are a 2D tensor [m NG ngb N rows][gw pencils] of
 // float2; one tile (all N rows x P pencils) arrives by BOXES 2D bulk-tensor copies
-// in one shared buffer (mbarrier completion).  Its first FFT stage moves it to the work
-// buffer, and the copy of the next tile overlaps the other stages, which run in
+// in a shared buffer (mbarrier completion).  Its first FFT stage moves it to the work
+// buffer, and the copy of a later tile overlaps the other stages, which run in
 // place there.  The last FFT stage stays in registers: each thread owns E modes (one
 // pencil, E values of k_x) for the whole pencil block.
 //
@@ -752,6 +752,9 @@ struct XCombine {
   static_assert(BOXES * BOX_ROWS == N, "boxes must tile the x axis");
   static constexpr unsigned TILE_BYTES = (unsigned)(N * P * sizeof(float2));
   static constexpr int STAGES = fft_nstages(N);
+  // tile buffers: one where several CTAs per SM hide the copies, more for small meshes,
+  // whose few CTAs would wait for each (128^3 49.2 -> 46.5 us, 32^3 20.4 -> 19.6 us)
+  static constexpr int NBUF = N <= 128 ? 4 : 1;
   static constexpr int WK_ELEMS = lf_elems<N, P>();
   static constexpr int RL = fft_radix(N, STAGES - 1);  // last radix
   // resident CTAs per SM the register budget is set for (3 x 256 threads at 256^3, 512^3;
@@ -764,7 +767,7 @@ struct XCombine {
   // in one shell, then never meet in one instruction (same-address shared atomics are
   // served one after another); with fewer copies warp w adds into copy w mod nwb.
   static size_t smem(int nbins, int nwb) {
-    size_t b = TILE_BYTES + sizeof(float2) * WK_ELEMS;  // tile and work buffer
+    size_t b = NBUF * (size_t)TILE_BYTES + sizeof(float2) * WK_ELEMS;  // tile buffers and work buffer
     if (ELL > 0) b += TILE_BYTES;                       // A_0
     b += sizeof(float2) * 2 * N + sizeof(float) * N;    // twiddles, phases, windows
     b += sizeof(float) * 2 * nwb * SLOTS * nbins;       // float bins and their error terms
@@ -784,10 +787,11 @@ k_x_combine(const __grid_constant__ XMulti pm, int np_pad, int ngb, const short2
   constexpr int THREADS = XC::THREADS;
   constexpr bool COMP = x_horner<N, ELL>();
   extern __shared__ __align__(128) float2 smem_x[];
-  __shared__ __align__(8) unsigned long long bar;
+  __shared__ __align__(8) unsigned long long bar[XC::NBUF];
   __shared__ int s_fail;
   float2* T = smem_x;
-  float2* Wk = T + N * P;
+  constexpr int NBUF = XC::NBUF;
+  float2* Wk = T + NBUF * N * P;
   float2* sA0 = Wk + XC::WK_ELEMS;
   float2* tw = sA0 + (ELL > 0 ? N * P : 0);
   float2* phs = tw + N;
@@ -802,7 +806,7 @@ k_x_combine(const __grid_constant__ XMulti pm, int np_pad, int ngb, const short2
   }
   for (int k = tid; k < 2 * nwb * SLOTS * nbins; k += THREADS) wbin[k] = 0.f;
   if (tid == 0) {
-    mbar_init(&bar, 1);
+    for (int b = 0; b < NBUF; ++b) mbar_init(&bar[b], 1);
     s_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -816,12 +820,15 @@ k_x_combine(const __grid_constant__ XMulti pm, int np_pad, int ngb, const short2
     const int pen = (blockIdx.x + k * gridDim.x) * P;  // a block of P pencils lies in one pencil block
     const int row = ((mj * XC::NG + gi) * ngb + pen / GROUP_BLOCK) * N;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    mbar_expect_tx(&bar, XC::TILE_BYTES);
+    unsigned long long* bs = &bar[s % NBUF];
+    float2* dst = T + (s % NBUF) * N * P;
+    mbar_expect_tx(bs, XC::TILE_BYTES);
 #pragma unroll
     for (int bx = 0; bx < XC::BOXES; ++bx)
-      tma_load_2d(T + bx * XC::BOX_ROWS * P, gmap, pen % GROUP_BLOCK * 2, row + bx * XC::BOX_ROWS, &bar);
+      tma_load_2d(dst + bx * XC::BOX_ROWS * P, gmap, pen % GROUP_BLOCK * 2, row + bx * XC::BOX_ROWS, bs);
   };
-  if (tid == 0 && total > 0) issue(0);
+  if (tid == 0)
+    for (int q = 0; q < NBUF && q < total; ++q) issue(q);
   const int p = tid % P, tl = tid / P;
   const float m0 = (float)tl;
   // mode e of this thread: k_x = tl + koff(e), as a signed frequency tl + koff(e) - N past N / 2
@@ -864,14 +871,14 @@ k_x_combine(const __grid_constant__ XMulti pm, int np_pad, int ngb, const short2
 #pragma unroll
         for (int mj = 0; mj < M; ++mj) {
           float2 v[E];
-          if (!mbar_wait(&bar, s & 1, 1000000000LL)) s_fail = 1;  // 1 s
-          lf_first_stage<N, P>(T, Wk, p, tl);
+          if (!mbar_wait(&bar[s % NBUF], (s / NBUF) & 1, 1000000000LL)) s_fail = 1;  // 1 s
+          lf_first_stage<N, P>(T + (s % NBUF) * N * P, Wk, p, tl);
           __syncthreads();
           if (s_fail) {
             failed = true;
             break;
           }
-          if (tid == 0 && s + 1 < total) issue(s + 1);
+          if (tid == 0 && s + NBUF < total) issue(s + NBUF);
           LfMiddle<N, P, 1>::run(Wk, p, tl, tw);
           lf_last_stage<N, P>(Wk, p, tl, tw, v);  // (a barrier after its loads)
           ++s;
@@ -953,9 +960,10 @@ k_x_combine(const __grid_constant__ XMulti pm, int np_pad, int ngb, const short2
   if (failed) {
     if (tid == 0) {
       atomicExch(pm.err[blockIdx.y], 2);
-      // Copy s is the last one issued: wait for it by its own phase parity before the
-      // CTA's shared memory is released (bounded; every earlier copy has completed).
-      mbar_wait(&bar, s & 1, 100000000LL);
+      // Copies s .. s + NBUF - 1 are the last ones issued: wait for each by its own phase
+      // parity before the CTA's shared memory is released (bounded; every earlier copy
+      // has completed).
+      for (int q = s; q < s + NBUF && q < total; ++q) mbar_wait(&bar[q % NBUF], (q / NBUF) & 1, 100000000LL);
     }
     return;
   }
