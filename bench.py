@@ -174,15 +174,22 @@ FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 
 def fft_flops(cls, n, m, n_pencils, nzc, pairs=8, fields=16, groups=9):
     """Nominal FFT flops per launch (5 L log2 L per complex line of length L) of the
-    two transform kernels: the y,z stage transforms m N^2 lines along z per field
-    pair and m N nzc lines along y per basis field; the x stage m G lines per kept
-    pencil."""
+    two transform kernels: the y,z stage transforms m N^2 lines along z per pair of real
+    fields and m N nzc lines along y per field; the x stage m G lines per kept pencil.
+    The defaults are the 16 basis fields of l <= 4; YZ_LINES is what the library
+    transforms of them."""
     line = 5.0 * n * math.log2(n)
     if cls == "yz_stage":
         return line * (m * n * n * pairs + m * n * nzc * fields)
     if cls == "x_combine":
         return line * m * groups * n_pencils
     return 0.0
+
+
+# Lines that the y,z stage transforms for l <= 4: along z the five source fields in pairs
+# (F of two rows in one line), along y every basis field but F', which differs from F at
+# one node at most.
+YZ_LINES = {"pairs": 2.5, "fields": 15}
 
 
 # DRAM bytes (read + write) per launch that ncu measured for the current build of
@@ -417,10 +424,12 @@ def run_ours(args):
     dom = max(prof.items(), key=lambda kv: kv[1][1])[0]
     launches_dom = per_cls[dom][0]
     bytes_dom = kernel_bytes(dom, gal.n, ran.n, N_MESH, m, groups, n_pencils, launches_dom, None)
+    if dom in ("particle_count", "particle_bin"):
+        bytes_dom *= 2  # one launch takes both catalogues (kernel_bytes: per catalogue)
     avg_ms = per_cls[dom][1]
     peak, peak_src = _peaks()
     achieved = bytes_dom / (avg_ms / 1e3) / 1e9
-    flops_dom = fft_flops(dom, N_MESH, m, n_pencils, nzc)
+    flops_dom = fft_flops(dom, N_MESH, m, n_pencils, nzc, **(YZ_LINES if dom == "yz_stage" else {}))
     # the ncu DRAM table holds the headline workload in its tuned configuration only
     traffic = TRAFFIC if (args.workload == WORKLOAD and not args.no_tune) else {}
     b_alg = alg_bytes(gal.n, ran.n, N_MESH, m, groups, n_pencils)
