@@ -55,7 +55,7 @@ void free_all(Plan& p) {
   dfree(p.d_tw); dfree(p.d_twl); dfree(p.d_nodes); dfree(p.d_rel); dfree(p.d_relz); dfree(p.d_invw); dfree(p.d_phase);
   dfree(p.d_col_off); dfree(p.d_pencil); dfree(p.d_lut); dfree(p.d_shell);
   dfree(p.d_mesh); dfree(p.d_z); dfree(p.d_sync); dfree(p.d_g); dfree(p.d_acc); dfree(p.d_sums); dfree(p.d_result);
-  dfree(p.d_tile_count); dfree(p.d_tile_off); dfree(p.d_tile_cur); dfree(p.d_rec);
+  dfree(p.d_tile_count); dfree(p.d_tile_off); dfree(p.d_tile_cur); dfree(p.d_rec); dfree(p.d_codes);
   dfree(p.d_stage);
   dfree(p.d_rmesh); dfree(p.d_rsums);
   p.device_bytes = 0;
@@ -364,6 +364,10 @@ ys_status ensure_particles(Plan& p, int64_t total) {
     p.device_bytes -= (size_t)p.rec_cap * sizeof(float4) + 16;
     dfree(p.d_rec);
   }
+  if (p.d_codes) {
+    p.device_bytes -= (size_t)p.part_cap * sizeof(unsigned) + 16;
+    dfree(p.d_codes);
+  }
   // records per particle: up to 2 tiles per axis that has more than one tile, for
   // any scatter-tile shape the tuner may switch to
   int factor = 1;
@@ -372,9 +376,11 @@ ys_status ensure_particles(Plan& p, int64_t total) {
     for (int a = 0; a < 3; ++a) f *= std::min(t[a], p.n) < p.n ? 2 : 1;
     factor = std::max(factor, f);
   }
-  p.part_cap = total;
+  p.part_cap = 0;
   p.rec_cap = total * factor;
   if ((e = dalloc(p, p.d_rec, (size_t)p.rec_cap))) return cuda_fail(e);
+  if (p.n <= 256 && (e = dalloc(p, p.d_codes, (size_t)total))) return cuda_fail(e);
+  p.part_cap = total;
   return YS_OK;
 }
 

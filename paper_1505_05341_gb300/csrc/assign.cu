@@ -233,14 +233,34 @@ __device__ __forceinline__ Touched touched_tiles(float x, float y, float z, cons
   return r;
 }
 
-// Counting pass.  HIST: the tile counts go to a histogram in shared memory (ntiles
+// What the binning pass needs of a particle's tiles, kept by the counting pass in 32 bits:
+// the first tile (16 bits), two bits per axis (0: one tile, 1: the next one too, 2: the
+// first one of the axis too, across the periodic edge), and the inner flag.
+__device__ __forceinline__ unsigned pack_touched(const Touched& t) {
+  auto step = [](int d) { return d == 0 ? 0u : (d > 0 ? 1u : 2u); };
+  return (unsigned)t.first | step(t.dx) << 16 | step(t.dy) << 18 | step(t.dz) << 20 | (t.inner ? 1u << 22 : 0u);
+}
+__device__ __forceinline__ Touched unpack_touched(unsigned c, const Geom& g) {
+  Touched t;
+  auto delta = [](unsigned s, int stride, int tiles) { return s == 0u ? 0 : (s == 1u ? stride : -(tiles - 1) * stride); };
+  t.first = (int)(c & 0xffffu);
+  t.dx = delta(c >> 16 & 3u, g.tiles[1] * g.tiles[2], g.tiles[0]);
+  t.dy = delta(c >> 18 & 3u, g.tiles[2], g.tiles[1]);
+  t.dz = delta(c >> 20 & 3u, 1, g.tiles[2]);
+  t.inner = (c >> 22 & 1u) != 0u;
+  t.ok = true;
+  return t;
+}
+
+// Counting pass.  codes: where the aggregated binning pass finds each particle's tiles
+// (galaxies first, then randoms; nullptr: it locates them again).  HIST: the tile counts go to a histogram in shared memory (ntiles
 // counters), added to the global counts once per CTA at the end -- a few CTAs per SM and
 // a grid-stride loop, instead of one global atomic per (particle, tile) on counters that
 // every SM contends for.
 template <int KIND, int M, bool HIST, int NT>
 __global__ void __launch_bounds__(NT)
 k_particles(const __grid_constant__ Cats cats, Geom g, const float2* __restrict__ nodes,
-            unsigned* __restrict__ tile_count, double* __restrict__ sums, int ntiles) {
+            unsigned* __restrict__ tile_count, double* __restrict__ sums, int ntiles, unsigned* __restrict__ codes) {
   extern __shared__ unsigned s_hist[];
   if (HIST) {
     for (int t = threadIdx.x; t < ntiles; t += NT) s_hist[t] = 0u;
@@ -254,6 +274,7 @@ k_particles(const __grid_constant__ Cats cats, Geom g, const float2* __restrict_
   const float* __restrict__ pw = cats.w[is_ran];
   const float* __restrict__ pnbar = is_ran ? cats.nbar[1] : nullptr;
   const int64_t n = cats.n[is_ran];
+  if (codes && is_ran) codes += cats.n[0];
   ThreadSums ts;
   unsigned bad = 0;
   const int64_t stride = (int64_t)nblk * NT;
@@ -277,6 +298,7 @@ k_particles(const __grid_constant__ Cats cats, Geom g, const float2* __restrict_
       const float x = xs[u], y = ys[u], z = zs[u], w = ws[u];
       const Touched tt = touched_tiles<KIND, M>(x, y, z, g, nodes);
       bad += tt.ok ? 0u : 1u;
+      if (codes) codes[base + u * stride] = pack_touched(tt);
       ts.kahan(0, w);
       ts.kahan(1, w * w);
       if (pnbar) ts.kahan(2, w * w * nbs[u]);
@@ -310,16 +332,19 @@ __device__ __forceinline__ float catalogue_scale(int is_ran, double alpha_cfg, c
 // particles per tile in shared memory, reserves each tile's range with one global
 // atomic, and hands out the slots from shared-memory cursors.  One global atomic per
 // record serialises on the tiles' cursors when there are few of them: 6.6e6 particles
-// on the 512 tiles of a 128^3 mesh took 790 us.
+// on the 512 tiles of a 128^3 mesh took 790 us, 151 us now.  CODES: the tiles come from the
+// counting pass (4 bytes per particle instead of two locates; counting and binning
+// together 333 -> 298 us on the 256^3 cone, 243 -> 236 at 128^3).
 // Many tiles (k_bin): a chunk would hold about one record per tile, so each record takes
 // its own global atomic; each thread takes U particles per iteration, whose loads and
 // first-tile cursor atomics are independent, so that their latencies overlap.
 constexpr int BIN_AGG_TILES = 4096;
 constexpr int BIN_AGG_NT = 512;
 
-template <int KIND, int M>
+template <int KIND, int M, bool CODES>
 __global__ void __launch_bounds__(BIN_AGG_NT)
-k_bin_agg(const __grid_constant__ Cats cats, int per_thread, Geom g, const float2* __restrict__ nodes, int ntiles,
+k_bin_agg(const __grid_constant__ Cats cats, int per_thread, Geom g, const float2* __restrict__ nodes,
+          const unsigned* __restrict__ codes, int ntiles,
           const unsigned* __restrict__ off, unsigned* __restrict__ tile_left, unsigned* __restrict__ tile_cur,
           float4* __restrict__ rec, const double* __restrict__ sums, double alpha_cfg) {
   extern __shared__ unsigned s_cur[];  // [2][ntiles]: interior, border
@@ -335,11 +360,12 @@ k_bin_agg(const __grid_constant__ Cats cats, int per_thread, Geom g, const float
   py += first;
   pz += first;
   if (pw) pw += first;
+  if (CODES) codes += first + (is_ran ? cats.n[0] : 0);
   const int last = (int)min(cats.n[is_ran] - first, (int64_t)BIN_AGG_NT * per_thread);
   __syncthreads();
 #pragma unroll 2
   for (int i = threadIdx.x; i < last; i += BIN_AGG_NT) {
-    const Touched tt = touched_tiles<KIND, M>(px[i], py[i], pz[i], g, nodes);
+    const Touched tt = CODES ? unpack_touched(codes[i], g) : touched_tiles<KIND, M>(px[i], py[i], pz[i], g, nodes);
     unsigned* cnt = s_cur + (tt.inner ? 0 : ntiles);
     atomicAdd(cnt + tt.first, 1u);
     if (!tt.inner) tt.others([&](int tile) { atomicAdd(cnt + tile, 1u); });
@@ -355,7 +381,7 @@ k_bin_agg(const __grid_constant__ Cats cats, int per_thread, Geom g, const float
 #pragma unroll 2
   for (int i = threadIdx.x; i < last; i += BIN_AGG_NT) {
     const float4 q = make_float4(px[i], py[i], pz[i], (pw ? pw[i] : 1.f) * wscale);
-    const Touched tt = touched_tiles<KIND, M>(q.x, q.y, q.z, g, nodes);
+    const Touched tt = CODES ? unpack_touched(codes[i], g) : touched_tiles<KIND, M>(q.x, q.y, q.z, g, nodes);
     unsigned* cur = s_cur + (tt.inner ? 0 : ntiles);
     rec[atomicAdd(cur + tt.first, 1u)] = q;
     if (!tt.inner) tt.others([&](int tile) { rec[atomicAdd(cur + tile, 1u)] = q; });
@@ -923,7 +949,8 @@ cudaError_t run_count(Plan& p, const ys_catalog& gal, const ys_catalog& ran, int
   int grid = blocks_for(total, NT, std::max(1, per) * sms);
   const Cats cats = make_cats(gal, ran, grid);
   LaunchScope ls(p, 0);
-  kern<<<grid, NT, smem, p.stream>>>(cats, p.geom, p.d_nodes, p.d_tile_count, p.d_sums, p.ntiles);
+  kern<<<grid, NT, smem, p.stream>>>(cats, p.geom, p.d_nodes, p.d_tile_count, p.d_sums, p.ntiles,
+                                       p.ntiles <= BIN_AGG_TILES ? p.d_codes : nullptr);
   return cudaGetLastError();
 }
 
@@ -973,8 +1000,9 @@ cudaError_t run_assign(Plan& p, const ys_catalog& gal, const ys_catalog& ran, co
     grid = cats.blocks0 + (int)((ran.n + chunk - 1) / chunk);
     const size_t smem = 2 * sizeof(unsigned) * (size_t)p.ntiles;
     LaunchScope ls(p, 2);
-    k_bin_agg<KIND, M><<<grid, BIN_AGG_NT, smem, st>>>(cats, per_thread, p.geom, p.d_nodes, p.ntiles, p.d_tile_off,
-                                                       p.d_tile_count, p.d_tile_cur, p.d_rec, p.d_sums, p.cfg.alpha);
+    auto bin = p.d_codes ? k_bin_agg<KIND, M, true> : k_bin_agg<KIND, M, false>;
+    bin<<<grid, BIN_AGG_NT, smem, st>>>(cats, per_thread, p.geom, p.d_nodes, p.d_codes, p.ntiles, p.d_tile_off,
+                                        p.d_tile_count, p.d_tile_cur, p.d_rec, p.d_sums, p.cfg.alpha);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
   } else if (total > 0) {
     constexpr int U = 2;

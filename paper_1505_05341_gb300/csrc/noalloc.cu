@@ -101,15 +101,18 @@ ys_status assign_noalloc(Plan& p, const ys_catalog& gal, const ys_catalog& ran, 
   unsigned* s_off = p.d_tile_off;
   unsigned* s_cur = p.d_tile_cur;
   float4* s_rec = p.d_rec;
+  unsigned* s_codes = p.d_codes;
   p.d_tile_count = reinterpret_cast<unsigned*>(b);
   p.d_tile_off = reinterpret_cast<unsigned*>(b + off_off);
   p.d_tile_cur = reinterpret_cast<unsigned*>(b + off_cur);
   p.d_rec = reinterpret_cast<float4*>(b + off_rec);
+  p.d_codes = nullptr;  // sized for other catalogues, if at all: the tiles are located twice
   e = launch_assign(p, gal, ran);
   p.d_tile_count = s_count;
   p.d_tile_off = s_off;
   p.d_tile_cur = s_cur;
   p.d_rec = s_rec;
+  p.d_codes = s_codes;
   if (e != cudaSuccess) {
     why = cudaGetErrorString(e);
     return YS_ERR_CUDA;

@@ -122,6 +122,8 @@ struct Plan {
   unsigned* d_tile_count = nullptr;  // [ntiles] records per tile, counted down as border records are placed
   unsigned* d_tile_off = nullptr;    // [ntiles + 1] first record of each tile's list
   unsigned* d_tile_cur = nullptr;    // [ntiles] front cursors; after binning the ends of the interior records
+  unsigned* d_codes = nullptr;   // [part_cap] tiles of each particle, from the counting to the binning pass
+                                 // (nullptr: meshes above 256^3, and the no-allocation path)
   float4* d_rec = nullptr;       // [rec_cap] (x, y, z, signed weight) per (particle, tile)
   // shared randoms (ys_randoms_cache): sum_ran w W per mesh node, and its FP64 sums
   float* d_rmesh = nullptr;      // [m][n][n][n]
