@@ -195,10 +195,9 @@ YZ_LINES = {"pairs": 2.5, "fields": 15}
 # DRAM bytes (read + write) per launch that ncu measured for the current build of
 # each kernel on the 512^3 survey workload in its tuned launch configuration (one-pass
 # dram__bytes_{read,write}.sum capture; profiles/dram_traffic_shell512_tsc_il.md).
-# Remove an entry when its kernel changes.  particle_count and particle_bin: the mean
-# of the galaxy and random launches.
-TRAFFIC = {"yz_stage": 8.86e9, "x_combine": 5.77e9, "tile_deposit": 2.50e9, "particle_bin": 1.26e9,
-           "particle_count": 0.58e9}
+# Remove an entry when its kernel changes.
+TRAFFIC = {"yz_stage": 7.18e9, "x_combine": 5.81e9, "tile_deposit": 2.50e9, "particle_bin": 2.52e9,
+           "particle_count": 1.16e9}
 
 
 def kernel_bytes(cls, n_gal, n_ran, n, m, groups, n_pencils, launches_per_step, batch_planes):
