@@ -2,6 +2,7 @@
 // allocation), the assign / measure entry points, and the final Eqs. (6)-(8).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -301,22 +302,20 @@ ys_status build_tables(Plan& p) {
   std::frexp(far, &unit);
   std::vector<float2> rel(rel64.size());
   for (size_t i = 0; i < rel.size(); ++i) {
-    const float v = (float)std::ldexp(rel64[i], -unit);
-    const int ex = v != 0.f ? std::max(-30, std::ilogb(v)) : -30;
-    rel[i] = make_float2(v, std::ldexp(1.f, -ex));
+    float v = (float)std::ldexp(rel64[i], -unit);
+    if (std::fabs(v) < std::ldexp(1.f, YZ_EXP_MIN)) v = 0.f;
+    rel[i] = make_float2(v, std::ldexp(1.f, -(v != 0.f ? std::ilogb(v) : YZ_EXP_MIN)));
   }
-  // the node that carries no line-of-sight weight, if the observer sits on one
+  // the node at r = 0, which carries no line-of-sight weight, if the observer sits on one
   for (int j = 0; j < p.m; ++j) {
     int at[3];
-    float r2 = 0.f;
+    bool hit = true;
     for (int a = 0; a < 3; ++a) {
       const float2* r = rel.data() + ((size_t)j * 3 + a) * n;
-      at[a] = 0;
-      for (int i = 1; i < n; ++i)
-        if (std::fabs(r[i].x) < std::fabs(r[at[a]].x)) at[a] = i;
-      r2 += r[at[a]].x * r[at[a]].x;
+      at[a] = (int)(std::find_if(r, r + n, [](const float2& v) { return v.x == 0.f; }) - r);
+      hit = hit && at[a] < n;
     }
-    if (r2 <= YZ_R2_MIN)
+    if (hit)
       for (int a = 0; a < 3; ++a) p.org[j][a] = at[a];
   }
   cudaError_t e;

@@ -48,12 +48,14 @@ namespace ys {
 // Ranges.  r is held in units of a power of two near the largest |r| component (the
 // monomials have degree 0, so the unit cancels exactly).  The sources of one row are
 // scaled by rho^(d - c) and X, Y divided by rho, rho = max(2^floor(log2 |X|),
-// 2^floor(log2 |Y|)), at least 2^-30.  With rho within a factor of two of the row's
+// 2^floor(log2 |Y|)), at least 2^-90.  With rho within a factor of two of the row's
 // distance from the z axis through the observer, both sources of a degree, which share
 // a complex line, and the factors (X / rho)^a (Y / rho)^b are O(F) and O(1): neither
 // source's rounding shows in the other's field (one rho per x-plane instead lost 3.5
 // bits next to the observer's planes), and nothing overflows next to the observer.
-// Nodes with |r|^2 <= YZ_R2_MIN carry no line-of-sight weight, as the node at r = 0.
+// (|r| / rho)^2 is at least 1 except at r = 0, the one node without a line-of-sight weight
+// (its components are 0, see YZ_EXP_MIN); it is cut at 2^125, where the sources are at most
+// 2^-35 F, so that rows much nearer the axis than 2^-62 stay finite.
 // Line l of a column item: basis field 0 (l = 0) or l + 1 (F' is left out); its source
 // field and the exponents of X and Y.
 template <int ELL>
@@ -96,7 +98,7 @@ template <int ELL> __constant__ constexpr YLines<ELL> kYLines{};
 
 struct YZParams {
   const float* mesh;     // [m][N][N][N]
-  const float2* rel;     // [m][2][N] x, y of node - observer v, and 2^-floor(log2 |v|) (at most 2^30)
+  const float2* rel;     // [m][2][N] x, y of node - observer v, and 2^-floor(log2 |v|) (2^90 for v = 0)
   const float* relz;     // [m][N] z of node - observer
   const float2* tw;      // [TWN] twiddles of the line transforms (LineFft<N>)
   float2* ring;          // [S][nzc][NF][N]
@@ -236,14 +238,13 @@ __device__ __forceinline__ bool row_item(float2* S, const float2* tws, const flo
         const float2 Yc = rely[row0 + r];
         irho = fminf(X.y, Yc.y);  // a power of two: every product with it is exact
         const float xs = X.x * irho, ys = Yc.x * irho, xy2 = fmaf(xs, xs, ys * ys);
-        const float r2_min = YZ_R2_MIN * irho * irho;
         const float* frow = plane + (size_t)(row0 + r) * N + t;
 #pragma unroll
         for (int k = 0; k < R1; ++k) f[k] = frow[k * TPL];
 #pragma unroll
         for (int k = 0; k < R1; ++k) {
           const float zs = relz[t + k * TPL] * irho, r2 = fmaf(zs, zs, xy2);  // (|r| / rho)^2
-          i2[k] = r2 > r2_min ? recip_nr(r2) : 0.f;
+          i2[k] = r2 > 0.f ? recip_nr(fminf(r2, 0x1p125f)) : 0.f;
           f[k] *= 0.5f;  // for line_halves
         }
       }

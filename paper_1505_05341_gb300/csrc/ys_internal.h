@@ -50,11 +50,11 @@ struct Geom {
   int tshift[3];    // its logarithm
 };
 
-// Nodes with |r|^2 (r from the observer, in units of the mesh's largest |r| component
-// rounded up to a power of two) at most this, 2^-60, carry no line-of-sight weight: at
-// 2^-30 of the mesh's extent the direction is rounding noise, and one node at most is
-// that near.
-constexpr float YZ_R2_MIN = 8.673617379884035e-19f;
+// Components of r (node - observer, in units of the mesh's largest |r| component rounded up
+// to a power of two) below 2^YZ_EXP_MIN are held as 0, and only a node whose three components
+// are 0 carries no line-of-sight weight.  2^-90 of the mesh's extent is far below the
+// resolution of double coordinates; the limit keeps the scale factors 2^90 inside float.
+constexpr int YZ_EXP_MIN = -90;
 
 // Pencils per block of the grouped transforms d_g: pencil p of plane x sits in row
 // (block p / GROUP_BLOCK, x) at p % GROUP_BLOCK.  An x-stage tile (a few pencils, every x)
