@@ -168,8 +168,10 @@ template <bool GRAD>
 __device__ __forceinline__ void forward_tile(MlpSmem& s, const float* __restrict__ X, int64_t r0, int nr,
                                              const Block& t, float (&gp)[3][4][4]) {
   for (int k = threadIdx.x; k < IN * MLP_ROWS; k += MLP_THREADS) {
+    // rows past the end repeat the last row: their deltas are zero, and activations that a
+    // made-up input might overflow would turn zero deltas into NaN
     const int r = k / IN, f = k % IN;
-    s.x[f * RS + r] = r < nr ? X[r0 * IN + k] : 0.f;
+    s.x[f * RS + r] = X[(r0 + min(r, nr - 1)) * IN + f];
   }
   __syncthreads();
   float acc[4][4];
