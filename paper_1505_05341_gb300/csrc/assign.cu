@@ -60,38 +60,65 @@ __device__ __forceinline__ int block_catalogue(const Cats& c, int& bid, int& nbl
   return k;
 }
 
-// (s, c) += (s2, c2) for float sums with their collected rounding errors (TwoSum).
-__device__ __forceinline__ void pair_add(float& s, float& c, float s2, float c2) {
-  const float t = s + s2, bb = t - s;
-  c += c2 + ((s - (t - bb)) + (s2 - bb));
-  s = t;
+// a + b and its rounding error (TwoSum, error-free).
+__device__ __forceinline__ float two_sum(float a, float b, float& err) {
+  const float t = a + b, bb = t - a;
+  err = (a - (t - bb)) + (b - bb);
+  return t;
 }
 
-// Sums of w, w^2 and w^2 nbar over this thread's particles: compensated float (Kahan).
+// Sums of w, w^2 and w^2 nbar over this thread's particles: float sums s, and in c the exact
+// rounding errors of every addition and product.
 struct ThreadSums {
   float s[3] = {0.f, 0.f, 0.f}, c[3] = {0.f, 0.f, 0.f};
-  __device__ __forceinline__ void kahan(int k, float v) {
-    const float y = v - c[k], t = s[k] + y;
-    c[k] = (t - s[k]) - y;
-    s[k] = t;
+  __device__ __forceinline__ float add(int k, float v) {
+    float err;
+    s[k] = two_sum(s[k], v, err);
+    return err;
+  }
+  // (__fmul_rn: a product contracted into the addition would not be the one whose error is taken)
+  __device__ __forceinline__ void particle(float w, const float* nbar, float nb) {
+    c[0] += add(0, w);
+    const float p = __fmul_rn(w, w), e = fmaf(w, w, -p);
+    c[1] += add(1, p) + e;
+    if (nbar) {
+      const float q = __fmul_rn(p, nb);
+      c[2] += add(2, q) + fmaf(e, nb, fmaf(p, nb, -q));
+    }
   }
 };
 
 // Adds the block's sums (and its count of particles outside the box) to the catalogue
-// sums.  Threads meet in compensated float pairs (~2^-46; an FP64 shuffle tree of three
-// sums took 15 x 16 cycles of the SM per warp) and each CTA makes one FP64 atomic per
-// sum: per-warp atomics on the three addresses alone took ~30 us per catalogue.
+// sums.  The lanes of a warp meet in expansions of three floats (~2^-70, below an FP64
+// addition's rounding; an FP64 shuffle tree of three sums took 15 x 16 cycles of the SM per
+// warp), scaled by 2^-10 where 32 of the sums might overflow; the warps meet in FP64, and
+// each CTA makes one FP64 atomic per sum: per-warp atomics on the three addresses alone
+// took ~30 us per catalogue.  FKP-weighted catalogues of 6e6 to 3e7 particles: alpha, I and
+// S / I are within 5e-15 of FP64 sums (4e-11 to 8e-11 with Kahan sums, which round every term).
 template <int NT>
 __device__ __forceinline__ void block_sums(ThreadSums& ts, unsigned bad, int is_ran, double* __restrict__ sums) {
-  __shared__ float2 red[NT / 32][3];
+  __shared__ float4 red[3][NT / 32];  // sum, its two tails, scale
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    float s = ts.s[k], c = -ts.c[k];
+    if (!is_ran && k == 2) break;
+    float s = ts.s[k], c = ts.c[k], e = 0.f, scale = 1.f;
+    if (__any_sync(0xffffffffu, !(fabsf(s) < 0x1p120f))) {
+      scale = 1024.f;
+      s *= 0x1p-10f;
+      c *= 0x1p-10f;
+    }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-      pair_add(s, c, __shfl_xor_sync(0xffffffffu, s, o), __shfl_xor_sync(0xffffffffu, c, o));
-    if (lane == 0) red[wid][k] = make_float2(s, c);
+    for (int o = 16; o > 0; o >>= 1) {
+      float e1, e2, e3;
+      const float s2 = __shfl_xor_sync(0xffffffffu, s, o), c2 = __shfl_xor_sync(0xffffffffu, c, o);
+      e += __shfl_xor_sync(0xffffffffu, e, o);
+      s = two_sum(s, s2, e1);
+      c = two_sum(c, c2, e2);
+      c = two_sum(c, e1, e3);
+      e += e2 + e3;
+    }
+    if (lane == 0) red[k][wid] = make_float4(s, c, e, scale);
   }
   const int nbad = __syncthreads_or(bad != 0);
   if (nbad) {
@@ -100,12 +127,18 @@ __device__ __forceinline__ void block_sums(ThreadSums& ts, unsigned bad, int is_
     for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
     if (lane == 0 && tot) atomicAdd(&sums[SUM_BAD], (double)tot);
   }
-  if (threadIdx.x < 3) {
-    const int k = threadIdx.x;
-    float s = red[0][k].x, c = red[0][k].y;
-    for (int q = 1; q < NT / 32; ++q) pair_add(s, c, red[q][k].x, red[q][k].y);
-    const int slot = is_ran ? (k == 0 ? SUM_WR : (k == 1 ? SUM_WR2 : SUM_WR2N)) : (k == 0 ? SUM_WG : SUM_WG2);
-    if (is_ran || k < 2) atomicAdd(&sums[slot], (double)s + (double)c);
+  if (wid == 0) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      if (!is_ran && k == 2) break;
+      const float4 r = lane < NT / 32 ? red[k][lane] : make_float4(0.f, 0.f, 0.f, 1.f);
+      double v = ((double)r.x + ((double)r.y + (double)r.z)) * (double)r.w;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+        if (o < NT / 32) v += __shfl_xor_sync(0xffffffffu, v, o);
+      const int slot = is_ran ? (k == 0 ? SUM_WR : (k == 1 ? SUM_WR2 : SUM_WR2N)) : (k == 0 ? SUM_WG : SUM_WG2);
+      if (lane == 0) atomicAdd(&sums[slot], v);
+    }
   }
 }
 
@@ -299,9 +332,7 @@ k_particles(const __grid_constant__ Cats cats, Geom g, const float2* __restrict_
       const Touched tt = touched_tiles<KIND, M>(x, y, z, g, nodes);
       bad += tt.ok ? 0u : 1u;
       if (codes) codes[base + u * stride] = pack_touched(tt);
-      ts.kahan(0, w);
-      ts.kahan(1, w * w);
-      if (pnbar) ts.kahan(2, w * w * nbs[u]);
+      ts.particle(w, pnbar, nbs[u]);
       auto count = [&](int tile) {
         if constexpr (HIST) atomicAdd(&s_hist[tile], 1u);
         else atomicAdd(&tile_count[tile], 1u);
@@ -767,7 +798,9 @@ __global__ void k_ran_sums(const float* __restrict__ w, const float* __restrict_
   }
 }
 
-// Catalogue sums of Eqs. (1) and (3) without the counting pass.
+// Catalogue sums of Eqs. (1) and (3) without the counting pass: four CTAs per SM with eight
+// particles in flight per thread (with eight CTAs and four the meeting of the threads, twice
+// as much, takes 1 us longer).
 __global__ void __launch_bounds__(THREADS)
 k_sums(const __grid_constant__ Cats cats, double* __restrict__ sums) {
   int bid, nblk;
@@ -777,12 +810,18 @@ k_sums(const __grid_constant__ Cats cats, double* __restrict__ sums) {
   const int64_t n = cats.n[is_ran];
   ThreadSums ts;
   const int64_t stride = (int64_t)nblk * THREADS;
-#pragma unroll 4
-  for (int64_t i = (int64_t)bid * THREADS + threadIdx.x; i < n; i += stride) {
-    const float w = pw ? pw[i] : 1.f;
-    ts.kahan(0, w);
-    ts.kahan(1, w * w);
-    if (pnbar) ts.kahan(2, w * w * pnbar[i]);
+  constexpr int U = 8;  // particles per iteration, whose loads are issued together
+  for (int64_t base = (int64_t)bid * THREADS + threadIdx.x; base < n; base += U * stride) {
+    float w[U], nb[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t i = min(base + u * stride, n - 1);
+      w[u] = pw ? pw[i] : 1.f;
+      nb[u] = pnbar ? pnbar[i] : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (base + u * stride < n) ts.particle(w[u], pnbar, nb[u]);
   }
   block_sums<THREADS>(ts, 0u, is_ran, sums);
 }
@@ -920,7 +959,7 @@ cudaError_t run_direct(Plan& p, const ys_catalog& gal, const ys_catalog& ran) {
   const int64_t total = gal.n + ran.n;
   if (total == 0) return cudaSuccess;
   {
-    int grid = blocks_for(total, 4 * THREADS, sms * 8);
+    int grid = blocks_for(total, 8 * THREADS, sms * 4);
     const Cats cats = make_cats(gal, ran, grid);
     LaunchScope ls(p, 0);
     k_sums<<<grid, THREADS, 0, st>>>(cats, p.d_sums);
