@@ -17,18 +17,21 @@
 // sums in registers; points stream through shared memory in chunks that every thread
 // reads as broadcasts.  Positions are 32-bit fixed-point fractions of the box,
 // u = (x - box_min) / L, so the phase k.x = 2 pi m.u is taken mod one turn exactly by
-// integer multiply-adds; only the final angle in [-pi, pi) is rounded.  The group's
-// middle mode takes sine and cosine of its phase, the others multiply by the point's
-// e^{-2 pi i j u_z}, j = +-1, +-2, formed once per point the same way.  SG_BLOCK terms of
-// a sum are added in float, and the block's sum goes into a compensated float sum
-// (TwoSum); CTAs that split the points add their sums into FP64 per-mode accumulators,
-// and a second kernel forms the shell sums in FP64.
+// integer multiply-adds.  The group's middle mode takes sine and cosine of its phase
+// (cis_minus: beyond the angle's float rounding), the others multiply by the point's
+// e^{-2 pi i j u_z}, j = +-1, +-2, formed once per point in FP64.  Every term of A_0 and of the
+// top-hat sum goes into a compensated float sum (add_comp); of A_2, A_4, .. SG_BLOCK terms
+// are added in float first.  CTAs that split the points add their sums into FP64 per-mode
+// accumulators, and a second kernel forms the shell sums in FP64.
 //
-// What bounds the mode kernel: FP32 issue, about 35 instructions per mode and point at
-// l_max = 4 (105 with one sincospif and six compensated adds per mode and point).  The sums
-// carry (m . r_hat)^n, normalised in FP64 afterwards: with k_hat in float its rounding was
-// common to all points.  Against FP64, over eight catalogues: P_2 and P_4 are off by 1e-8
-// to 2e-7 (7e-8 to 9e-7 before), P_0 by 2e-9 to 9e-9 (1e-9 to 5e-9 before).
+// What bounds the mode kernel: the FP32 pipes and issue, about 30 instructions per mode and
+// point at l_max = 4, the sums in packed pairs (105 with one sincospif and six scalar
+// compensated adds per mode and point).  The sums carry (m . r_hat)^n, normalised in FP64
+// afterwards: with k_hat in float its rounding was common to all points.  Against FP64, over
+// 10 to 40 catalogues and lattices of 20 to 64: P_2 and P_4 are off by 0.3 to 0.5 times what
+// one sincospif and one compensated add per term give, P_0 and the wedges by 0.8 to 1.1 times
+// (with the angles rounded to float and A_0 summed in blocks 1.2 to 2.0 times): 4.7e-8 rms a
+// term, 7.2e-8 then.
 // 68 000 modes of a 64^3 lattice, 120 000 points: 26.9 -> 9.8 ms a call.
 #include <cuda_runtime.h>
 
@@ -38,6 +41,7 @@
 #include <string>
 #include <vector>
 
+#include "fft.cuh"
 #include "ys_internal.h"
 
 namespace ys {
@@ -71,16 +75,12 @@ struct SgGroup {
   int first;
 };
 
-__device__ __forceinline__ float two_sum_err(float a, float b) {
-  const float s = a + b;
-  const float bb = s - a;
-  return (a - (s - bb)) + (b - bb);
-}
-
-// s += v with its exact rounding error added to c.
-__device__ __forceinline__ void add_comp(float& s, float& c, float v) {
-  const float t = s + v;
-  c += two_sum_err(s, v);
+// s += v with the rounding error added to c, both components (Fast2Sum: exact where |s| >= |v|,
+// else off by an ulp of v at most; over a walk of 64 to 1024 terms that leaves 3e-9 to 5e-9 of
+// a term per term, a tenth of the terms' own rounding, for 4 instructions instead of 7).
+__device__ __forceinline__ void add_comp(float2& s, float2& c, float2 v) {
+  const float2 t = cadd(s, v);
+  c = cadd(c, csub(v, csub(t, s)));
   s = t;
 }
 
@@ -124,11 +124,22 @@ __device__ __forceinline__ void unit3(double x, double y, double z, float (&o)[3
   o[2] = (float)(z * inv);
 }
 
-// The phase of `turn` (units of 2^-32 turns) as e^{-2 pi i turn}.
-__device__ __forceinline__ float2 cis_minus(uint32_t turn) {
+// w e^{-2 pi i turn}, turn in units of 2^-32.  The angle's leading 24 bits are exact in float;
+// the rest, at most 1.9e-7, is applied to first order (an angle rounded to float is off by up
+// to 9.4e-8, more than all other roundings of the result).
+__device__ __forceinline__ float2 cis_minus(uint32_t turn, float w) {
+  const uint32_t hi = (turn + 128u) & ~255u;
   float sn, cs;
-  sincospif((float)(int32_t)turn * 4.656612873077393e-10f, &sn, &cs);  // angle / pi in [-1, 1)
-  return make_float2(cs, -sn);
+  sincospif((float)(int32_t)hi * 4.656612873077393e-10f, &sn, &cs);  // angle / pi in [-1, 1)
+  const float d = w * ((float)(int32_t)(turn - hi) * 1.4629180792671596e-9f);  // pi 2^-31
+  return make_float2(fmaf(w, cs, -d * sn), -fmaf(w, sn, d * cs));
+}
+
+// e^{-2 pi i turn} from FP64: the points' rotations, which four of a group's five modes share.
+__device__ __forceinline__ float2 cis_minus64(uint32_t turn) {
+  double sn, cs;
+  sincospi((double)(int32_t)turn * 4.656612873077393e-10, &sn, &cs);
+  return make_float2((float)cs, (float)-sn);
 }
 
 // Catalogue particles as points: galaxies +w, randoms -alpha w.
@@ -148,8 +159,8 @@ __global__ void k_sg_points_cat(const float* __restrict__ x, const float* __rest
   q.sw = (float)(sgn * (w ? (double)w[i] : 1.0));
   unit3(px - ox, py - oy, pz - oz, q.rh);
   q.pad = 0.f;
-  q.w1 = cis_minus(q.u[2]);
-  q.w2 = cis_minus(2u * q.u[2]);
+  q.w1 = cis_minus64(q.u[2]);
+  q.w2 = cis_minus64(2u * q.u[2]);
   out[i] = q;
 }
 
@@ -173,13 +184,9 @@ __global__ void k_sg_points_mesh(const float* __restrict__ mesh, int n, int j, i
   q.sw = f * scale;
   unit3(rel_x0 + (ix + s) * H, rel_y0 + (iy + s) * H, rel_z0 + (iz + s) * H, q.rh);
   q.pad = 0.f;
-  q.w1 = cis_minus(q.u[2]);
-  q.w2 = cis_minus(2u * q.u[2]);
+  q.w1 = cis_minus64(q.u[2]);
+  q.w2 = cis_minus64(2u * q.u[2]);
   out[atomicAdd(count, 1u)] = q;
-}
-
-__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-  return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
 
 // Per-mode sums over the points of this CTA's split (blockIdx.y); FP64 atomics into
@@ -214,11 +221,11 @@ __global__ void __launch_bounds__(SG_THREADS) k_sg_modes(const SgGroup* __restri
   }
   constexpr int NM = ELL >= 6 ? 4 : ELL / 2 + 1;  // A_0, A_2, ..
   constexpr int NC = NM + (WEDGE ? 1 : 0);
-  float sre[SG_GROUP][NC], sim[SG_GROUP][NC], cre[SG_GROUP][NC], cim[SG_GROUP][NC];
+  float2 S[SG_GROUP][NC], C[SG_GROUP][NC];
 #pragma unroll
   for (int j = 0; j < SG_GROUP; ++j)
 #pragma unroll
-    for (int c = 0; c < NC; ++c) sre[j][c] = sim[j][c] = cre[j][c] = cim[j][c] = 0.f;
+    for (int c = 0; c < NC; ++c) S[j][c] = C[j][c] = make_float2(0.f, 0.f);
   for (int64_t base = p_lo; base < p_hi; base += SG_CHUNK) {
     const int cnt = (int)std::min<int64_t>(SG_CHUNK, p_hi - base);
     __syncthreads();
@@ -234,13 +241,12 @@ __global__ void __launch_bounds__(SG_THREADS) k_sg_modes(const SgGroup* __restri
       for (int b = 0; b < SG_BLOCK; ++b) {
         const SgPoint& q = s_pts[i + b];
         // one turn = 2^32: the phase m.u mod 1 is exact in wrapping integer arithmetic
-        const float2 c = cis_minus((uint32_t)(int)g.mx * q.u[0] + (uint32_t)(int)g.my * q.u[1] + (uint32_t)mid * q.u[2]);
-        e[b] = make_float2(q.sw * c.x, q.sw * c.y);
+        e[b] = cis_minus((uint32_t)(int)g.mx * q.u[0] + (uint32_t)(int)g.my * q.u[1] + (uint32_t)mid * q.u[2], q.sw);
         d[b] = fmaf(fx, q.rh[0], fy * q.rh[1]);
       }
 #pragma unroll
       for (int j = 0; j < SG_GROUP; ++j) {
-        float pr[NC], pi[NC];  // the block's plain sums
+        [[maybe_unused]] float2 p[NM];  // the block's plain sums of A_2, A_4, ..
 #pragma unroll
         for (int b = 0; b < SG_BLOCK; ++b) {
           const SgPoint& q = s_pts[i + b];
@@ -250,30 +256,25 @@ __global__ void __launch_bounds__(SG_THREADS) k_sg_modes(const SgGroup* __restri
             const float2 w = (o == 1 || o == -1) ? q.w1 : q.w2;
             t = cmul(t, o > 0 ? w : make_float2(w.x, -w.y));
           }
-          pr[0] = b == 0 ? t.x : pr[0] + t.x;
-          pi[0] = b == 0 ? t.y : pi[0] + t.y;
-          if constexpr (NC > 1) {
+          add_comp(S[j][0], C[j][0], t);
+          if constexpr (NM > 1) {
             const float md = fmaf((float)(g.mz + j), q.rh[2], d[b]), md2 = md * md;  // m . r_hat
             float f = md2;
 #pragma unroll
             for (int c = 1; c < NM; ++c) {
-              pr[c] = b == 0 ? f * t.x : fmaf(f, t.x, pr[c]);
-              pi[c] = b == 0 ? f * t.y : fmaf(f, t.y, pi[c]);
+              const float2 ff = make_float2(f, f);
+              p[c] = b == 0 ? __fmul2_rn(ff, t) : __ffma2_rn(ff, t, p[c]);
               f *= md2;
             }
-            if constexpr (WEDGE) {
-              const float mu = fmaf(kh[j][0], q.rh[0], fmaf(kh[j][1], q.rh[1], kh[j][2] * q.rh[2]));
-              const bool in = fabsf(mu) <= 0.5f;
-              pr[NC - 1] = (b == 0 ? 0.f : pr[NC - 1]) + (in ? t.x : 0.f);
-              pi[NC - 1] = (b == 0 ? 0.f : pi[NC - 1]) + (in ? t.y : 0.f);
-            }
+          }
+          if constexpr (WEDGE) {
+            const float mu = fmaf(kh[j][0], q.rh[0], fmaf(kh[j][1], q.rh[1], kh[j][2] * q.rh[2]));
+            const bool in = fabsf(mu) <= 0.5f;
+            add_comp(S[j][NC - 1], C[j][NC - 1], make_float2(in ? t.x : 0.f, in ? t.y : 0.f));
           }
         }
 #pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          add_comp(sre[j][c], cre[j][c], pr[c]);
-          add_comp(sim[j][c], cim[j][c], pi[c]);
-        }
+        for (int c = 1; c < NM; ++c) add_comp(S[j][c], C[j][c], p[c]);
       }
     }
   }
@@ -285,8 +286,8 @@ __global__ void __launch_bounds__(SG_THREADS) k_sg_modes(const SgGroup* __restri
     for (int c = 0; c < NC; ++c) {
       const int comp = (WEDGE && c == NC - 1) ? C_BP : c;
       double* a = acc + ((size_t)comp * nmodes + g.first + j) * 2;
-      atomicAdd(a, (double)sre[j][c] + (double)cre[j][c]);
-      atomicAdd(a + 1, (double)sim[j][c] + (double)cim[j][c]);
+      atomicAdd(a, (double)S[j][c].x + (double)C[j][c].x);
+      atomicAdd(a + 1, (double)S[j][c].y + (double)C[j][c].y);
     }
   }
 }
