@@ -205,8 +205,13 @@ __global__ void __launch_bounds__(SG_THREADS) k_sg_modes(const SgGroup* __restri
   SgGroup g{};
   if (active) g = groups[gi];
   const int mid = g.mz + SG_GROUP / 2;
-  const float fx = g.mx, fy = g.my;
-  // The sums carry (m . r_hat)^n: the mode's 1 / |m|^n is applied in FP64 (k_sg_shells).
+  // The sums carry (m . r_hat)^n: the mode's 1 / |m|^n is applied in FP64 (k_sg_shells).  In
+  // float m is scaled by 2^-sh, |m| <= 2^sh over the group, so that no power leaves the range
+  // of the weights.
+  const int mz_far = max(abs((int)g.mz), abs((int)g.mz + SG_GROUP - 1));
+  const int sh = (33 - __clz(g.mx * g.mx + g.my * g.my + mz_far * mz_far)) / 2;
+  const float unit = __int_as_float((127 - sh) << 23);
+  const float fx = g.mx * unit, fy = g.my * unit;
   // The top hat, which jumps at |mu| = 1/2, takes mu from k_hat's components.
   [[maybe_unused]] float kh[WEDGE ? SG_GROUP : 1][3];
   if constexpr (WEDGE) {
@@ -236,7 +241,7 @@ __global__ void __launch_bounds__(SG_THREADS) k_sg_modes(const SgGroup* __restri
 #pragma unroll 1
     for (int i = 0; i < cnt; i += SG_BLOCK) {
       float2 e[SG_BLOCK];  // s w e^{-i k.x} of the middle mode
-      float d[SG_BLOCK];   // m_x r_hat_x + m_y r_hat_y
+      float d[SG_BLOCK];   // (m_x r_hat_x + m_y r_hat_y) 2^-sh
 #pragma unroll
       for (int b = 0; b < SG_BLOCK; ++b) {
         const SgPoint& q = s_pts[i + b];
@@ -258,7 +263,7 @@ __global__ void __launch_bounds__(SG_THREADS) k_sg_modes(const SgGroup* __restri
           }
           add_comp(S[j][0], C[j][0], t);
           if constexpr (NM > 1) {
-            const float md = fmaf((float)(g.mz + j), q.rh[2], d[b]), md2 = md * md;  // m . r_hat
+            const float md = fmaf((float)(g.mz + j) * unit, q.rh[2], d[b]), md2 = md * md;  // m . r_hat 2^-sh
             float f = md2;
 #pragma unroll
             for (int c = 1; c < NM; ++c) {
@@ -286,8 +291,9 @@ __global__ void __launch_bounds__(SG_THREADS) k_sg_modes(const SgGroup* __restri
     for (int c = 0; c < NC; ++c) {
       const int comp = (WEDGE && c == NC - 1) ? C_BP : c;
       double* a = acc + ((size_t)comp * nmodes + g.first + j) * 2;
-      atomicAdd(a, (double)S[j][c].x + (double)C[j][c].x);
-      atomicAdd(a + 1, (double)S[j][c].y + (double)C[j][c].y);
+      const double back = c < NM ? __longlong_as_double((1023ll + 2 * c * sh) << 52) : 1.0;  // 2^(2 c sh)
+      atomicAdd(a, ((double)S[j][c].x + (double)C[j][c].x) * back);
+      atomicAdd(a + 1, ((double)S[j][c].y + (double)C[j][c].y) * back);
     }
   }
 }
