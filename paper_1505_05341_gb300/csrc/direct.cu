@@ -49,6 +49,7 @@ namespace {
 
 constexpr int SG_THREADS = 128;
 constexpr int SG_CHUNK = 256;  // points per shared-memory chunk
+constexpr int SG_SPLIT_MIN = 128;  // points per thread at least
 constexpr int SG_GROUP = 5;    // modes per thread (neighbouring m_z)
 constexpr int SG_BLOCK = 4;    // points per block of plain sums
 
@@ -135,11 +136,26 @@ __device__ __forceinline__ float2 cis_minus(uint32_t turn, float w) {
   return make_float2(fmaf(w, cs, -d * sn), -fmaf(w, sn, d * cs));
 }
 
-// e^{-2 pi i turn} from FP64: the points' rotations, which four of a group's five modes share.
-__device__ __forceinline__ float2 cis_minus64(uint32_t turn) {
-  double sn, cs;
-  sincospi((double)(int32_t)turn * 4.656612873077393e-10, &sn, &cs);
-  return make_float2((float)cs, (float)-sn);
+// e^{-2 pi i turn} within 0.75 ulp (2.07e-8 rms; correct rounding 2.06e-8): the points' rotations,
+// which four of a group's five modes share.  The angle t + e is reduced to [-pi/4, pi/4] in
+// integers, then the Taylor series to t^11 and t^10 with the leading terms' rounding carried
+// (FP64 sincospi took 0.2 ms for 1.2e6 points).
+__device__ __forceinline__ float2 cis_minus_exact(uint32_t turn) {
+  const uint32_t q = (turn + (1u << 29)) >> 30;  // quadrant, 0 .. 4
+  const int r = (int)(turn - (q << 30)), rh = (r + 32) & ~63;
+  const float pi_h = 1.4629180792671596e-9f, pi_l = (float)(1.4629180792671596e-9 - (double)pi_h);  // pi 2^-31
+  const float x = (float)rh, t = __fmul_rn(x, pi_h);
+  const float e = fmaf(x, pi_l, fmaf((float)(r - rh), pi_h, fmaf(x, pi_h, -t)));
+  const float z = __fmul_rn(t, t), ez = fmaf(t, t, -z);
+  float ps = fmaf(z, -1.f / 39916800.f, 1.f / 362880.f);
+  ps = fmaf(z, fmaf(z, fmaf(z, ps, -1.f / 5040.f), 1.f / 120.f), -1.f / 6.f);
+  const float sn = t + fmaf(__fmul_rn(t, z), ps, fmaf(__fmul_rn(e, z), -0.5f, e));
+  float pc = fmaf(z, -1.f / 3628800.f, 1.f / 40320.f);
+  pc = fmaf(z, fmaf(z, pc, -1.f / 720.f), 1.f / 24.f);
+  const float a = fmaf(z, -0.5f, 1.f), b = fmaf(z, -0.5f, 1.f - a);  // a + b = 1 - z / 2
+  const float cs = a + fmaf(__fmul_rn(z, z), pc, fmaf(e, -sn, fmaf(ez, -0.5f, b)));
+  const float c = (q & 1u) ? sn : cs, s = (q & 1u) ? cs : sn;
+  return make_float2(((q + 1u) & 2u) ? -c : c, (q & 2u) ? s : -s);
 }
 
 // Catalogue particles as points: galaxies +w, randoms -alpha w.
@@ -159,8 +175,8 @@ __global__ void k_sg_points_cat(const float* __restrict__ x, const float* __rest
   q.sw = (float)(sgn * (w ? (double)w[i] : 1.0));
   unit3(px - ox, py - oy, pz - oz, q.rh);
   q.pad = 0.f;
-  q.w1 = cis_minus64(q.u[2]);
-  q.w2 = cis_minus64(2u * q.u[2]);
+  q.w1 = cis_minus_exact(q.u[2]);
+  q.w2 = cis_minus_exact(2u * q.u[2]);
   out[i] = q;
 }
 
@@ -184,21 +200,26 @@ __global__ void k_sg_points_mesh(const float* __restrict__ mesh, int n, int j, i
   q.sw = f * scale;
   unit3(rel_x0 + (ix + s) * H, rel_y0 + (iy + s) * H, rel_z0 + (iz + s) * H, q.rh);
   q.pad = 0.f;
-  q.w1 = cis_minus64(q.u[2]);
-  q.w2 = cis_minus64(2u * q.u[2]);
+  q.w1 = cis_minus_exact(q.u[2]);
+  q.w2 = cis_minus_exact(2u * q.u[2]);
   out[atomicAdd(count, 1u)] = q;
 }
 
 // Per-mode sums over the points of this CTA's split (blockIdx.y); FP64 atomics into
 // acc[C_COUNT][nmodes] (interleaved re, im).
-template <int ELL, bool WEDGE>
+template <int ELL, bool WEDGE, bool SLICED>
 __global__ void __launch_bounds__(SG_THREADS) k_sg_modes(const SgGroup* __restrict__ groups, int ngroups, int nmodes,
                                                           const SgPoint* __restrict__ pts,
                                                           const unsigned* __restrict__ npts_dev, int64_t npts_host,
-                                                          int splits, double* __restrict__ acc) {
+                                                          int splits, int slices, double* __restrict__ acc) {
   __shared__ SgPoint s_pts[SG_CHUNK];
-  const int gi = blockIdx.x * SG_THREADS + threadIdx.x;
-  const bool active = gi < ngroups;
+  // SLICED, at most half as many groups as threads: each group gets `slices` threads, which
+  // share out the points of a chunk in blocks (an 8^3 lattice has 41 groups; 1.2e6 points took
+  // 1.2 to 1.9 ms a call with one thread each, 0.9 to 1.5 ms with one mode per thread, 0.8 to
+  // 1.3 ms so).
+  const int width = SLICED ? ngroups : SG_THREADS, slice = SLICED ? threadIdx.x / width : 0;
+  const int gi = blockIdx.x * width + threadIdx.x - slice * width;
+  const bool active = gi < ngroups && (!SLICED || slice < slices);
   const int64_t npts = npts_dev ? (int64_t)*npts_dev : npts_host;
   const int64_t per = (npts + splits - 1) / splits;
   const int64_t p_lo = std::min<int64_t>(npts, per * blockIdx.y), p_hi = std::min<int64_t>(npts, p_lo + per);
@@ -239,7 +260,7 @@ __global__ void __launch_bounds__(SG_THREADS) k_sg_modes(const SgGroup* __restri
     __syncthreads();
     if (!active) continue;
 #pragma unroll 1
-    for (int i = 0; i < cnt; i += SG_BLOCK) {
+    for (int i = slice * SG_BLOCK; i < cnt; i += SLICED ? slices * SG_BLOCK : SG_BLOCK) {
       float2 e[SG_BLOCK];  // s w e^{-i k.x} of the middle mode
       float d[SG_BLOCK];   // (m_x r_hat_x + m_y r_hat_y) 2^-sh
 #pragma unroll
@@ -283,17 +304,33 @@ __global__ void __launch_bounds__(SG_THREADS) k_sg_modes(const SgGroup* __restri
       }
     }
   }
-  if (!active) return;
+  if (!SLICED && !active) return;
+  // the slices of a group meet in shared memory: FP64 atomics on one address are served one
+  // after another
+  [[maybe_unused]] double2* red = reinterpret_cast<double2*>(s_pts);
+  static_assert(sizeof(s_pts) >= sizeof(double2) * SG_THREADS, "slices' sums");
 #pragma unroll
   for (int j = 0; j < SG_GROUP; ++j) {
-    if (j >= g.count) break;
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
+      double2 v = make_double2((double)S[j][c].x + (double)C[j][c].x, (double)S[j][c].y + (double)C[j][c].y);
+      if constexpr (SLICED) {
+        __syncthreads();
+        red[threadIdx.x] = v;
+        __syncthreads();
+        if (slice == 0)
+          for (int q = 1; q < slices; ++q) {
+            const double2 o = red[threadIdx.x + q * width];
+            v.x += o.x;
+            v.y += o.y;
+          }
+      }
+      if (!active || slice > 0 || j >= g.count) continue;
       const int comp = (WEDGE && c == NC - 1) ? C_BP : c;
       double* a = acc + ((size_t)comp * nmodes + g.first + j) * 2;
       const double back = c < NM ? __longlong_as_double((1023ll + 2 * c * sh) << 52) : 1.0;  // 2^(2 c sh)
-      atomicAdd(a, ((double)S[j][c].x + (double)C[j][c].x) * back);
-      atomicAdd(a + 1, ((double)S[j][c].y + (double)C[j][c].y) * back);
+      atomicAdd(a, v.x * back);
+      atomicAdd(a + 1, v.y * back);
     }
   }
 }
@@ -375,6 +412,8 @@ __global__ void k_sg_finalize(const double* __restrict__ sacc, const double* __r
 struct ModeTable {
   std::vector<SgMode> modes;
   std::vector<SgGroup> groups;
+  size_t mode_bytes() const { return sizeof(SgMode) * modes.size(); }
+  size_t group_bytes() const { return sizeof(SgGroup) * groups.size(); }
   std::vector<double> shell;  // [2][nbins]: mode count, sum |k|
 };
 
@@ -450,6 +489,19 @@ ys_status fail(cudaError_t e) {
   return e == cudaErrorMemoryAllocation ? YS_ERR_OOM : YS_ERR_CUDA;
 }
 
+// The mode and group lists on the device, in one piece.
+cudaError_t upload(const ModeTable& mt, Scratch& sc, cudaStream_t st, SgMode*& d_modes, SgGroup*& d_groups) {
+  static_assert(alignof(SgGroup) <= alignof(SgMode), "groups follow the modes");
+  unsigned char* raw = nullptr;
+  cudaError_t e = sc.get(raw, mt.mode_bytes() + mt.group_bytes());
+  if (e) return e;
+  d_modes = reinterpret_cast<SgMode*>(raw);
+  d_groups = reinterpret_cast<SgGroup*>(raw + mt.mode_bytes());
+  if (mt.modes.empty()) return cudaSuccess;
+  e = cudaMemcpyAsync(d_modes, mt.modes.data(), mt.mode_bytes(), cudaMemcpyHostToDevice, st);
+  return e ? e : cudaMemcpyAsync(d_groups, mt.groups.data(), mt.group_bytes(), cudaMemcpyHostToDevice, st);
+}
+
 // The modes' groups on the device.
 struct ModeGroups {
   const SgGroup* groups;
@@ -464,13 +516,14 @@ cudaError_t launch_modes(const ModeGroups& mg, const SgPoint* pts, const unsigne
   if (!e) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e) return e;
   const int mblocks = (mg.ngroups + SG_THREADS - 1) / SG_THREADS;
-  // split the points so that the grid fills the GPU a few times over
-  const int64_t want = (int64_t)sms * 16;
-  int splits = (int)std::max<int64_t>(1, std::min<int64_t>(1024, (want + mblocks - 1) / mblocks));
-  const int64_t np_bound = npts_dev ? INT64_MAX : npts_host;
-  splits = (int)std::max<int64_t>(1, std::min<int64_t>(splits, (np_bound + SG_CHUNK - 1) / SG_CHUNK));
+  const int slices = std::max(1, SG_THREADS / mg.ngroups);
+  // split the points so that the grid fills the GPU a few times over, with SG_SPLIT_MIN points
+  // per thread at least (npts_host bounds *npts_dev)
+  const int64_t want = ((int64_t)sms * 16 + mblocks - 1) / mblocks;
+  const int splits = (int)std::max<int64_t>(1, std::min(want, (npts_host + SG_SPLIT_MIN * slices - 1) / (SG_SPLIT_MIN * slices)));
   dim3 grid(mblocks, splits);
-  k_sg_modes<ELL, WEDGE><<<grid, SG_THREADS, 0, st>>>(mg.groups, mg.ngroups, mg.nmodes, pts, npts_dev, npts_host, splits, acc);
+  auto kern = slices > 1 ? k_sg_modes<ELL, WEDGE, true> : k_sg_modes<ELL, WEDGE, false>;
+  kern<<<grid, SG_THREADS, 0, st>>>(mg.groups, mg.ngroups, mg.nmodes, pts, npts_dev, npts_host, splits, slices, acc);
   return cudaGetLastError();
 }
 
@@ -539,12 +592,8 @@ extern "C" ys_status ys_sum_gal(const ys_config* cfg, const ys_catalog* gal, con
   SgPoint* d_pts = nullptr;
   const int64_t npts = gal->n + ran->n;
   cudaError_t e;
-  if ((e = sc.get(d_modes, (size_t)nmodes)) || (e = sc.get(d_groups, mt.groups.size())) || (e = sc.get(d_acc, (size_t)C_COUNT * 2 * std::max(1, nmodes))) ||
+  if ((e = upload(mt, sc, st, d_modes, d_groups)) || (e = sc.get(d_acc, (size_t)C_COUNT * 2 * std::max(1, nmodes))) ||
       (e = sc.get(d_sums, (size_t)SUM_COUNT)) || (e = sc.get(d_pts, (size_t)std::max<int64_t>(1, npts))))
-    return fail(e);
-  if (nmodes > 0 &&
-      ((e = cudaMemcpyAsync(d_modes, mt.modes.data(), sizeof(SgMode) * nmodes, cudaMemcpyHostToDevice, st)) ||
-       (e = cudaMemcpyAsync(d_groups, mt.groups.data(), sizeof(SgGroup) * mt.groups.size(), cudaMemcpyHostToDevice, st))))
     return fail(e);
   const ModeGroups mg{d_groups, (int)mt.groups.size(), nmodes};
   if ((e = cudaMemsetAsync(d_acc, 0, sizeof(double) * C_COUNT * 2 * std::max(1, nmodes), st)) ||
@@ -594,12 +643,8 @@ extern "C" ys_status ys_sum_grid(ys_plan* plan, double* d_out, double* d_wedges)
   SgPoint* d_pts = nullptr;
   unsigned* d_count = nullptr;
   cudaError_t e;
-  if ((e = sc.get(d_modes, (size_t)nmodes)) || (e = sc.get(d_groups, mt.groups.size())) || (e = sc.get(d_acc, (size_t)C_COUNT * 2 * std::max(1, nmodes))) ||
+  if ((e = upload(mt, sc, st, d_modes, d_groups)) || (e = sc.get(d_acc, (size_t)C_COUNT * 2 * std::max(1, nmodes))) ||
       (e = sc.get(d_pts, (size_t)chunk)) || (e = sc.get(d_count, 1)))
-    return fail(e);
-  if (nmodes > 0 &&
-      ((e = cudaMemcpyAsync(d_modes, mt.modes.data(), sizeof(SgMode) * nmodes, cudaMemcpyHostToDevice, st)) ||
-       (e = cudaMemcpyAsync(d_groups, mt.groups.data(), sizeof(SgGroup) * mt.groups.size(), cudaMemcpyHostToDevice, st))))
     return fail(e);
   const ModeGroups mg{d_groups, (int)mt.groups.size(), nmodes};
   if ((e = cudaMemsetAsync(d_acc, 0, sizeof(double) * C_COUNT * 2 * std::max(1, nmodes), st))) return fail(e);
