@@ -633,9 +633,9 @@ extern "C" ys_status ys_sum_grid(ys_plan* plan, double* d_out, double* d_wedges)
   const int nmodes = (int)mt.modes.size();
   const bool wedge = d_wedges != nullptr;
   const int64_t n3 = (int64_t)p.n * p.n * p.n;
-  // the nodes go through in chunks of at most 2^26 (2 GB of points), each added into
-  // the FP64 per-mode sums
-  const int64_t chunk = std::min<int64_t>(n3, (int64_t)1 << 26);
+  // the nodes go through in chunks of at most 2 GB of points, each added into the FP64
+  // per-mode sums
+  const int64_t chunk = std::min<int64_t>(n3, ((int64_t)2 << 30) / (int64_t)sizeof(SgPoint));
   Scratch sc;
   SgMode* d_modes = nullptr;
   SgGroup* d_groups = nullptr;
