@@ -233,13 +233,23 @@ struct LineFft {
 // Line handled by thread group g.  Where several groups share a half-warp, their lines
 // are TPL apart, so that the groups' elements fall on different banks (LINE is odd).
 template <int TPL>
-__device__ __forceinline__ int line_of_group(int g) {
+__host__ __device__ constexpr int line_of_group(int g) {
   if constexpr (TPL >= 16) {
     return g;
   } else {
     constexpr int G = 16 / TPL;
     return (g % G) * TPL + (g / G) % TPL + (g / 16) * 16;
   }
+}
+
+// Whether in each warp of `groups` thread groups all lines lie below r, or all from r on: a
+// branch on the line is then uniform over every barrier of line_group_sync.
+template <int TPL>
+__host__ __device__ constexpr bool warps_on_one_side(int groups, int r) {
+  constexpr int PER = TPL >= 32 ? 1 : 32 / TPL;  // groups per warp
+  for (int g = 0; g < groups; ++g)
+    if ((line_of_group<TPL>(g) >= r) != (line_of_group<TPL>(g / PER * PER) >= r)) return false;
+  return true;
 }
 
 // The twiddles of thread t of a line, from the table.

@@ -176,7 +176,8 @@ struct YZ {
   static constexpr int R0 = ELL == 0 ? 2 * GROUPS : (N <= 256 ? (ELL == 6 ? GROUPS / 2 : GROUPS) : 8);
   static constexpr int R = R0 > N ? N : (N % R0 ? 8 : R0);
   // With twice as many groups as rows, half of the groups take the upper degrees and F.
-  static constexpr bool SPLIT = ND > 1 && GROUPS >= 2 * R && (TPL >= 32 || R % (32 / TPL) == 0);
+  // (The half of a group is decided by its line, and the halves skip each other's transforms.)
+  static constexpr bool SPLIT = ND > 1 && GROUPS >= 2 * R && warps_on_one_side<TPL>(GROUPS, R);
   static constexpr int DSPLIT = SPLIT ? (ND + 1) / 2 : ND;  // degrees of the first half
   static constexpr int RLINES = R * ND + R / 2;  // the F lines hold two rows each
   // Columns per column item: as many as the thread groups transform at once.
