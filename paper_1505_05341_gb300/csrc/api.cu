@@ -418,8 +418,11 @@ void set_yz_grid(Plan& p, int grid, int lead_pct) {
   const int per_plane = p.n / p.yz_rows + std::max(1, (p.nzc + p.yz_cols - 1) / p.yz_cols);
   const int gap = 2 + (p.yz_grid + per_plane - 1) / per_plane;
   const int slots_max = p.ring_slots_cap > 0 ? p.ring_slots_cap : p.m * p.n;
-  p.ring_lead = std::min(ring_lead_for(p, p.yz_grid, p.ring_lead_pct), std::max(1, slots_max - gap));
-  p.ring_slots = std::min(p.m * p.n, p.ring_lead + gap);
+  const int planes = p.m * p.n, lead = ring_lead_for(p, p.yz_grid, p.ring_lead_pct);
+  // with a slot for every plane none is reused, and the lead need not leave a gap
+  const bool all = slots_max >= planes && lead + gap >= planes;
+  p.ring_lead = std::min(lead, all ? planes - 1 : std::max(1, slots_max - gap));
+  p.ring_slots = all ? planes : std::min(planes, p.ring_lead + gap);
 }
 
 LaunchScope::LaunchScope(Plan& plan, int c) : p(plan), cls(c) {
