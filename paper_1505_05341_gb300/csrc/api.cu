@@ -580,7 +580,6 @@ ys_status ys_plan_create(const ys_config* cfg, ys_plan** out) {
   ys::Geom& g = p.geom;
   g.n = n;
   g.inv_h = (float)(n / c.box_len);
-  g.inv_h_lo = (float)(n / c.box_len - (double)g.inv_h);
   for (int a = 0; a < 3; ++a) g.bmin[a] = (float)c.box_min[a];
   // tile counters sized for every scatter-tile candidate the tuner may pick
   p.ntiles_max = 0;

@@ -151,24 +151,18 @@ __device__ __forceinline__ bool locate(float x, int axis, const Geom& g, const f
   int i = max(-1, min(n, __float2int_rd(u0)));  // (the conversion saturates; NaN gives 0)
   const float2* nd = nodes + axis * (n + 3) + 1;  // nd[i] for i in [-1, n + 1]
   float2 nv = nd[i];
-  // 1 / H in two floats: its rounding alone (5e-8 for H = 500 / 32) stretches every offset of
-  // the mesh alike, which moved P_0 of the 500 Mpc/h cube with CIC by 6e-8
-  auto offset = [&]() {
-    const float t = (x - nv.x) - nv.y;
-    return fmaf(t, g.inv_h, t * g.inv_h_lo);
-  };
-  float d = offset();
+  float d = ((x - nv.x) - nv.y) * g.inv_h;
   // One-cell correction of the float guess (rarely needed); a particle within rounding
   // of a node can land on d = 1.0f (or a hair below 0) after it, so d is clamped into
   // [0, 1): the stencils are continuous across the node, so either side gives the same mesh.
   if (d < 0.f) {
     i = max(i - 1, -1);
     nv = nd[i];
-    d = fminf(offset(), 0.99999994f);
+    d = fminf(((x - nv.x) - nv.y) * g.inv_h, 0.99999994f);
   } else if (d >= 1.f) {
     i = min(i + 1, n);
     nv = nd[i];
-    d = fmaxf(offset(), 0.f);
+    d = fmaxf(((x - nv.x) - nv.y) * g.inv_h, 0.f);
   }
   d = fminf(fmaxf(d, 0.f), 0.99999994f);
   const bool ok = (unsigned)i < (unsigned)n && u0 == u0;

@@ -43,8 +43,7 @@ constexpr int kTileCandidates[5][3] = {{16, 16, 32}, {8, 16, 32}, {16, 16, 16}, 
 
 struct Geom {
   int n;            // mesh side N
-  float inv_h;      // 1 / H, and what its rounding leaves
-  float inv_h_lo;
+  float inv_h;      // 1 / H
   float bmin[3];    // box_min (float) for the first guess of the cell index
   int tiles[3];     // tiles per axis
   int tdim[3];      // tile extent per axis, a power of two
