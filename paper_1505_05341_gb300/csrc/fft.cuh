@@ -12,6 +12,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 namespace ys {
 
 __host__ __device__ constexpr bool is_pow2(int n) { return n > 0 && (n & (n - 1)) == 0; }
@@ -132,14 +134,19 @@ template <> struct Dft<8> {
 };
 
 // 16 = 4 x 4: DFT-4 over the inputs 4 a + b for each b, twiddles w16^(b k1), DFT-4 over b.
-template <> struct Dft<16> {
+//
+// LONG, for lines whose second radix is 16 too: cos(pi / 8) rounded up.  The nearest float makes
+// |c1 - i s1| 2.9e-8 short, which with h (1.7e-8 short) biases every mode the same way: over a
+// line of 256 (512) the mean gain was 2.7e-8 (3.4e-8) short, 2.1e-8 (2.4e-8) with radix-8 stages,
+// and P_0 1.4e-7 (1.6e-7) low.  One float up it is 2.7e-8 long and cancels h: mean gains 1e-9 and
+// 6e-9 short, P_0 4e-8 and 5e-8 low.  Lines with one radix-16 stage gain nothing (their gain is
+// that of radix 8) and would take the larger phase error, 1.8e-8 instead of 0.5e-8: P_2 of a
+// 32^3 mesh was off by 1.1 times as much.
+template <bool LONG>
+struct Dft16 {
   __device__ static __forceinline__ void run(float2* v) {
     const float h = 0.707106781186547524f, s1 = 0.382683432365089772f;
-    // cos(pi / 8) rounded up.  The nearest float makes |c1 - i s1| 2.9e-8 short, which with h
-    // (1.7e-8 short) biases every mode the same way: over a line of 512 the mean gain was 3.4e-8
-    // short (2.4e-8 with radix-8 stages), P_0 1.6e-7 low at 512^3.  One float up it is 2.7e-8
-    // long and cancels h: mean gain 6e-9 short, P_0 7e-8 low.
-    const float c1 = 0.92387956380844116f;
+    const float c1 = LONG ? 0.92387956380844116f : 0.923879532511286756f;
     float2 t[4][4];  // [k1][b]
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
@@ -267,8 +274,10 @@ __device__ __forceinline__ void line_fft(float2 (&v)[LineFft<N>::R1], float2* li
                                          const float2 (&tw)[LineFft<N>::R1 - 1], const float2* wE, bool ok) {
   using L = LineFft<N>;
   constexpr int R1 = L::R1, R2 = L::R2, E2 = L::E2, P = L::P, TPL = L::TPL;
+  using First = std::conditional_t<R1 == 16, Dft16<R2 == 16>, Dft<R1>>;
+  using Second = std::conditional_t<R2 == 16, Dft16<true>, Dft<R2>>;
   if (ok) {
-    Dft<R1>::run(v);
+    First::run(v);
     line[t] = v[0];
 #pragma unroll
     for (int k = 1; k < R1; ++k) line[k * P + t] = cmul(v[k], tw[k - 1]);
@@ -284,7 +293,7 @@ __device__ __forceinline__ void line_fft(float2 (&v)[LineFft<N>::R1], float2* li
         float2 b[R2];
 #pragma unroll
         for (int s = 0; s < R2; ++s) b[s] = q[E2 * s];
-        Dft<R2>::run(b);
+        Second::run(b);
         if constexpr (E2 == 4) {
 #pragma unroll
           for (int s = 1; s < R2; ++s) b[s] = cmul(b[s], wE[17 * e + s]);
