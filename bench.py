@@ -196,7 +196,7 @@ YZ_LINES = {"pairs": 2.5, "fields": 15}
 # each kernel on the 512^3 survey workload in its tuned launch configuration (one-pass
 # dram__bytes_{read,write}.sum capture; profiles/dram_traffic_shell512_tsc_il.md).
 # Remove an entry when its kernel changes.
-TRAFFIC = {"yz_stage": 7.18e9, "x_combine": 5.81e9, "tile_deposit": 2.50e9, "particle_bin": 2.52e9,
+TRAFFIC = {"yz_stage": 7.17e9, "x_combine": 5.81e9, "tile_deposit": 2.50e9, "particle_bin": 2.52e9,
            "particle_count": 1.16e9}
 
 

@@ -466,7 +466,7 @@ k_bin(const __grid_constant__ Cats cats, Geom g, const float2* __restrict__ node
 
 // Exclusive scan of the tile counts into off and the front cursors cur, one CTA per 1024
 // tiles.  Each CTA sums all counts before its own (at most 1 MB, from L2) instead of
-// waiting for the CTAs before it: 32768 tiles 102 -> 6 us, 262144 tiles 785 -> 16 us
+// waiting for the CTAs before it: 32768 tiles 102 -> 8 us, 262144 tiles 785 -> 16 us
 // against one CTA for all.
 __global__ void __launch_bounds__(1024)
 k_scan(const unsigned* __restrict__ count, int ntiles, unsigned* __restrict__ off, unsigned* __restrict__ cur) {
@@ -994,9 +994,11 @@ cudaError_t run_count(Plan& p, const ys_catalog& gal, const ys_catalog& ran, int
 }
 
 // CTAs per tile of the deposit: doubled (up to 8) while there are fewer than five per SM
-// and a CTA would still get 256 records.  6.6e6 particles, CIC: 512 tiles (128^3) 198 us
-// with one CTA each (1.1 waves of three per SM) and 157 us with four; 1728 tiles (192^3)
-// 142 us with one and 182 us with two, so the line lies between.
+// and a CTA would still get 256 records.  Times in us with 1, 2, 4 and 8 CTAs per tile, on
+// 152 SMs, CIC, 6.6e6 particles: 64 tiles 491, 368, 204, 189 (8 taken); 216 tiles 175, 140, 130,
+// 168 (4); 512 tiles 142, 153, 153, 210 (2; TSC interlaced 532, 481, 491, 577); 1728 tiles 104,
+// 176, 234, 416 (1).  6e5 particles: 64 tiles 40, 35, 25, 34; 216 tiles 21, 23, 31, 58; 512
+// tiles 23, 38, 52, 108: so few records would want half of what the rule takes.
 int deposit_cluster(int ntiles, int64_t particles, int sms) {
   int cl = 1;
   while (cl < 8 && (int64_t)ntiles * cl < 5 * sms && particles / ((int64_t)ntiles * 2 * cl) >= 256) cl *= 2;

@@ -93,7 +93,7 @@ template <int ELL> __constant__ constexpr YLines<ELL> kYLines{};
 // 12.1 ms when every basis field was transformed along z (16 real lines per row instead of
 // 5) with radix-8 stages, 6.5 ms with source fields and line transforms, 5.7 ms with two
 // barriers per item and the radix-2 twiddles left to the readers; l_max = 6 30.8, 13.9,
-// 11.6 ms; 1024^3 87, 40, 35 ms; 256^3 interlaced 1.76, 1.19, 0.97 ms.
+// 11.8 ms; 1024^3 87, 40, 35 ms; 256^3 interlaced 1.76, 1.19, 0.97 ms.
 // ---------------------------------------------------------------------------
 
 struct YZParams {
@@ -660,7 +660,8 @@ __host__ __device__ constexpr int tile_group(int q) {
 // (see k_x_combine): always for l_max = 6, and for l_max = 2, 4 except at 256^3 and
 // 512^3, where the x stage is held to 80 registers for three CTAs per SM and the extra
 // error terms would spill (shells there hold many modes, and the plain sums meet the
-// parity bar with a wide margin).
+// parity bar with a wide margin).  The rule goes by the mesh size alone, so that a plan's
+// accuracy does not depend on the tile size the autotuner picks.
 template <int N, int ELL>
 __host__ __device__ constexpr bool x_horner() { return ELL == 6 || (ELL >= 2 && N != 256 && N != 512); }
 
